@@ -89,3 +89,29 @@ def test_stage3_closed_forms(nla):
     e = np.array([1.0, 2.0, 0.5, 1.5, 0.25])
     S, _ = nla.bdsvd_vals(torch.from_numpy(d).cuda(), torch.from_numpy(e).cuda())
     assert err_rel(S.cpu().numpy(), oracle.bdsvd(d, e)) <= 1e-13
+
+
+@pytest.mark.parametrize("dt", [0, 1])
+@pytest.mark.parametrize("n", [8, 9, 17, 40, 609, 1217])
+@pytest.mark.parametrize("kind", ["graded", "decoupled", "identity", "no_diagonal"])
+def test_stage3_minors_keep_their_signs(nla, dt, n, kind):
+    # graded and decoupled bidiagonals make the minors of a Sturm count shrink or vanish; the sizes
+    # straddle its blocks of 16 terms and the lanes-per-value limits.  Bound: the search stops at
+    # 2^-51 (FP64) / 2^-23 (FP32) of the Gershgorin bound <= 2 sigma_1, plus a few roundings.
+    d, e = np.ones(n), np.zeros(n - 1)
+    if kind == "graded":
+        d = 10.0 ** -np.linspace(0, 16, n)
+        e = 0.5 * d[:-1]
+    elif kind == "decoupled":
+        g = np.random.default_rng(40 + n)
+        d, e = g.standard_normal(n), g.standard_normal(n - 1)
+        e[::3] = 0.0
+        d[::5] = 0.0
+    elif kind == "no_diagonal":
+        d, e = np.zeros(n), np.ones(n - 1)
+    tdt = torch.float64 if dt == 0 else torch.float32
+    S, info = nla.bdsvd_vals(torch.from_numpy(d).cuda(), torch.from_numpy(e).cuda(), dtype=tdt)
+    torch.cuda.synchronize()
+    assert int(info.item()) == 0
+    B = np.diag(d) + np.diag(e, 1)
+    assert err_rel(S.double().cpu().numpy(), np.linalg.svd(B, compute_uv=False)) <= (n * 2.0 ** -51 if dt == 0 else 2.0 ** -20)
