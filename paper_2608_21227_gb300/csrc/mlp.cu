@@ -30,74 +30,276 @@ size_t w_off(int l) {  // offset of W_l (0-based layer) in the packed parameter 
     for (int i = 0; i < l; ++i) o += (size_t)kDims[i + 1] * kDims[i] + kDims[i + 1];
     return o;
 }
-size_t b_off(int l) { return w_off(l) + (size_t)kDims[l + 1] * kDims[l]; }
 constexpr size_t kParams = (size_t)kH * kIn + kH + 2 * ((size_t)kH * kH + kH) + kH + 1;
 
-// C(i, j) = sum_k A(i, k) B(k, j) over generic strides; epilogue:
-//   mode 0: C = acc                      mode 1: C = acc + bias[j]
-//   mode 2: Z = acc + bias[j], H = relu(Z) (C = Z, C2 = H)
-//   mode 3: C = acc * [Zmask(i, j) > 0]  (backward through ReLU)
-constexpr int kTile = 32;
-__global__ void gemm_kernel(int M, int N, int K, const float *__restrict__ A, long sa0, long sa1,
-                            const float *__restrict__ B, long sb0, long sb1, float *C, long sc0, long sc1,
-                            const float *__restrict__ bias, float *C2, const float *__restrict__ Zmask, int mode) {
-    __shared__ float As[kTile][kTile + 1];
-    __shared__ float Bs[kTile][kTile + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
-    const int i0 = blockIdx.y * kTile, j0 = blockIdx.x * kTile;
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int k0 = 0; k0 < K; k0 += kTile) {
-        for (int r = ty; r < kTile; r += 8) {
-            int i = i0 + r, k = k0 + tx;
-            As[r][tx] = (i < M && k < K) ? A[i * sa0 + k * sa1] : 0.f;
-            int kk = k0 + r, j = j0 + tx;
-            Bs[r][tx] = (kk < K && j < N) ? B[kk * sb0 + j * sb1] : 0.f;
+// One block takes tiles of R rows through the whole network: forward, loss gradient and
+// backward, with every activation in shared memory and one layer's weights staged at a time.
+// The weights' gradients of a block's rows are 35,201 partial sums; each block writes its own
+// (grad_sum_kernel adds them in block order, so results do not depend on timing).
+//
+// Why fused: as separate matrix products the step was 17 launches whose weight gradients had
+// K = rows on 16 blocks (4096 rows: 101 us per product, 90 us per bias sum).  What bounds it
+// now is shared-memory reads (a thread's 4 x 4 outputs read 8 values per 16 FMAs).
+// One training step of 4096 rows: 1501 -> 59 us.
+//
+// Shared memory (floats): Ws kH x kLd (one layer's weights, transposed for the forward pass),
+// X R x 16, H1..H3 and two gradient buffers R x kLd.
+constexpr int kLd = kH + 4;  // rows stay 16-byte aligned, neighbouring rows shift by four banks
+constexpr int kMlpThreads = 256;
+
+constexpr size_t mlp_smem_floats(int R) { return (size_t)kH * kLd + (size_t)R * 16 + (size_t)5 * R * kLd + R + 8; }
+
+// Rows per tile: small batches are spread over more blocks (8 rows: two blocks per SM fit).
+int mlp_tile(int rows) { return rows <= 8 * 304 ? 8 : 32; }
+int mlp_blocks(int rows) {
+    const int tiles = (rows + mlp_tile(rows) - 1) / mlp_tile(rows);
+    return std::min(tiles, mlp_tile(rows) == 8 ? 304 : 152);
+}
+
+// Ws(k, o) = W[o * K + k] (TRANS) or Ws(o, k) = W[o * K + k], K = kH.
+template <bool TRANS>
+__device__ void stage_weights(float *Ws, const float *__restrict__ W, int tid, bool vec) {
+    if (vec) {
+        for (int i = tid; i < kH * kH / 4; i += kMlpThreads) {
+            if (TRANS) {
+                const int o = i % kH, k = i / kH * 4;  // lanes along o: conflict-free stores
+                const float4 w = *reinterpret_cast<const float4 *>(W + o * kH + k);
+                Ws[k * kLd + o] = w.x, Ws[(k + 1) * kLd + o] = w.y;
+                Ws[(k + 2) * kLd + o] = w.z, Ws[(k + 3) * kLd + o] = w.w;
+            } else {
+                const int k = i % (kH / 4) * 4, o = i / (kH / 4);
+                *reinterpret_cast<float4 *>(Ws + o * kLd + k) = *reinterpret_cast<const float4 *>(W + o * kH + k);
+            }
         }
-        __syncthreads();
-#pragma unroll 8
-        for (int k = 0; k < kTile; ++k) {
-            float bv = Bs[k][tx];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[q] += As[ty + 8 * q][k] * bv;
+    } else {
+        for (int i = tid; i < kH * kH; i += kMlpThreads) {
+            const int o = i / kH, k = i % kH;
+            Ws[TRANS ? k * kLd + o : o * kLd + k] = W[i];
         }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        int i = i0 + ty + 8 * q, j = j0 + tx;
-        if (i >= M || j >= N) continue;
-        float v = acc[q];
-        if (mode == 1 || mode == 2) v += bias[j];
-        if (mode == 3) v = Zmask[i * sc0 + j * sc1] > 0.f ? v : 0.f;
-        C[i * sc0 + j * sc1] = v;
-        if (mode == 2) C2[i * sc0 + j * sc1] = fmaxf(v, 0.f);
     }
 }
 
-void gemm(cudaStream_t st, int M, int N, int K, const float *A, long sa0, long sa1, const float *B, long sb0, long sb1,
-          float *C, long sc0, long sc1, const float *bias, float *C2, const float *Zmask, int mode) {
-    dim3 grid((N + kTile - 1) / kTile, (M + kTile - 1) / kTile), block(32, 8);
-    gemm_kernel<<<grid, block, 0, st>>>(M, N, K, A, sa0, sa1, B, sb0, sb1, C, sc0, sc1, bias, C2, Zmask, mode);
+// acc(r, q) += sum_k In(r0 + r, k) Ws(k, 4 c + q) over the first K columns of In (leading dimension ld).
+template <int RT>
+__device__ void tile_product(float (&acc)[RT][4], const float *In, int ld, const float *Ws, int K, int r0, int c) {
+#pragma unroll 2
+    for (int k = 0; k < K; k += 4) {
+        float4 h[RT], w[4];
+#pragma unroll
+        for (int r = 0; r < RT; ++r) h[r] = *reinterpret_cast<const float4 *>(In + (r0 + r) * ld + k);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) w[u] = *reinterpret_cast<const float4 *>(Ws + (k + u) * kLd + 4 * c);
+#pragma unroll
+        for (int r = 0; r < RT; ++r) {
+            const float hv[4] = {h[r].x, h[r].y, h[r].z, h[r].w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                acc[r][0] += hv[u] * w[u].x, acc[r][1] += hv[u] * w[u].y;
+                acc[r][2] += hv[u] * w[u].z, acc[r][3] += hv[u] * w[u].w;
+            }
+        }
+    }
 }
 
-// column sums: out[j] = sum_i G[i*ld + j]
-__global__ void colsum_kernel(const float *G, int rows, int cols, long ld, float *out) {
-    int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= cols) return;
+// dW(o, k) (+)= sum_r G(r, o) H(r, k): thread t owns outputs o = 8 (t / 16) .., k = 4 (t % 16) .. and
+// 64 + 4 (t % 16) ..; db(o) likewise.
+template <int R>
+__device__ void weight_grads(const float *G, const float *H, float *dW, float *db, bool first, int tid) {
+    const int o0 = 8 * (tid / 16), k0 = 4 * (tid % 16);
+    float acc[8][8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+#pragma unroll 2
+    for (int r = 0; r < R; ++r) {
+        float g[8], h[8];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const float4 gv = *reinterpret_cast<const float4 *>(G + r * kLd + o0 + 4 * u);
+            const float4 hv = *reinterpret_cast<const float4 *>(H + r * kLd + k0 + 64 * u);
+            g[4 * u] = gv.x, g[4 * u + 1] = gv.y, g[4 * u + 2] = gv.z, g[4 * u + 3] = gv.w;
+            h[4 * u] = hv.x, h[4 * u + 1] = hv.y, h[4 * u + 2] = hv.z, h[4 * u + 3] = hv.w;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[i][j] += g[i] * h[j];
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            float *d = dW + (o0 + i) * kH + k0 + (j & 3) + 64 * (j >> 2);
+            *d = first ? acc[i][j] : *d + acc[i][j];
+        }
+    if (tid < kH) {
+        float s = 0.f;
+        for (int r = 0; r < R; ++r) s += G[r * kLd + tid];
+        db[tid] = first ? s : db[tid] + s;
+    }
+}
+
+template <int R>
+__global__ void __launch_bounds__(kMlpThreads)
+mlp_kernel(const float *__restrict__ P, const float *__restrict__ X, const float *__restrict__ y, int rows,
+           float *pred, float *part, float *loss_acc, int train) {
+    extern __shared__ __align__(16) float smem[];
+    constexpr int RT = R / 8;  // rows per thread: 8 row groups x 32 output groups
+    float *Ws = smem, *Xs = Ws + kH * kLd, *H[3], *Ga, *Gb, *gout;
+    H[0] = Xs + R * 16;
+    H[1] = H[0] + R * kLd, H[2] = H[1] + R * kLd;
+    Ga = H[2] + R * kLd, Gb = Ga + R * kLd, gout = Gb + R * kLd;
+    const int tid = threadIdx.x, c = tid % 32, r0 = tid / 32 * RT;
+    const bool vec = (reinterpret_cast<uintptr_t>(P) & 15) == 0;  // (every layer starts on a multiple of four)
+    constexpr size_t oW[kLayers] = {0, (size_t)kH * kIn + kH, (size_t)kH * kIn + kH + kH * kH + kH,
+                                    (size_t)kH * kIn + kH + 2 * (kH * kH + kH)};
+    constexpr size_t oB[kLayers] = {(size_t)kH * kIn, oW[1] + kH * kH, oW[2] + kH * kH, oW[3] + kH};
+    float *dP = part + (size_t)blockIdx.x * kParams;
+    bool first = true;
+    for (int row0 = blockIdx.x * R; row0 < rows; row0 += gridDim.x * R, first = false) {
+        __syncthreads();
+        for (int i = tid; i < R * 16; i += kMlpThreads) {
+            const int r = i / 16, k = i % 16;
+            Xs[i] = (row0 + r < rows && k < kIn) ? X[(size_t)(row0 + r) * kIn + k] : 0.f;
+        }
+        // ---- forward
+        for (int l = 0; l < 3; ++l) {
+            if (l == 0) {
+                for (int i = tid; i < kH * 16; i += kMlpThreads) {
+                    const int o = i % kH, k = i / kH;
+                    Ws[k * kLd + o] = k < kIn ? P[o * kIn + k] : 0.f;
+                }
+            } else {
+                stage_weights<true>(Ws, P + oW[l], tid, vec);
+            }
+            __syncthreads();
+            float acc[RT][4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float bq = P[oB[l] + 4 * c + q];
+#pragma unroll
+                for (int r = 0; r < RT; ++r) acc[r][q] = bq;
+            }
+            if (l == 0)
+                tile_product<RT>(acc, Xs, 16, Ws, 16, r0, c);
+            else
+                tile_product<RT>(acc, H[l - 1], kLd, Ws, kH, r0, c);
+#pragma unroll
+            for (int r = 0; r < RT; ++r)
+                *reinterpret_cast<float4 *>(H[l] + (r0 + r) * kLd + 4 * c) =
+                    make_float4(fmaxf(acc[r][0], 0.f), fmaxf(acc[r][1], 0.f), fmaxf(acc[r][2], 0.f), fmaxf(acc[r][3], 0.f));
+            __syncthreads();
+        }
+        // ---- output layer: a warp per row (R / 8 rows each)
+#pragma unroll
+        for (int r = 0; r < RT; ++r) {
+            float s = 0.f;
+#pragma unroll
+            for (int k = 0; k < kH; k += 32) s += H[2][(r0 + r) * kLd + k + c] * P[oW[3] + k + c];
+            s = nla::warp_sum(s) + P[oB[3]];
+            const int row = row0 + r0 + r;
+            float d = 0.f;
+            if (row < rows) {
+                if (c == 0) pred[row] = s;
+                if (train) d = s - y[row];
+            }
+            if (c == 0) {
+                gout[r0 + r] = 2.f * d / (float)rows;
+                if (train && loss_acc && row < rows) atomicAdd(loss_acc, d * d / (float)rows);
+            }
+        }
+        if (!train) continue;
+        __syncthreads();
+        // ---- backward: output layer
+        if (tid < kH) {
+            float s = 0.f;
+            const float w4 = P[oW[3] + tid];
+            for (int r = 0; r < R; ++r) {
+                const float h = H[2][r * kLd + tid], g = gout[r];
+                s += g * h;
+                Ga[r * kLd + tid] = h > 0.f ? g * w4 : 0.f;
+            }
+            dP[oW[3] + tid] = first ? s : dP[oW[3] + tid] + s;
+        } else if (tid == kH) {
+            float s = 0.f;
+            for (int r = 0; r < R; ++r) s += gout[r];
+            dP[oB[3]] = first ? s : dP[oB[3]] + s;
+        }
+        // ---- hidden layers 3 and 2: dW = G^T H, G' = (G W) .* [H > 0]
+        float *G = Ga, *Gn = Gb;
+        for (int l = 2; l >= 1; --l) {
+            stage_weights<false>(Ws, P + oW[l], tid, vec);
+            __syncthreads();
+            weight_grads<R>(G, H[l - 1], dP + oW[l], dP + oB[l], first, tid);
+            float acc[RT][4];
+#pragma unroll
+            for (int r = 0; r < RT; ++r)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[r][q] = 0.f;
+            tile_product<RT>(acc, G, kLd, Ws, kH, r0, c);
+#pragma unroll
+            for (int r = 0; r < RT; ++r) {
+                const float4 h = *reinterpret_cast<const float4 *>(H[l - 1] + (r0 + r) * kLd + 4 * c);
+                *reinterpret_cast<float4 *>(Gn + (r0 + r) * kLd + 4 * c) =
+                    make_float4(h.x > 0.f ? acc[r][0] : 0.f, h.y > 0.f ? acc[r][1] : 0.f, h.z > 0.f ? acc[r][2] : 0.f,
+                                h.w > 0.f ? acc[r][3] : 0.f);
+            }
+            __syncthreads();
+            float *t = G;
+            G = Gn;
+            Gn = t;
+        }
+        // ---- first layer: dW1 (kH x kIn), db1
+        for (int i = tid; i < kH * 16; i += kMlpThreads) {
+            const int o = i % kH, k = i / kH;  // k == kIn: the bias
+            float s = 0.f;
+            for (int r = 0; r < R; ++r) s += G[r * kLd + o] * (k < kIn ? Xs[r * 16 + k] : 1.f);
+            float *d = k < kIn ? dP + o * kIn + k : dP + oB[0] + o;
+            *d = first ? s : *d + s;
+        }
+    }
+}
+
+// grads[i] = sum over the blocks' partial sums, in block order.  32 parameters x 8 slices of
+// the blocks per thread block: enough loads in flight to read the partials at L2 speed.
+__global__ void grad_sum_kernel(const float *__restrict__ part, int nblk, float *__restrict__ grads) {
+    __shared__ float sh[8][33];
+    const size_t i = (size_t)blockIdx.x * 32 + threadIdx.x;
+    const int per = (nblk + 7) / 8, b0 = threadIdx.y * per, b1 = min(nblk, b0 + per);
     float s = 0.f;
-    for (int i = 0; i < rows; ++i) s += G[i * ld + j];
-    out[j] = s;
+    if (i < kParams) {
+#pragma unroll 8
+        for (int b = b0; b < b1; ++b) s += part[(size_t)b * kParams + i];
+    }
+    sh[threadIdx.y][threadIdx.x] = s;
+    __syncthreads();
+    if (threadIdx.y == 0 && i < kParams) {
+#pragma unroll
+        for (int q = 1; q < 8; ++q) s += sh[q][threadIdx.x];
+        grads[i] = s;
+    }
 }
 
-__global__ void loss_grad_kernel(const float *pred, const float *y, int rows, float *G, float *loss_acc) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    float d = 0.f;
-    if (i < rows) {
-        d = pred[i] - y[i];
-        G[i] = 2.f * d / (float)rows;
-    }
-    float sq = nla::warp_sum(d * d);
-    if (loss_acc && (threadIdx.x & 31) == 0) atomicAdd(loss_acc, sq / (float)rows);
+// Floats of work for a batch of `rows`: the predictions and the blocks' partial gradients.
+size_t work_floats(int rows) { return (size_t)((rows + 63) & ~63) + (size_t)mlp_blocks(rows) * kParams; }
+
+// Predictions (into pred) and, when grads is given, the gradients of the mean squared error.
+cudaError_t mlp_pass(cudaStream_t st, const float *P, const float *X, const float *y, int rows, float *work,
+                     float *pred, float *grads, float *loss_acc) {
+    const int R = mlp_tile(rows), nblk = mlp_blocks(rows);
+    const size_t smem = mlp_smem_floats(R) * sizeof(float);
+    float *part = work + ((rows + 63) & ~63);
+    auto kern = R == 8 ? mlp_kernel<8> : mlp_kernel<32>;
+    static nla::PerDeviceOnce attr;
+    attr.run([] {
+        cudaFuncSetAttribute(mlp_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(mlp_smem_floats(8) * 4));
+        cudaFuncSetAttribute(mlp_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(mlp_smem_floats(32) * 4));
+        cudaGetLastError();
+    });
+    kern<<<nblk, kMlpThreads, smem, st>>>(P, X, y, rows, pred ? pred : work, part, loss_acc, grads ? 1 : 0);
+    if (grads) grad_sum_kernel<<<(int)((kParams + 31) / 32), dim3(32, 8), 0, st>>>(part, nblk, grads);
+    return cudaGetLastError();
 }
 
 __global__ void adam_kernel(float *w, const float *g, float *m, float *v, size_t count, float lr, float b1, float b2,
@@ -118,54 +320,6 @@ __global__ void gather_rows_kernel(const float *X, const float *y, const int *id
     int src = idx[i];
     for (int k = threadIdx.x; k < kIn; k += blockDim.x) Xb[i * kIn + k] = X[(long)src * kIn + k];
     if (threadIdx.x == 0) yb[i] = y[src];
-}
-
-// Work buffers for a batch of `rows`: Z1..Z3, H1..H3 (rows x 128), pred (rows), G (rows x 128) x 2.
-size_t work_floats(int rows) { return (size_t)rows * (6 * kH + 1 + 2 * kH) + 64; }
-
-struct Act {
-    float *Z[3], *H[3], *pred, *G0, *G1;
-};
-Act carve(float *w, int rows) {
-    Act a;
-    for (int l = 0; l < 3; ++l) {
-        a.Z[l] = w + (size_t)l * rows * kH;
-        a.H[l] = w + (size_t)(3 + l) * rows * kH;
-    }
-    a.pred = w + (size_t)6 * rows * kH;
-    a.G0 = a.pred + rows + 32;
-    a.G1 = a.G0 + (size_t)rows * kH;
-    return a;
-}
-
-void forward(cudaStream_t st, const float *P, const float *X, int rows, const Act &a) {
-    const float *h = X;
-    int in = kIn;
-    for (int l = 0; l < 3; ++l) {
-        gemm(st, rows, kH, in, h, in, 1, P + w_off(l), 1, in, a.Z[l], kH, 1, P + b_off(l), a.H[l], nullptr, 2);
-        h = a.H[l];
-        in = kH;
-    }
-    gemm(st, rows, 1, kH, h, kH, 1, P + w_off(3), 1, kH, a.pred, 1, 1, P + b_off(3), nullptr, nullptr, 1);
-}
-
-void backward(cudaStream_t st, const float *P, const float *X, const float *y, int rows, const Act &a, float *grads,
-              float *loss_acc) {
-    float *G = a.G0, *Gn = a.G1;
-    loss_grad_kernel<<<(rows + 255) / 256, 256, 0, st>>>(a.pred, y, rows, G, loss_acc);
-    int out = 1;
-    for (int l = 3; l >= 0; --l) {
-        const int in = kDims[l];
-        const float *Hprev = l == 0 ? X : a.H[l - 1];
-        // dW_l (out x in) = G^T Hprev
-        gemm(st, out, in, rows, G, 1, out, Hprev, in, 1, grads + w_off(l), in, 1, nullptr, nullptr, nullptr, 0);
-        colsum_kernel<<<(out + 127) / 128, 128, 0, st>>>(G, rows, out, out, grads + b_off(l));
-        if (l > 0) {  // G_{l-1} = (G W_l) .* [Z_{l-1} > 0]
-            gemm(st, rows, in, out, G, out, 1, P + w_off(l), in, 1, Gn, in, 1, nullptr, nullptr, a.Z[l - 1], 3);
-            std::swap(G, Gn);
-        }
-        out = in;
-    }
 }
 
 struct Model {
@@ -243,9 +397,8 @@ nla_status mlp_predict_host(const char *model_path, const float *X, int rows, fl
     } else {
         cudaMemcpyAsync(dP, m.params.data(), kParams * sizeof(float), cudaMemcpyHostToDevice, st);
         cudaMemcpyAsync(dX, Xs.data(), Xs.size() * sizeof(float), cudaMemcpyHostToDevice, st);
-        Act a = carve(dW, rows);
-        forward(st, dP, dX, rows, a);
-        cudaMemcpyAsync(y, a.pred, rows * sizeof(float), cudaMemcpyDeviceToHost, st);
+        mlp_pass(st, dP, dX, nullptr, rows, dW, dW, nullptr, nullptr);
+        cudaMemcpyAsync(y, dW, rows * sizeof(float), cudaMemcpyDeviceToHost, st);
         if (cudaStreamSynchronize(st) != cudaSuccess) s = merr(NLA_ERR_CUDA, "MLP inference failed");
         for (int i = 0; i < rows; ++i) y[i] = y[i] * m.ysd + m.ymean;
     }
@@ -269,11 +422,7 @@ nla_status kt_mlp_forward_backward(const float *dParams, const float *dX, const 
     if (rows <= 0 || !dParams || !dX || !dY || !dGrads || !dWork) return merr(NLA_ERR_ARG, "bad arguments");
     if (work_bytes < kt_mlp_work_bytes(rows)) return merr(NLA_ERR_WORKSPACE, "MLP workspace too small");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    Act a = carve(reinterpret_cast<float *>(dWork), rows);
-    forward(st, dParams, dX, rows, a);
-    backward(st, dParams, dX, dY, rows, a, dGrads, nullptr);
-    if (dPred) cudaMemcpyAsync(dPred, a.pred, rows * sizeof(float), cudaMemcpyDeviceToDevice, st);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = mlp_pass(st, dParams, dX, dY, rows, reinterpret_cast<float *>(dWork), dPred, dGrads, nullptr);
     return e == cudaSuccess ? NLA_OK : merr(NLA_ERR_CUDA, cudaGetErrorString(e));
 }
 
@@ -360,9 +509,7 @@ nla_status kt_mlp_train(const float *X, const float *y, int rows, int epochs, in
             int nb = 0;
             for (int b0 = 0; b0 + batch <= rows; b0 += batch, ++nb) {
                 gather_rows_kernel<<<batch, 32, 0, st>>>(dX, dY, dIdx + b0, batch, dXb, dYb);
-                Act a = carve(dW, batch);
-                forward(st, dP, dXb, batch, a);
-                backward(st, dP, dXb, dYb, batch, a, dG, dLoss);
+                mlp_pass(st, dP, dXb, dYb, batch, dW, nullptr, dG, dLoss);
                 kt_mlp_adam_step(dP, dG, dM, dV, kParams, ++t, lr, st);
             }
             float h = 0.f;

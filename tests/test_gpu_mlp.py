@@ -49,6 +49,28 @@ def test_forward_backward_match_oracle(kt):
             assert np.max(np.abs(a - r)) <= 1e-3 * max(1e-6, np.max(np.abs(r)))
 
 
+@pytest.mark.parametrize("rows,shift", [(1, 0), (7, 0), (8, 1), (9, 0), (33, 0), (2432, 0), (2433, 0), (5000, 3)])
+def test_forward_backward_at_tile_edges(kt, rows, shift):
+    # batches around the row tiles (8 rows up to 2432, 32 above; blocks that take several tiles) and
+    # parameters that are not 16-byte aligned; the same bound as the plain case
+    params = omlp.init(15, seed=30 + rows)
+    p32 = pack(params)
+    params = unpack(p32.astype(np.float64), params)
+    g = np.random.default_rng(rows)
+    X = g.standard_normal((rows, 15)).astype(np.float32)
+    y = g.standard_normal(rows).astype(np.float32)
+    buf = torch.empty(p32.size + shift, dtype=torch.float32, device="cuda")
+    buf[shift:] = torch.from_numpy(p32).cuda()
+    pred, grads = kt.mlp_forward_backward(buf[shift:], torch.from_numpy(X).cuda(), torch.from_numpy(y).cuda())
+    torch.cuda.synchronize()
+    p_ref, _ = omlp.forward(params, X.astype(np.float64))
+    assert np.max(np.abs(pred.cpu().numpy() - p_ref)) <= 1e-3 * max(1.0, np.max(np.abs(p_ref)))
+    g_gpu = unpack(grads.cpu().numpy().astype(np.float64), params)
+    for (gW, gb), (rW, rb) in zip(g_gpu, omlp.backward(params, X.astype(np.float64), y.astype(np.float64))):
+        for a, r in ((gW, rW), (gb, rb)):
+            assert np.max(np.abs(a - r)) <= 1e-3 * max(1e-6, np.max(np.abs(r)))
+
+
 def test_adam_step_matches_oracle(kt):
     params = omlp.init(15, seed=5)
     p32 = pack(params)
