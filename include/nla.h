@@ -172,7 +172,10 @@ nla_status nla_band_extract(int n, int band, nla_dtype dtype, const void *dA, in
  * matrix in dAB (layout of nla_band_extract, overwritten) to upper bidiagonal
  * form by Householder bulge chasing; dD (n) and dE (n-1) receive the FP64
  * diagonal and superdiagonal.  dWork: >= nla_band2bd_workspace bytes (the
- * sweeps' progress counters; the library allocates nothing on this path). */
+ * sweeps' progress counters and, for bands of 8, 16, 32 and 64, a packed copy of
+ * the band; with room for the counters only, n ints, the chase works on dAB
+ * itself, which is slower unless ldab is the packed leading dimension; the
+ * library allocates nothing on this path). */
 nla_status nla_band2bd_workspace(int n, int band, nla_dtype dtype, size_t *bytes);
 nla_status nla_band2bd(int n, int band, nla_dtype dtype, void *dAB, int ldab, double *dD,
                        double *dE, void *dWork, size_t work_bytes, int *dInfo,

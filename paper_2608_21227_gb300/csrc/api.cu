@@ -282,7 +282,7 @@ GesvdLayout gesvd_layout(char *base, int m, int n, nla_dtype dt, const nla_opts 
     carve_stage1(cv, M, N, dt, p.b, p.update, L.s1);
     L.ldw = (long)align_up((size_t)std::max(M, 1), 32);
     L.Aw = need_copy ? cv.take<char>(es * L.ldw * N) : nullptr;
-    L.ldab = 3 * p.b + 1;
+    L.ldab = std::max(nla::chase_ld(p.b, (int)es), 3 * p.b + 1);
     L.AB = cv.take<char>(es * L.ldab * std::max(N, 1));
     L.prog = cv.take<char>(nla::band2bd_scratch_bytes(N));
     L.bd = cv.take<char>(nla::bdsvd_scratch_bytes(N));
@@ -290,6 +290,17 @@ GesvdLayout gesvd_layout(char *base, int m, int n, nla_dtype dt, const nla_opts 
     L.e = cv.take<double>(std::max(N, 1));
     L.bytes = align_up(cv.off, 256);
     return L;
+}
+
+// Workspace of nla_band2bd: the sweeps' progress counters and, for the band widths that are
+// chased in packed form, the packed band.
+struct Band2bdLayout {
+    size_t packed_off, bytes;
+};
+Band2bdLayout band2bd_layout(int n, int band, nla_dtype dt) {
+    const size_t es = elem_size(dt), cnt = align_up(nla::band2bd_scratch_bytes(n), 256);
+    const size_t ld = (size_t)nla::chase_ld(band, (int)es);
+    return {ld ? cnt : 0, align_up(cnt + ld * es * (size_t)std::max(n, 1), 256)};
 }
 
 template <typename T>
@@ -435,10 +446,8 @@ nla_status nla_band_extract(int n, int band, nla_dtype dtype, const void *dA, in
 }
 
 nla_status nla_band2bd_workspace(int n, int band, nla_dtype dtype, size_t *bytes) {
-    (void)band;
-    (void)dtype;
     if (!bytes || n < 0) return fail(NLA_ERR_ARG, "bad arguments");
-    *bytes = align_up(nla::band2bd_scratch_bytes(n), 256);
+    *bytes = band2bd_layout(n, band, dtype).bytes;
     return NLA_OK;
 }
 
@@ -454,10 +463,14 @@ nla_status nla_band2bd(int n, int band, nla_dtype dtype, void *dAB, int ldab, do
         return fail(NLA_ERR_WORKSPACE, "workspace too small");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     NLA_CUDA(cudaMemsetAsync(dInfo, 0, sizeof(int), st), "memset info");
+    // a workspace that holds the counters but not the packed band is enough: the chase then
+    // works on the caller's storage
+    const Band2bdLayout L = band2bd_layout(n, band, dtype);
+    void *packed = L.packed_off && work_bytes >= L.bytes && (uintptr_t)dWork % 16 == 0 ? (char *)dWork + L.packed_off : nullptr;
     if (dtype == NLA_F64)
-        NLA_LAUNCH(nla::kTrBand2bd, st, nla::band2bd<double>((double *)dAB, ldab, n, band, dD, dE, dWork, dInfo, st), "bulge chase");
+        NLA_LAUNCH(nla::kTrBand2bd, st, nla::band2bd<double>((double *)dAB, ldab, n, band, dD, dE, dWork, dInfo, st, (double *)packed), "bulge chase");
     else
-        NLA_LAUNCH(nla::kTrBand2bd, st, nla::band2bd<float>((float *)dAB, ldab, n, band, dD, dE, dWork, dInfo, st), "bulge chase");
+        NLA_LAUNCH(nla::kTrBand2bd, st, nla::band2bd<float>((float *)dAB, ldab, n, band, dD, dE, dWork, dInfo, st, (float *)packed), "bulge chase");
     return NLA_OK;
 }
 

@@ -291,11 +291,9 @@ NLA_DEV void house_scalars(T alpha, T xn2, T &beta, T &tau, T &scale) {
     }
 }
 
-// One block step (right + left reflector) of sweep s at position k by one warp;
-// sl0 = window slot of column c0 = s + k b + 1.  B = the band width when it is a
-// compile-time constant (<= 32: the reflector and the lane's row or column are then
-// held in registers, every load issues at once and nothing is reloaded), 0 otherwise.
-template <typename T, int B>
+// One half of a block step (part 0: right reflector, 1: left) of sweep s at position k by
+// one warp; sl0 = window slot of column c0 = s + k b + 1.
+template <typename T>
 NLA_DEV void warp_chase_step(const Win<T> &W, int n, int b, int s, int k, int sl0, T *v, int part) {
     const int lane = threadIdx.x & 31;
     const int c0 = s + k * b + 1;
@@ -304,11 +302,10 @@ NLA_DEV void warp_chase_step(const Win<T> &W, int n, int b, int s, int k, int sl
     const int cend = min(s + (k + 2) * b, n - 1);
     const int L = c1 - c0 + 1;
     if (L < 2) return;
-    constexpr int UB = (B > 0 && B <= 32) ? B : 1;
     T xa, xb, xn2, alpha, tau, beta, scale;
     if (part == 1) goto left;
     // ---- right reflector on columns c0..c1 from row tr, applied to rows tr+1..c1
-    // (lane c < 32 holds entry (tr, c0 + c); L <= 64 for the generic form)
+    // (lane c < 32 holds entries (tr, c0 + c) and (tr, c0 + 32 + c))
     xa = lane < L ? W.col_from(sl0, c0, lane)[tr] : T(0);
     xb = lane + 32 < L ? W.col_from(sl0, c0, lane + 32)[tr] : T(0);
     xn2 = warp_sum((lane > 0 ? xa * xa : T(0)) + xb * xb);
@@ -324,55 +321,11 @@ NLA_DEV void warp_chase_step(const Win<T> &W, int n, int b, int s, int k, int sl
             W.col_from(sl0, c0, lane + 32)[tr] = T(0);
         }
         __syncwarp();
-        if (B > 0 && B <= 32 && L == B) {
-            T vr[UB];
-#pragma unroll
-            for (int c = 0; c < UB; ++c) vr[c] = v[c];
-            // apply to the lane's row held in xr (columns c0 .. c0 + B - 1)
-            auto apply_row = [&](T(&xr)[UB]) {
-                T d0 = T(0), d1 = T(0), d2 = T(0), d3 = T(0);
-#pragma unroll
-                for (int c = 0; c < UB; c += 4) {
-                    d0 += xr[c] * vr[c];
-                    if (c + 1 < UB) d1 += xr[c + 1] * vr[c + 1];
-                    if (c + 2 < UB) d2 += xr[c + 2] * vr[c + 2];
-                    if (c + 3 < UB) d3 += xr[c + 3] * vr[c + 3];
-                }
-                const T w = tau * ((d0 + d1) + (d2 + d3));
-#pragma unroll
-                for (int c = 0; c < UB; ++c) xr[c] -= w * vr[c];
-            };
-            if (sl0 + B <= W.wc) {
-                // the B columns sit in consecutive slots: entry (i, c0 + c) is
-                // base[i + c (ldw - 1)], constant offsets from one address per lane
-                constexpr int LDW1 = ((3 * UB + 2) & ~1) - 1;
-                T *base = W.w + (size_t)sl0 * W.ldw + W.b2 - c0;
-                for (int i = tr + 1 + lane; i <= c1; i += 32) {  // one lane per row
-                    T *rp = base + i;
-                    T xr[UB];
-#pragma unroll
-                    for (int c = 0; c < UB; ++c) xr[c] = rp[c * LDW1];
-                    apply_row(xr);
-#pragma unroll
-                    for (int c = 0; c < UB; ++c) rp[c * LDW1] = xr[c];
-                }
-            } else {
-                for (int i = tr + 1 + lane; i <= c1; i += 32) {
-                    T xr[UB];
-#pragma unroll
-                    for (int c = 0; c < UB; ++c) xr[c] = W.col_from(sl0, c0, c)[i];
-                    apply_row(xr);
-#pragma unroll
-                    for (int c = 0; c < UB; ++c) W.col_from(sl0, c0, c)[i] = xr[c];
-                }
-            }
-        } else {
-            for (int i = tr + 1 + lane; i <= c1; i += 32) {  // one lane per row
-                T w = T(0);
-                for (int c = 0; c < L; ++c) w += W.col_from(sl0, c0, c)[i] * v[c];
-                w *= tau;
-                for (int c = 0; c < L; ++c) W.col_from(sl0, c0, c)[i] -= w * v[c];
-            }
+        for (int i = tr + 1 + lane; i <= c1; i += 32) {  // one lane per row
+            T w = T(0);
+            for (int c = 0; c < L; ++c) w += W.col_from(sl0, c0, c)[i] * v[c];
+            w *= tau;
+            for (int c = 0; c < L; ++c) W.col_from(sl0, c0, c)[i] -= w * v[c];
         }
         __syncwarp();
     }
@@ -395,35 +348,12 @@ left:
             clw[lane + 32] = T(0);
         }
         __syncwarp();
-        if (B > 0 && B <= 32 && L == B) {
-            T vr[UB];
-#pragma unroll
-            for (int r = 0; r < UB; ++r) vr[r] = v[r];
-            for (int j = c0 + 1 + lane; j <= cend; j += 32) {  // one lane per column
-                T *cj = W.col_from(sl0, c0, j - c0) + c0;
-                T xr[UB];
-#pragma unroll
-                for (int r = 0; r < UB; ++r) xr[r] = cj[r];
-                T d0 = T(0), d1 = T(0), d2 = T(0), d3 = T(0);
-#pragma unroll
-                for (int r = 0; r < UB; r += 4) {
-                    d0 += xr[r] * vr[r];
-                    if (r + 1 < UB) d1 += xr[r + 1] * vr[r + 1];
-                    if (r + 2 < UB) d2 += xr[r + 2] * vr[r + 2];
-                    if (r + 3 < UB) d3 += xr[r + 3] * vr[r + 3];
-                }
-                const T w = tau * ((d0 + d1) + (d2 + d3));
-#pragma unroll
-                for (int r = 0; r < UB; ++r) cj[r] = xr[r] - w * vr[r];
-            }
-        } else {
-            for (int j = c0 + 1 + lane; j <= cend; j += 32) {  // one lane per column
-                T *cj = W.col_from(sl0, c0, j - c0);
-                T w = T(0);
-                for (int r = 0; r < L; ++r) w += v[r] * cj[c0 + r];
-                w *= tau;
-                for (int r = 0; r < L; ++r) cj[c0 + r] -= w * v[r];
-            }
+        for (int j = c0 + 1 + lane; j <= cend; j += 32) {  // one lane per column
+            T *cj = W.col_from(sl0, c0, j - c0);
+            T w = T(0);
+            for (int r = 0; r < L; ++r) w += v[r] * cj[c0 + r];
+            w *= tau;
+            for (int r = 0; r < L; ++r) cj[c0 + r] -= w * v[r];
         }
         __syncwarp();
     }
@@ -469,68 +399,23 @@ NLA_DEV void cp_async_elem(T *dst_smem, const T *src) {
 NLA_DEV void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Mover warp: copy band columns j0..j1 (3b+1 storage rows each) between global
-// memory and the window.  With the compact layout (ldab = 3b+1) the columns are
-// one contiguous run in global memory: lanes walk it element by element (coalesced);
-// otherwise column by column.  Loads are asynchronous copies that all issue before
-// the one wait (a single memory latency per call); write-backs keep eight loads from
-// the window in flight before their stores.
-template <typename T, bool LOAD, int B>
+// memory and the window.  Loads are asynchronous copies that all issue before
+// the one wait (a single memory latency per call).
+template <typename T, bool LOAD>
 NLA_DEV void mover_copy(const Win<T> &W, const Band<T> &A, int n, int b, int j0, int j1, int lane) {
     const int h = 3 * b + 1;
-    if (LOAD) {
-        if (B > 0 && A.ldab == (long)(3 * B + 1)) {
-            constexpr int H = 3 * B + 1;
-            const T *g = A.AB + (long)j0 * H;
-            const int tot = (j1 - j0 + 1) * H;
-            const int sl0 = j0 % W.wc;
-            for (int e = lane; e < tot; e += 32) {
-                int sl = sl0 + e / H;
-                sl -= sl >= W.wc ? W.wc : 0;
-                cp_async_elem(W.w + (size_t)sl * W.ldw + (e % H), g + e);
-            }
-        } else {
-            for (int j = j0; j <= j1; ++j) {
-                T *cw = W.col(j);
-                for (int q = lane; q < h; q += 32) {
-                    const int i = j + q - 2 * b;
-                    if (i >= 0 && i < n) cp_async_elem(cw + i, A.at(i, j));
-                }
-            }
-        }
-        cp_async_wait_all();
-        return;
-    }
-    if (B > 0 && A.ldab == (long)(3 * B + 1)) {
-        constexpr int H = 3 * B + 1;
-        T *g = A.AB + (long)j0 * H;
-        const int tot = (j1 - j0 + 1) * H;
-        const int sl0 = j0 % W.wc;
-        for (int base = 0; base < tot; base += 32 * 8) {
-            T r[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int e = base + u * 32 + lane;
-                if (e < tot) {
-                    int sl = sl0 + e / H;
-                    sl -= sl >= W.wc ? W.wc : 0;
-                    r[u] = W.w[(size_t)sl * W.ldw + (e % H)];
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int e = base + u * 32 + lane;
-                if (e < tot) __stcg(g + e, r[u]);
-            }
-        }
-        return;
-    }
     for (int j = j0; j <= j1; ++j) {
-        const T *cw = W.col(j);
+        T *cw = W.col(j);
         for (int q = lane; q < h; q += 32) {
             const int i = j + q - 2 * b;
-            if (i >= 0 && i < n) __stcg(A.at(i, j), cw[i]);
+            if (i < 0 || i >= n) continue;
+            if (LOAD)
+                cp_async_elem(cw + i, A.at(i, j));
+            else
+                __stcg(A.at(i, j), cw[i]);
         }
     }
+    if (LOAD) cp_async_wait_all();
 }
 
 // Bounded spin of a chase warp on the window's "loaded up to" column.
@@ -556,7 +441,7 @@ NLA_DEV bool wait_loaded(volatile int *sh_hi, int hi, volatile int *sh_abort, in
 // done[group]; the loader brings in, up to `pf` steps ahead, the columns the
 // previous group has released.  The window holds columns [flushed + 1, loaded]
 // in wc >= (2G - 1) b + G + 1 + pf b circular slots.
-template <typename T, int B>
+template <typename T>
 __global__ void band2bd_group_kernel(T *AB, long ldab, int n, int b, int G, int wc, int pf, int *done, int *info) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     // chase progress, loaded-up-to column, flushed-up-to column, loader finished, abort flag
@@ -618,13 +503,13 @@ __global__ void band2bd_group_kernel(T *AB, long ldab, int n, int b, int G, int 
                             wslot += b;
                             if (wslot >= wc) wslot -= wc;
                         }
-                        warp_chase_step<T, B>(W, n, b, s, k, wslot, v, 0);  // right reflector
+                        warp_chase_step<T>(W, n, b, s, k, wslot, v, 0);  // right reflector
                     }
                 }
                 // the right reflectors of this step all precede every left reflector:
                 // with sweeps two steps apart that is the order the sequential chase needs
                 asm volatile("bar.sync 1, %0;" ::"r"(32 * G) : "memory");
-                if (ok && mine) warp_chase_step<T, B>(W, n, b, s, k, wslot, v, 1);  // left reflector
+                if (ok && mine) warp_chase_step<T>(W, n, b, s, k, wslot, v, 1);  // left reflector
                 asm volatile("bar.sync 1, %0;" ::"r"(32 * G) : "memory");
                 if (*vabort) break;
                 if (warp == 0 && lane == 0) {
@@ -658,7 +543,7 @@ __global__ void band2bd_group_kernel(T *AB, long ldab, int n, int b, int G, int 
                     __threadfence_block();
                     if (*vabort) break;
                     const int fin = *vhi;
-                    if (fin > flushed) mover_copy<T, false, B>(W, A, n, b, flushed + 1, fin, lane);
+                    if (fin > flushed) mover_copy<T, false>(W, A, n, b, flushed + 1, fin, lane);
                     __threadfence();
                     __syncwarp();
                     if (lane == 0) st_release(&done[grp], INT_MAX);
@@ -666,7 +551,7 @@ __global__ void band2bd_group_kernel(T *AB, long ldab, int n, int b, int G, int 
                 }
                 const int fin = lo - 1;  // columns <= fin are final
                 if (fin > flushed) {
-                    mover_copy<T, false, B>(W, A, n, b, flushed + 1, fin, lane);
+                    mover_copy<T, false>(W, A, n, b, flushed + 1, fin, lane);
                     flushed = fin;
                     __threadfence();
                     __syncwarp();
@@ -715,7 +600,7 @@ __global__ void band2bd_group_kernel(T *AB, long ldab, int n, int b, int G, int 
                     }
                     const int avail = min(want, have - 1);
                     if (avail > loaded) {
-                        mover_copy<T, true, B>(W, A, n, b, loaded + 1, avail, lane);
+                        mover_copy<T, true>(W, A, n, b, loaded + 1, avail, lane);
                         loaded = avail;
                         __syncwarp();
                         __threadfence_block();
@@ -764,64 +649,61 @@ __global__ void bidiag_extract_kernel(const T *__restrict__ AB, long ldab, int n
 
 template <typename T>
 cudaError_t band2bd(T *AB, long ldab, int n, int b, double *d, double *e, void *scratch, int *info,
-                    cudaStream_t st) {
+                    cudaStream_t st, T *packed) {
     if (n <= 0) return cudaSuccess;
     int *progress = reinterpret_cast<int *>(scratch);
     const int nsweeps = n - 2;
     const size_t kGroupBudget = 200 * 1024;
-    // Sweeps per block: FP32 up to 16 (the occupancy check below lowers it to what one
-    // SM holds), FP64 4 -- an FP64 block step is bound by the SM's small FP64 pipe, so
-    // more sweeps per SM slow every step down (measured at n = 256, 2048 and 8192).
-    // NLA_CHASE_GROUP overrides it (0: one sweep per block on the global band).
+    // NLA_CHASE_GROUP: sweeps per block (0: one sweep per block on the global band)
     static const int gset = [] {
         const char *v = getenv("NLA_CHASE_GROUP");
-        return v ? atoi(v) : (sizeof(T) == 8 ? 4 : 16);
+        return v ? std::max(0, atoi(v)) : -1;
     }();
-    auto kern = b == 16 ? band2bd_group_kernel<T, 16>
-                : b == 32 ? band2bd_group_kernel<T, 32>
-                : b == 64 ? band2bd_group_kernel<T, 64> : band2bd_group_kernel<T, 0>;
+    if (nsweeps > 0 && gset != 0 && chase_ld(b, (int)sizeof(T)) > 0) {
+        const int ld = chase_ld(b, (int)sizeof(T));
+        T *P = AB;
+        long ldp = ldab;
+        if (packed && ldab != ld) {
+            cudaError_t err = band_repack<T>(AB, ldab, packed, ld, n, b, st);
+            if (err != cudaSuccess) return err;
+            P = packed;
+            ldp = ld;
+        }
+        cudaError_t err = chase_fixed<T>(P, ldp, n, b, std::max(gset, 0), progress, info, st);
+        if (err != cudaSuccess) return err;
+        if (P != AB) {
+            err = band_repack<T>(P, ldp, AB, ldab, n, b, st);
+            if (err != cudaSuccess) return err;
+        }
+        bidiag_extract_kernel<T><<<(n + 255) / 256, 256, 0, st>>>(P, ldp, n, b, d, e);
+        return cudaGetLastError();
+    }
+    // ---- other band widths.  Sweeps per block: FP32 up to 16, FP64 4 -- an FP64 block step
+    // is bound by the SM's small FP64 pipe, so more sweeps per SM slow every step down.
+    const int gwant = gset >= 0 ? gset : (sizeof(T) == 8 ? 4 : 16);
+    auto kern = band2bd_group_kernel<T>;
     static PerDeviceOnce gattr;
     gattr.run([&] {
-        for (auto k : {band2bd_group_kernel<T, 0>, band2bd_group_kernel<T, 16>, band2bd_group_kernel<T, 32>,
-                       band2bd_group_kernel<T, 64>})
-            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGroupBudget);
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGroupBudget);
         cudaGetLastError();
     });
     // the largest G (<= the requested one) whose block -- G chase warps + 2 movers, its
-    // window -- is resident on every SM (registers, shared memory), cached per device and
-    // band width (16, 32, 64; other widths are asked every call)
-    auto pick_group = [&](int &G, int &pf) {
-        G = 0;
-        pf = 0;
-        for (int gmax = std::min(gset, 30); gmax >= 1; --gmax) {
-            int p2 = 0;
-            const int g2 = chase_group_size(b, (int)sizeof(T), kGroupBudget, gmax, p2);
-            if (g2 < 1) break;
-            const int wc2 = (kLag * g2 - 1) * b + g2 + 1 + p2 * b;
-            const size_t sm2 = (size_t)wc2 * ((3 * b + 2) & ~1) * sizeof(T) + (size_t)g2 * 64 * sizeof(T);
-            int nb = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, 32 * (g2 + 2), sm2) == cudaSuccess && nb >= 1) {
-                G = g2;
-                pf = p2;
-                break;
-            }
-            cudaGetLastError();
-            gmax = std::min(gmax, g2);
-        }
-    };
-    static PerDeviceValue<int2> gcache[4];
-    const int ci = b == 16 ? 1 : b == 32 ? 2 : b == 64 ? 3 : 0;
+    // window -- is resident on every SM (registers, shared memory)
     int G = 0, pf = 0;
-    if (gset > 0 && ci > 0) {
-        const int2 gp = gcache[ci].get([&] {
-            int g = 0, p = 0;
-            pick_group(g, p);
-            return make_int2(g, p);
-        });
-        G = gp.x;
-        pf = gp.y;
-    } else if (gset > 0) {
-        pick_group(G, pf);
+    for (int gmax = std::min(gwant, 30); gmax >= 1; --gmax) {
+        int p2 = 0;
+        const int g2 = chase_group_size(b, (int)sizeof(T), kGroupBudget, gmax, p2);
+        if (g2 < 1) break;
+        const int wc2 = (kLag * g2 - 1) * b + g2 + 1 + p2 * b;
+        const size_t sm2 = (size_t)wc2 * ((3 * b + 2) & ~1) * sizeof(T) + (size_t)g2 * 64 * sizeof(T);
+        int nb = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, 32 * (g2 + 2), sm2) == cudaSuccess && nb >= 1) {
+            G = g2;
+            pf = p2;
+            break;
+        }
+        cudaGetLastError();
+        gmax = std::min(gmax, g2);
     }
     if (nsweeps > 0 && b > 1 && G >= 1) {
         const int ngroups = (nsweeps + G - 1) / G;
@@ -872,7 +754,7 @@ cudaError_t band2bd(T *AB, long ldab, int n, int b, double *d, double *e, void *
 #define NLA_INST(T)                                                                                       \
     template cudaError_t copy_matrix<T>(const T *, long, int, int, T *, long, bool, cudaStream_t);      \
     template cudaError_t band_extract<T>(const T *, long, int, int, T *, long, cudaStream_t);           \
-    template cudaError_t band2bd<T>(T *, long, int, int, double *, double *, void *, int *, cudaStream_t);
+    template cudaError_t band2bd<T>(T *, long, int, int, double *, double *, void *, int *, cudaStream_t, T *);
 NLA_INST(double)
 NLA_INST(float)
 #undef NLA_INST

@@ -104,9 +104,18 @@ cudaError_t band_extract(const T *A, long lda, int n, int b, T *AB, long ldab, c
 
 // ---------------------------------------------------------------- stage 2 / 3
 size_t band2bd_scratch_bytes(int n);
+// scratch: band2bd_scratch_bytes(n).  packed (may be NULL): room for n columns of chase_ld
+// entries, 16-byte aligned, where a band with another leading dimension is chased (its columns
+// then move as bulk copies); the result is copied back.
 template <typename T>
 cudaError_t band2bd(T *AB, long ldab, int n, int b, double *d, double *e, void *scratch,
-                    int *info, cudaStream_t st);
+                    int *info, cudaStream_t st, T *packed = nullptr);
+// chase.cu: the chase for band widths 8, 16, 32, 64 (chase_ld > 0: its packed leading dimension).
+int chase_ld(int b, int elem);
+template <typename T>
+cudaError_t chase_fixed(T *AB, long ldab, int n, int b, int gmax, int *done, int *info, cudaStream_t st);
+template <typename T>
+cudaError_t band_repack(const T *src, long lds, T *dst, long ldd, int n, int b, cudaStream_t st);
 size_t bdsvd_scratch_bytes(int n);
 template <typename T>
 cudaError_t bdsvd_bisect(int n, const double *d, const double *e, T *S, void *scratch, int *info,

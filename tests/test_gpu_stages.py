@@ -115,3 +115,48 @@ def test_stage3_minors_keep_their_signs(nla, dt, n, kind):
     assert int(info.item()) == 0
     B = np.diag(d) + np.diag(e, 1)
     assert err_rel(S.double().cpu().numpy(), np.linalg.svd(B, compute_uv=False)) <= (n * 2.0 ** -51 if dt == 0 else 2.0 ** -20)
+
+
+@pytest.mark.parametrize("dt", [0, 1])
+@pytest.mark.parametrize("b", [7, 8, 16, 32, 64])
+@pytest.mark.parametrize("n", ["3", "b", "b+1", "2*b", "2*b+2", "5*b+3"])
+@pytest.mark.parametrize("store", ["packed", "plain", "wide", "counters_only"])
+def test_stage2_widths_edges_and_storage(nla, dt, b, n, store):
+    # sizes around one and two block steps; the band in the chase's own leading dimension, in the
+    # compact one, in a wider one, and with a workspace that holds the counters only
+    import ctypes
+
+    n = max(3, eval(n, {"b": b}))
+    per = 2 if dt == 0 else 4
+    ldab = {"packed": (3 * b + per) // per * per, "plain": 3 * b + 1, "wide": 3 * b + 6,
+            "counters_only": 3 * b + 1}[store]
+    g = np.random.default_rng(50 * b + n)
+    i, j = np.indices((n, n))
+    D = np.where((j - i >= 0) & (j - i <= b), g.standard_normal((n, n)), 0.0)
+    tdt = torch.float64 if dt == 0 else torch.float32
+    if dt == 1:
+        D = D.astype(np.float32).astype(np.float64)
+    AB = np.zeros((n, ldab))
+    for c in range(n):
+        for r in range(max(0, c - b), c + 1):
+            AB[c, 2 * b + r - c] = D[r, c]
+    t = torch.from_numpy(AB).to("cuda", tdt)
+    L = nla.lib()
+    need = ctypes.c_size_t(0)
+    assert L.nla_band2bd_workspace(n, b, dt, ctypes.byref(need)) == 0
+    bytes_ = 4 * n if store == "counters_only" else need.value
+    work = torch.empty(max(bytes_, 256), dtype=torch.uint8, device="cuda")
+    d = torch.empty(n, dtype=torch.float64, device="cuda")
+    e = torch.empty(n, dtype=torch.float64, device="cuda")
+    info = torch.zeros(1, dtype=torch.int32, device="cuda")
+    st = L.nla_band2bd(n, b, dt, t.data_ptr(), ldab, d.data_ptr(), e.data_ptr(), work.data_ptr(), bytes_,
+                       info.data_ptr(), None, torch.cuda.current_stream().cuda_stream)
+    assert st == 0
+    torch.cuda.synchronize()
+    assert int(info.item()) == 0
+    dn, en = d.cpu().numpy(), e.cpu().numpy()[: n - 1]
+    assert err_rel(oracle.bdsvd(dn, en), oracle.svdvals(D)) <= tol_for(dt, n)
+    # the band storage holds the bidiagonal
+    got = t.double().cpu().numpy()
+    assert np.array_equal(got[:, 2 * b], dn)
+    assert np.array_equal(got[1:, 2 * b - 1], en)
