@@ -29,6 +29,7 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "house.cuh"
 #include "tc.cuh"
 
 namespace cg = cooperative_groups;
@@ -530,37 +531,6 @@ panel_cluster_kernel(T *__restrict__ P, long rs, long cs, int M, int nb, int R, 
     cluster.sync();  // no block leaves while another may still write to its shared memory
 }
 
-// ------------------------------------------------------------------ register-resident cluster variant
-// The same factorisation with each thread holding its panel rows in registers
-// (thread t of block p owns rows r0 + t + 512 q, q < RP; nb = NB fixed).  With
-// column indices instead of item indices, the partial sums of column j are
-//   x . a_c over rows below j, for every column c:
-//   c == j: ||x||^2;  c > j: x . a_c (trailing);  c < j: x . v_c (finished reflector c),
-// so one product per owned entry gives them all.  Per column: products and a warp
-// reduce-scatter in registers, per-warp sums into shared memory, a block barrier;
-// warp 0 adds the warps, pushes the block's sums (and row j, by its owner) to every
-// block over DSMEM, arrives on their barriers, waits for its own, forms beta / tau
-// and the coefficients; a block barrier; every thread updates its own rows.  Two
-// block barriers per column and no shared-memory pass over the panel.
-
-// Sum v[0..NB-1] over the warp's lanes, leaving the sum of column (NB == 32 ? lane
-// : lane >> 1) in the return value: halving exchanges (upper lanes keep the upper half).
-template <typename T, int NB>
-NLA_DEV T warp_reduce_scatter(T (&v)[NB], int lane) {
-#pragma unroll
-    for (int h = NB / 2, o = 16; h >= 1; h /= 2, o /= 2) {
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int i = 0; i < h; ++i) {
-            const T send = up ? v[i] : v[i + h];
-            const T keep = up ? v[i + h] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-        }
-    }
-    if (NB == 16) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
-    return v[0];
-}
-
 // Asynchronous store into another block's shared memory that completes as bytes on
 // that block's mbarrier (release at cluster scope); addresses from cluster_addr.
 NLA_DEV void st_async_remote(uint32_t addr, float v, uint32_t mbar) {
@@ -579,236 +549,269 @@ NLA_DEV void mbar_arrive_expect_tx(uint64_t *mbar, uint32_t bytes) {
                  : "memory");
 }
 
-template <typename T, int NB>
-NLA_DEV T select_col(const T (&a)[NB], int j) {
-    T x = T(0);
-#pragma unroll
-    for (int c = 0; c < NB; ++c) x = c == j ? a[c] : x;
-    return x;
+// ------------------------------------------------------------------ register-resident cluster variant
+// The same factorisation with the panel in registers, a thread owning R rows of one
+// column: lane c of a warp holds column c (NB = 32), or column c % 16 of one of two row groups
+// (NB = 16), so a warp holds all columns of its rows.  Column j then costs
+//   - the owner lanes' x (column j below the diagonal) through the warp's own shared memory,
+//     one 128-bit broadcast per four rows: no block barrier, no select;
+//   - R multiply-adds for x . a_c, the whole sum over the warp's rows but for one shuffle: c ==
+//     j gives ||x||^2, c > j the trailing columns, c < j the Gram matrix of the reflectors;
+//   - the warps' sums through shared memory and one block barrier;
+//   - with several blocks, every warp pushes the block's sums to its share of the blocks as
+//     st.async stores that complete as bytes on the receiver's mbarrier, and every warp
+//     waits on that mbarrier itself (no second block barrier);
+//   - the reflector's scalars in every warp, and R multiply-adds for the update.
+// Finished columns keep x unscaled until the panel is written: the scale of column c is one
+// number in its owners' registers.  Row j leaves the registers with column j (it is final then):
+// its group moves the rows below up by one, so the pivot row is always register 0.  T is formed by an extra warp of block 0, one column
+// behind the others, from the Gram column that warp 0 leaves in shared memory.
+//
+// Bound: latency of the chain above, per column (FP32 about 0.7 us, of which one exchange
+// between blocks is 0.2 us).  The variant this replaced, a thread per row with 16 products per
+// thread and column, a 16-value warp reduce-scatter and selects over the columns, took 1.7 us a
+// column; panel_reg_launch has the times per panel.
+
+constexpr int kRegWarps = 15;  // row warps per block at most (with the extra one: 128 registers a thread)
+
+// beta, tau and the scale 1 / (alpha - beta) of the reflector of [alpha; x], xn2 = ||x||^2 > 0.
+NLA_DEV void panel_scalars(float alpha, float xn2, float &beta, float &tau, float &scale) {
+    const float q = fmaf(alpha, alpha, xn2);
+    const float rs = rsqrtf(q), r = q * rs;
+    beta = alpha >= 0.f ? -r : r;
+    tau = fmaf(fabsf(alpha), rs, 1.f);
+    scale = __fdividef(1.f, alpha - beta);
+}
+NLA_DEV void panel_scalars(double alpha, double xn2, double &beta, double &tau, double &scale) {
+    double u0, g, one;
+    house(alpha, xn2, beta, u0, g, one);  // g = 1 / (|beta| |u0|)
+    const double ug = u0 * g;             // +-1 / |beta|
+    tau = u0 * ug;
+    scale = g * -beta;  // sign(u0) = -sign(beta)
 }
 
-template <typename T, int NB, int RP>
-__global__ void __launch_bounds__(kClusterThreads, 1)
-panel_reg_kernel(T *__restrict__ P, long rs, long cs, int M, int R, T *__restrict__ tau, T *__restrict__ Tm,
-                 int *info) {
+template <typename T, int NB, int R>
+__global__ void __launch_bounds__(32 * (kRegWarps + 1), 1)
+panel_reg_kernel(T *__restrict__ P, long rs, long cs, int M, int nb, int nw, T *__restrict__ tau,
+                 T *__restrict__ Tm, int *info) {
     pdl_wait();
     pdl_trigger();
     static_assert(NB == 16 || NB == 32, "NB");
+    constexpr int HV = 32 / NB, kMaxWarps = kRegWarps + 1, VEC = 16 / (int)sizeof(T);
+    constexpr int RT = R < NB ? R : NB;  // pivot rows a group can hold
     cg::cluster_group cluster = cg::this_cluster();
     const int p = (int)cluster.block_rank(), nP = (int)cluster.num_blocks();
-    constexpr int kWarps = kClusterThreads / 32;
-    __shared__ T red[kWarps][NB];   // per-warp column sums
-    __shared__ T inbox[2][16][NB];  // by column parity and source block
-    __shared__ T rowin[2][NB];
-    __shared__ T myrow[NB];
-    __shared__ T wcoef[NB];  // tau (v . a_c) for c > j, 0 otherwise
+    __shared__ __align__(16) T xs[kMaxWarps * HV * R];  // x of the current column, per row group
+    __shared__ T red[2][kMaxWarps][NB];                 // by column parity: the warps' column sums
+    __shared__ T inbox[2][16][NB];                      // the blocks' column sums
+    __shared__ T rowj[2][NB], rowin[2][NB];             // row j (block 0's, received)
+    // block 0: T(i, k), i <= k, at Tsh[i + k*NB]; G(i, k) = v_i . v_k, i < k, at Gsh[i + k*NB]
+    __shared__ T Tsh[NB * NB], Gsh[NB * NB];
+    __shared__ T top[NB][NB];  // block 0: the finished rows
     __shared__ T taus[NB];
-    // block 0: T(i, k), i <= k, at Tsh[i + k*NB]; G(i, k) = v_i . v_k, i < k, at Tsh[k + i*NB]
-    __shared__ T Tsh[NB * NB];
     __shared__ __align__(8) uint64_t mbar[2];
-    __shared__ T sh_scale, sh_beta;
     __shared__ int sh_abort;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int r0 = p * R;
-    const int nr = max(0, min(M, r0 + R) - r0);
-    const int kmax = min(NB, M);
+    const int c = lane % NB, group = warp * HV + lane / NB;
+    const int gr0 = (p * nw * HV + group) * R;  // first of the thread's rows
+    const int kmax = min(nb, M);
     if (tid == 0) {
-        // one arrival per phase (this block's expect_tx); the other blocks' partial sums
-        // and the owner's row j complete it as transaction bytes
+        // one arrival per phase (this block's expect_tx); the blocks' sums and row j
+        // complete it as transaction bytes
         tc::mbar_init(&mbar[0], 1);
         tc::mbar_init(&mbar[1], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         sh_abort = 0;
     }
     if (p == 0) {
-        for (int j = kmax + tid; j < NB; j += blockDim.x) tau[j] = T(0);
+        for (int j = kmax + tid; j < nb; j += blockDim.x) tau[j] = T(0);
         for (int i = tid; i < NB * NB; i += blockDim.x) Tsh[i] = T(0);
     }
-    T a[RP][NB];
-    // a row whose NB entries are contiguous and 16-byte aligned (the LQ panel: rs = ldx,
-    // cs = 1) moves as 16-byte vectors
-    const bool vec = cs == 1 && (rs * (long)sizeof(T)) % 16 == 0 && reinterpret_cast<uintptr_t>(P) % 16 == 0;
+    const int bar_threads = 32 * (p == 0 ? nw + 1 : nw);
+    const auto block_bar = [&] { asm volatile("bar.sync 1, %0;" ::"r"(bar_threads) : "memory"); };
+    if (warp < nw) {
+        T a[R];
+        // a column's rows are contiguous on the QR side: 16-byte vectors where they are aligned
+        T *Pc = P + (long)gr0 * rs + (long)c * cs;
+        const bool vec = rs == 1 && gr0 + R <= M && c < nb && reinterpret_cast<uintptr_t>(Pc) % 16 == 0;
+        if (vec) {
 #pragma unroll
-    for (int q = 0; q < RP; ++q) {
-        const int rr = tid + kClusterThreads * q;
-        if (vec && rr < nr) {
-            if constexpr (sizeof(T) == 4) {
-                const float4 *src = reinterpret_cast<const float4 *>(P + (long)(r0 + rr) * rs);
+            for (int i = 0; i < R; i += VEC) {
+                const float4 f = *reinterpret_cast<const float4 *>(Pc + i);
+                const T *q = reinterpret_cast<const T *>(&f);
 #pragma unroll
-                for (int u = 0; u < NB / 4; ++u) {
-                    const float4 f = src[u];
-                    a[q][4 * u] = f.x, a[q][4 * u + 1] = f.y, a[q][4 * u + 2] = f.z, a[q][4 * u + 3] = f.w;
-                }
-            } else {
-                const double2 *src = reinterpret_cast<const double2 *>(P + (long)(r0 + rr) * rs);
-#pragma unroll
-                for (int u = 0; u < NB / 2; ++u) {
-                    const double2 f = src[u];
-                    a[q][2 * u] = f.x, a[q][2 * u + 1] = f.y;
-                }
+                for (int u = 0; u < VEC; ++u) a[i + u] = q[u];
             }
         } else {
 #pragma unroll
-            for (int c = 0; c < NB; ++c) a[q][c] = rr < nr ? P[(long)(r0 + rr) * rs + (long)c * cs] : T(0);
+            for (int i = 0; i < R; ++i) a[i] = gr0 + i < M && c < nb ? Pc[(long)i * rs] : T(0);
         }
-    }
-    cluster.sync();  // every block's barriers are initialised before the first remote arrive
-    for (int j = 0; j < kmax; ++j) {
-        const int buf = j & 1;
-        T prod[NB];
-#pragma unroll
-        for (int c = 0; c < NB; ++c) prod[c] = T(0);
-#pragma unroll
-        for (int q = 0; q < RP; ++q) {
-            const int rr = tid + kClusterThreads * q;
-            const T x = (rr < nr && r0 + rr > j) ? select_col<T, NB>(a[q], j) : T(0);
-#pragma unroll
-            for (int c = 0; c < NB; ++c) prod[c] = fma(x, a[q][c], prod[c]);
+        T myscale = T(1);
+        if (nP > 1) {
+            cluster.sync();  // every block's barriers are initialised before the first remote store
+        } else {
+            block_bar();
         }
-        const T wsum = warp_reduce_scatter<T, NB>(prod, lane);
-        if (NB == 32 || (lane & 1) == 0) red[warp][NB == 32 ? lane : lane >> 1] = wsum;
-        if (j >= r0 && j < r0 + nr) {  // the owner of row j publishes it
-            const int rr = j - r0;
-            if (tid == rr % kClusterThreads) {
+        T *xw = xs + group * R;
+        for (int j = 0; j < kmax; ++j) {
+            const int buf = j & 1;
+            const bool pivot = p == 0 && gr0 <= j && j < gr0 + RT;  // the thread holds row j, in a[0]
+            T rv = a[0];
+            if (c == j) {
 #pragma unroll
-                for (int q = 0; q < RP; ++q)
-                    if (q == rr / kClusterThreads) {
+                for (int i = 0; i < R; i += VEC) {
+                    float4 f;
+                    T *q = reinterpret_cast<T *>(&f);
 #pragma unroll
-                        for (int c = 0; c < NB; ++c) myrow[c] = a[q][c];
-                    }
+                    for (int u = 0; u < VEC; ++u) q[u] = i + u == 0 && pivot ? T(0) : a[i + u];
+                    *reinterpret_cast<float4 *>(xw + i) = f;
+                }
             }
-        }
-        __syncthreads();
-        if (warp == 0) {
-            const bool owner = j >= r0 && j < r0 + nr;
-            if (lane == 0) mbar_arrive_expect_tx(&mbar[buf], (uint32_t)((nP + 1) * NB * sizeof(T)));
-            // lane l pushes column c = l mod NB to blocks l / NB, l / NB + 32 / NB, ...
-            const int c = lane % NB;
-            T sblk = T(0);
+            if (pivot) rowj[buf][c] = rv;
+            __syncwarp();
+            T x[R];
 #pragma unroll
-            for (int w = 0; w < kWarps; ++w) sblk += red[w][c];
-            const T rv = owner ? myrow[c] : T(0);
-            for (int q = lane / NB; q < nP; q += 32 / NB) {
-                const uint32_t mb = cluster_addr(&mbar[buf], q);
-                st_async_remote(cluster_addr(&inbox[buf][p][c], q), sblk, mb);
-                if (owner) st_async_remote(cluster_addr(&rowin[buf][c], q), rv, mb);
+            for (int i = 0; i < R; i += VEC) {
+                const float4 f = *reinterpret_cast<const float4 *>(xw + i);
+                const T *q = reinterpret_cast<const T *>(&f);
+#pragma unroll
+                for (int u = 0; u < VEC; ++u) x[i + u] = q[u];
             }
-            if (lane == 0 && !sh_abort) {
+            T s[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) s[u] = x[u] * a[u];
+#pragma unroll
+            for (int i = 4; i < R; ++i) s[i % 4] = fma(x[i], a[i], s[i % 4]);
+            T sum = (s[0] + s[1]) + (s[2] + s[3]);
+            if (HV == 2) sum += __shfl_xor_sync(0xffffffffu, sum, 16);
+            if (lane < NB) red[buf][warp][c] = sum;
+            block_bar();
+            // ---- the block's sums (in every warp, in a fixed order: HV == 2 halves add the even and odd warps)
+            sum = T(0);
+#pragma unroll
+            for (int w = 0; w < kMaxWarps; w += HV) {
+                const int v = w + (HV == 2 ? lane / NB : 0);
+                sum += v < nw ? red[buf][v][c] : T(0);
+            }
+            if (HV == 2) sum += __shfl_xor_sync(0xffffffffu, sum, 16);
+            if (nP > 1) {
+                if (tid == 0) mbar_arrive_expect_tx(&mbar[buf], (uint32_t)((nP + 1) * NB * sizeof(T)));
+                const T rj = p == 0 ? rowj[buf][c] : T(0);
+                for (int q = warp * HV + lane / NB; q < nP; q += nw * HV) {
+                    const uint32_t mb = cluster_addr(&mbar[buf], q);
+                    st_async_remote(cluster_addr(&inbox[buf][p][c], q), sum, mb);
+                    if (p == 0) st_async_remote(cluster_addr(&rowin[buf][c], q), rj, mb);
+                }
                 const uint32_t par = (uint32_t)((j >> 1) & 1);
                 if (!mbar_try_wait_cluster(&mbar[buf], par)) {
                     const unsigned long long t0 = global_ns();
+                    volatile int *vab = &sh_abort;
                     while (!mbar_try_wait_cluster(&mbar[buf], par)) {
+                        if (*vab) break;
                         if (global_ns() - t0 > kSpinBudgetNs) {
                             if (info) atomicExch(info, kInfoTimeout);
-                            sh_abort = 1;
+                            *vab = 1;
                             break;
                         }
                     }
                 }
-            }
-            __syncwarp();  // lane 0's acquire orders the warp's reads below
-            T sc_ = T(0), wc_ = T(0);
-            if (lane < NB) {
-                // unrolled over the largest cluster with the size as a predicate: the loads
-                // issue together instead of one load-to-add latency per block
+                __syncwarp();
+                sum = T(0);
 #pragma unroll
-                for (int q = 0; q < 16; ++q) sc_ += q < nP ? inbox[buf][q][lane] : T(0);
-                wc_ = rowin[buf][lane];
-            }
-            const T alpha = __shfl_sync(0xffffffffu, wc_, j), xn2 = __shfl_sync(0xffffffffu, sc_, j);
-            T tj = T(0), beta = alpha, scale = T(0);
-            if (xn2 > T(0)) {
-                if constexpr (sizeof(T) == 4) {  // a few ulp, far inside the FP32 path's tolerance
-                    const float q = alpha * alpha + xn2;
-                    const float r = q * rsqrtf(q);
-                    beta = alpha >= 0.f ? -r : r;
-                    tj = __fdividef(beta - alpha, beta);
-                    scale = __fdividef(1.f, alpha - beta);
-                } else {
-                    const T r = sqrt(alpha * alpha + xn2);
-                    beta = alpha >= T(0) ? -r : r;
-                    tj = (beta - alpha) / beta;
-                    scale = T(1) / (alpha - beta);
+                for (int w = 0; w < 16; w += HV) {  // (the cluster size as a predicate: the loads issue together)
+                    const int q = w + (HV == 2 ? lane / NB : 0);
+                    sum += q < nP ? inbox[buf][q][c] : T(0);
                 }
-            }
-            if (lane < NB) {
-                const T vdot = wc_ + scale * sc_;  // v . a_c (c > j) or G(c, j) = v_c . v_j (c < j)
-                wcoef[lane] = lane > j ? tj * vdot : T(0);
-                if (p == 0 && lane < j) Tsh[j + lane * NB] = vdot;
-            }
-            if (lane == 0) {
-                sh_scale = scale;
-                sh_beta = beta;
-                taus[j] = tj;
-                if (p == 0) tau[j] = tj;
-            }
-        }
-        __syncthreads();
-        const T tj = taus[j];
-        if (tj != T(0)) {
-            const T scl = sh_scale, bt = sh_beta;
-            T w[NB];
-#pragma unroll
-            for (int c = 0; c < NB; ++c) w[c] = wcoef[c];
-#pragma unroll
-            for (int q = 0; q < RP; ++q) {
-                const int rr = tid + kClusterThreads * q, gr = r0 + rr;
-                if (rr < nr && gr >= j) {
-                    // rows below j: a_c -= v w_c with v = x / (alpha - beta), and v into column j;
-                    // row j: a_c -= w_c (v_j = 1), beta into column j
-                    const T v = gr > j ? select_col<T, NB>(a[q], j) * scl : T(1);
-#pragma unroll
-                    for (int c = 0; c < NB; ++c) a[q][c] = c == j ? (gr > j ? v : bt) : fma(-v, w[c], a[q][c]);
-                }
-            }
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < RP; ++q) {
-        const int rr = tid + kClusterThreads * q;
-        if (rr < nr) {
-            if (vec) {
-                if constexpr (sizeof(T) == 4) {
-                    float4 *dst = reinterpret_cast<float4 *>(P + (long)(r0 + rr) * rs);
-#pragma unroll
-                    for (int u = 0; u < NB / 4; ++u)
-                        dst[u] = make_float4(a[q][4 * u], a[q][4 * u + 1], a[q][4 * u + 2], a[q][4 * u + 3]);
-                } else {
-                    double2 *dst = reinterpret_cast<double2 *>(P + (long)(r0 + rr) * rs);
-#pragma unroll
-                    for (int u = 0; u < NB / 2; ++u) dst[u] = make_double2(a[q][2 * u], a[q][2 * u + 1]);
-                }
+                if (HV == 2) sum += __shfl_xor_sync(0xffffffffu, sum, 16);
+                rv = rowin[buf][c];
             } else {
+                rv = rowj[buf][c];
+            }
+            // ---- the reflector
+            const T alpha = __shfl_sync(0xffffffffu, rv, j), xn2 = __shfl_sync(0xffffffffu, sum, j);
+            T beta = alpha, tj = T(0), scale = T(0);
+            if (xn2 > T(0)) panel_scalars(alpha, xn2, beta, tj, scale);
+            const T vdot = (rv + scale * sum) * myscale;  // v . a_c (c > j) or G(c, j) = v_c . v_j (c < j)
+            const T w = c > j ? tj * vdot : T(0);
+            if (c == j && tj != T(0)) myscale = scale;
+            if (p == 0 && warp == 0 && lane < NB) {
+                if (c < j) Gsh[c + j * NB] = vdot;
+                if (c == j) taus[j] = tau[j] = tj;
+            }
+            // ---- rows below j: a_c -= x (scale w_c); row j: a_c -= w_c, beta in column j
+            const T m = -scale * w;
 #pragma unroll
-                for (int c = 0; c < NB; ++c) P[(long)(r0 + rr) * rs + (long)c * cs] = a[q][c];
+            for (int i = 0; i < R; ++i) a[i] = fma(x[i], m, a[i]);
+            if (p == 0 && warp * HV * R < NB) {
+                if (pivot) top[j][c] = c < j ? rv * myscale : c == j ? beta : rv - w;
+#pragma unroll
+                for (int i = 0; i < RT; ++i) a[i] = !pivot ? a[i] : i + 1 < RT ? a[i + 1] : T(0);
             }
         }
-    }
-    if (p == 0) {
-        __syncthreads();
-        // T(0:k, k) = -tau_k T(0:k, 0:k) G(0:k, k), T(k, k) = tau_k -- one warp, column by column
-        if (warp == 0) {
-            // lane i forms T(i, kk) = -tau_kk sum_{i <= q < kk} T(i, q) G(q, kk); the q loop is
-            // unrolled over the whole width with the range as a predicate, so its loads issue at once
-            for (int kk = 0; kk < kmax; ++kk) {
-                const T tk = taus[kk];
-                if (lane < kk) {
-                    T t = T(0);
+        if (p == 0) block_bar();  // the last Gram column is there
+        // ---- v = x / (alpha - beta) below the diagonal, and the panel back to memory
 #pragma unroll
-                    for (int q = 0; q < NB; ++q) {
-                        const T tv = Tsh[lane + q * NB], gv = Tsh[kk + q * NB];  // T(i, q), G(q, kk)
-                        t = (q >= lane && q < kk) ? fma(tv, gv, t) : t;
-                    }
-                    Tsh[lane + kk * NB] = -tk * t;
+        for (int i = 0; i < R; ++i) a[i] *= myscale;
+        if (p == 0 && gr0 < NB) {
+            // rows below the last pivot that still sit where they were moved to
+            const int gone = min(max(kmax - gr0, 0), RT);
+            for (int r = gone; r < RT; ++r) {
+                top[gr0 + r][c] = a[0];
+#pragma unroll
+                for (int i = 0; i + 1 < RT; ++i) a[i] = a[i + 1];
+            }
+#pragma unroll
+            for (int i = 0; i < RT; ++i) a[i] = top[gr0 + i][c];
+        }
+        if (vec) {
+#pragma unroll
+            for (int i = 0; i < R; i += VEC) {
+                float4 f;
+                T *q = reinterpret_cast<T *>(&f);
+#pragma unroll
+                for (int u = 0; u < VEC; ++u) q[u] = a[i + u];
+                *reinterpret_cast<float4 *>(Pc + i) = f;
+            }
+        } else if (c < nb) {
+#pragma unroll
+            for (int i = 0; i < R; ++i)
+                if (gr0 + i < M) Pc[(long)i * rs] = a[i];
+        }
+    } else {
+        // ---------------- the extra warp: T(0:k, k) = -tau_k T(0:k, 0:k) G(0:k, k), T(k, k) = tau_k
+        if (nP > 1) cluster.sync();
+        if (p == 0) {
+            if (nP == 1) block_bar();
+            for (int j = 0; j <= kmax; ++j) {
+                block_bar();
+                const int k = j - 1;  // its Gram column was left before this barrier
+                if (k < 0) continue;
+                T t = T(0);
+                if (lane < k) {
+#pragma unroll 4
+                    for (int q = 0; q < k; ++q) t = fma(Tsh[lane + q * NB], Gsh[q + k * NB], t);
                 }
-                if (lane == 0) Tsh[kk + kk * NB] = tk;
+                if (lane < k) Tsh[lane + k * NB] = -taus[k] * t;
+                if (lane == k) Tsh[k + k * NB] = taus[k];
                 __syncwarp();
             }
+            for (int idx = lane; idx < nb * nb; idx += 32) {
+                const int i = idx % nb, k = idx / nb;
+                Tm[idx] = i <= k ? Tsh[i + k * NB] : T(0);
+            }
         }
-        __syncthreads();
-        for (int idx = tid; idx < NB * NB; idx += blockDim.x) Tm[idx] = (idx % NB) <= (idx / NB) ? Tsh[idx] : T(0);
     }
-    cluster.sync();  // no block leaves while another may still write to its shared memory
+    if (nP > 1) cluster.sync();  // no block leaves while another may still write to its shared memory
+}
+
+// NLA_PANEL_CLUSTER: cluster size of the shared-memory variant where it fits (0: the grid
+// kernel for every panel); -1 when not set.
+static int panel_cluster_forced() {
+    static const int force = [] {
+        const char *v = getenv("NLA_PANEL_CLUSTER");
+        return v ? atoi(v) : -1;
+    }();
+    return force;
 }
 
 // Cluster size and rows per block for an M x nb panel, or 0 if it does not fit one cluster.
@@ -856,10 +859,7 @@ static int cluster_plan(int M, int nb, int &R, size_t &dyn) {
     const bool *sched = caps.sched;
     int k0 = 0;
     while (k0 < 4 && (1 << k0) * kPanelRowsTarget < M) ++k0;  // smallest size with <= 256 rows per block
-    static const int force = [] {  // NLA_PANEL_CLUSTER: cluster size to use where it fits (0: grid kernel)
-        const char *v = getenv("NLA_PANEL_CLUSTER");
-        return v ? atoi(v) : -1;
-    }();
+    const int force = panel_cluster_forced();
     if (force == 0) return 0;
     int best = 0;
     for (int k = 0; k < 5; ++k) {
@@ -877,20 +877,27 @@ static int cluster_plan(int M, int nb, int &R, size_t &dyn) {
     return best;
 }
 
-// Register-resident cluster panel for the shapes it is built for (nb 16 or 32, one
-// row per thread: at most 512 rows per block); cudaErrorNotSupported otherwise.
-// NLA_PANEL_REG=0 keeps the shared-memory variant.
-template <typename T, int NB, int RP>
-cudaError_t panel_reg_launch_nb(T *P, long rs, long cs, int M, int R, int C, T *tau, T *Tm, int *info,
+// Register-resident panel: nb <= 32 columns and as many rows as 16 blocks hold; otherwise
+// cudaErrorNotSupported.  NLA_PANEL_REG=0 keeps the shared-memory variant.
+// Blocks of four row warps (one per SM sub-partition) up to 16 blocks, taller blocks above that.
+template <typename T, int NB, int R>
+cudaError_t panel_reg_launch_nb(T *P, long rs, long cs, int M, int nb, int max_warps, T *tau, T *Tm, int *info,
                                 cudaStream_t st) {
+    constexpr int per_warp = 32 / NB * R;  // rows
+    const int warps = (M + per_warp - 1) / per_warp;
+    int C = 1;
+    while (C < 16 && C * 4 < warps) C *= 2;
+    // (block 0 holds every pivot row)
+    const int nw = std::max((warps + C - 1) / C, C > 1 ? (NB + per_warp - 1) / per_warp : 1);
+    if (nw > max_warps) return cudaErrorNotSupported;
     static PerDeviceOnce attr;
     attr.run([] {
-        cudaFuncSetAttribute(panel_reg_kernel<T, NB, RP>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        cudaFuncSetAttribute(panel_reg_kernel<T, NB, R>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         cudaGetLastError();
     });
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(C);
-    cfg.blockDim = dim3(kClusterThreads);
+    cfg.blockDim = dim3(32 * (nw + 1));
     cfg.dynamicSmemBytes = 0;
     cfg.stream = st;
     cudaLaunchAttribute at[2];
@@ -902,26 +909,36 @@ cudaError_t panel_reg_launch_nb(T *P, long rs, long cs, int M, int R, int C, T *
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = pdl_enabled() ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, panel_reg_kernel<T, NB, RP>, P, rs, cs, M, R, tau, Tm, info);
+    return cudaLaunchKernelEx(&cfg, panel_reg_kernel<T, NB, R>, P, rs, cs, M, nb, nw, tau, Tm, info);
 }
 
+// Rows per thread.  FP32: 16 while 16 blocks of eight warps hold them (4,096 rows at 16
+// columns), then 32 (us per panel at 16 columns, R = 16 / 32: 1,024 rows 15.5 / 15.9, 3,001 rows
+// 17.2 / 18.2, 8,192 rows with R = 32 and 8 warps 19.4; 16 columns of 8,192 rows took 32 before).
+// FP64: 16 at 16 columns (2,048 rows: 57 us against 160 before), 8 at 32 columns while they fit
+// (256 rows: 104 us, 117 with 16, 355 before); its chain is the FP64 pipe's, so spreading the
+// rows over more SMs matters more than the exchange.
 template <typename T>
-cudaError_t panel_reg_launch(T *P, long rs, long cs, int M, int nb, int R, int C, T *tau, T *Tm, int *info,
-                             cudaStream_t st) {
+cudaError_t panel_reg_launch(T *P, long rs, long cs, int M, int nb, T *tau, T *Tm, int *info, cudaStream_t st) {
     static const bool on = [] {
         const char *v = getenv("NLA_PANEL_REG");
         return !v || atoi(v) != 0;
     }();
-    if (!on || C > 16) return cudaErrorNotSupported;
-    const int rp = (R + kClusterThreads - 1) / kClusterThreads;
+    if (!on || nb > 32) return cudaErrorNotSupported;
+    cudaError_t e = cudaErrorNotSupported;
     if constexpr (sizeof(T) == 4) {
-        // (two or more rows per thread spill at the 128-register limit of 512 threads)
-        if (nb == 16 && rp == 1) return panel_reg_launch_nb<T, 16, 1>(P, rs, cs, M, R, C, tau, Tm, info, st);
-        if (nb == 32 && rp == 1) return panel_reg_launch_nb<T, 32, 1>(P, rs, cs, M, R, C, tau, Tm, info, st);
+        e = nb <= 16 ? panel_reg_launch_nb<T, 16, 16>(P, rs, cs, M, nb, 8, tau, Tm, info, st)
+                     : panel_reg_launch_nb<T, 32, 16>(P, rs, cs, M, nb, 8, tau, Tm, info, st);
+        if (e == cudaErrorNotSupported)
+            e = nb <= 16 ? panel_reg_launch_nb<T, 16, 32>(P, rs, cs, M, nb, kRegWarps, tau, Tm, info, st)
+                         : panel_reg_launch_nb<T, 32, 32>(P, rs, cs, M, nb, kRegWarps, tau, Tm, info, st);
+    } else if (nb <= 16) {
+        e = panel_reg_launch_nb<T, 16, 16>(P, rs, cs, M, nb, kRegWarps, tau, Tm, info, st);
     } else {
-        if (nb == 16 && rp == 1) return panel_reg_launch_nb<T, 16, 1>(P, rs, cs, M, R, C, tau, Tm, info, st);
+        e = panel_reg_launch_nb<T, 32, 8>(P, rs, cs, M, nb, 4, tau, Tm, info, st);
+        if (e == cudaErrorNotSupported) e = panel_reg_launch_nb<T, 32, 16>(P, rs, cs, M, nb, kRegWarps, tau, Tm, info, st);
     }
-    return cudaErrorNotSupported;
+    return e;
 }
 
 template <typename T>
@@ -929,21 +946,15 @@ cudaError_t panel_factor(T *P, long rs, long cs, int M, int nb, T *tau, T *Tm, c
                          cudaStream_t st) {
     if (M <= 0 || nb <= 0) return cudaSuccess;
     if (nb > kNbMax) return cudaErrorInvalidValue;
-    {  // preferred: one thread-block cluster, no global barrier
+    if (panel_cluster_forced() < 0) {  // preferred: rows in registers, one thread-block cluster
+        cudaError_t e = panel_reg_launch<T>(P, rs, cs, M, nb, tau, Tm, ctl.info, st);
+        if (e == cudaSuccess) return e;
+        cudaGetLastError();  // not available for this shape: shared-memory variant
+    }
+    {
         int R = 0;
         size_t dyn = 0;
         const int C = cluster_plan<T>(M, nb, R, dyn);
-        if (C > 0) {
-            // rows in registers: one row per thread, so the smallest cluster with at
-            // most 512 rows per block (fewer blocks, fewer exchanges per column)
-            int Cr = 1;
-            while (Cr < 16 && (long)Cr * kClusterThreads < M) Cr *= 2;
-            const int Rr = (M + Cr - 1) / Cr;
-            cudaError_t e = Rr <= kClusterThreads ? panel_reg_launch<T>(P, rs, cs, M, nb, Rr, Cr, tau, Tm, ctl.info, st)
-                                                  : cudaErrorNotSupported;
-            if (e == cudaSuccess) return e;
-            cudaGetLastError();  // not available for this shape: shared-memory variant
-        }
         if (C > 0) {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(C);

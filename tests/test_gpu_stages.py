@@ -160,3 +160,22 @@ def test_stage2_widths_edges_and_storage(nla, dt, b, n, store):
     got = t.double().cpu().numpy()
     assert np.array_equal(got[:, 2 * b], dn)
     assert np.array_equal(got[1:, 2 * b - 1], en)
+
+
+@pytest.mark.parametrize("dt", [0, 1])
+@pytest.mark.parametrize("m,n,b", [(5, 5, 16), (16, 16, 16), (17, 16, 16), (31, 20, 8), (33, 33, 32), (129, 40, 4), (192, 64, 32),
+                                   (1025, 40, 16), (2049, 37, 32), (4097, 33, 16), (7681, 33, 16), (8193, 33, 32),
+                                   (15361, 20, 16), (16385, 40, 32)])
+def test_stage1_panel_row_limits(nla, dt, m, n, b):
+    # panels around the rows a warp, a block and a cluster hold (odd leading dimensions: no vector
+    # loads), widths below and at the compiled ones, and rows beyond every register variant
+    A = np.random.default_rng(m + n + b).standard_normal((m, n))
+    if dt == 1:
+        A = A.astype(np.float32).astype(np.float64)
+    t = to_device_colmajor(A, torch.float64 if dt == 0 else torch.float32)
+    tq, tp, info = nla.gebrd_band(t, b)
+    ABt = nla.band_extract(t, min(b, n))
+    d, e, info2 = nla.band2bd(ABt, min(b, n))
+    torch.cuda.synchronize()
+    assert int(info.item()) == 0 and int(info2.item()) == 0
+    assert err_rel(oracle.bdsvd(d.cpu().numpy(), e.cpu().numpy()), np.linalg.svd(A, compute_uv=False)) <= tol_for(dt, m)
