@@ -131,7 +131,7 @@ nla_status kt_tune(const kt_problem *problem, kt_strategy strategy, double budge
  * configurations and the pipeline-level band width); nla_gesvd_vals consults
  * it whenever opts->cfg is NULL, matching
  * dtype, update precision and side and taking the entry nearest in log size;
- * side-2 entries set the batched kernel's threads per matrix (cfg.band) for
+ * side-2 entries set the batched kernel's least threads per matrix (cfg.band) for
  * size bucket m (0..4).  path NULL clears the table. */
 nla_status kt_load_config(const char *path);
 

@@ -1,574 +1,565 @@
 // batched.cu -- singular values of many small matrices of uneven shapes in one
-// persistent launch (the batched form of the two-stage method, Section 5.1.1).
+// persistent launch (the batched form of the method of Section 5.1.1).
 //
-//  1. prep kernel (one block): orders the batch by element count, largest first
-//     (bitonic sort of (count, index) keys in shared memory), so that blocks
-//     draw similar matrices together and the long ones start first; counts the
-//     matrices too large for shared memory and sets the work counters.
-//     Everything stays on the device, so the whole call can be captured into a
+//  1. prep kernel (one block): orders the batch by (class, cost), most expensive first
+//     (a counting sort), so that blocks draw similar matrices together and the long ones
+//     start first.  Everything stays on the device, so the whole call can be captured into a
 //     CUDA graph.
-//  2. large-matrix kernel (4 blocks of 256 threads per SM, no matrix shared
-//     memory): one of those large matrices per block, in the block's global
-//     scratch slot (L2-resident); with several blocks per SM more of these
-//     latency-bound reductions are in flight.
-//  3. persistent kernel (one block of 256 threads per SM, 192 KiB of shared
-//     memory for matrices): each block takes rounds of the remaining work from
-//     an atomic counter.  In a round it splits into
-//     groups of g threads -- g chosen per size bucket (kt_load_config installs
-//     tuned values; defaults otherwise) -- and each group reduces one matrix:
-//       * the matrix (or its transpose, so that m >= n) is copied into the
-//         group's share of shared memory when it fits, else into a global
-//         scratch slot of the block (L2-resident at these sizes);
-//       * band width 1: one-stage Householder bidiagonalisation (the band
-//         stage degenerates to the bidiagonal for these sizes), left and right
-//         reflectors with group-wide reductions;
-//       * the bidiagonal singular values by bisection on Sturm counts of the
-//         Golub-Kahan tridiagonal, one thread per value (FP32 arithmetic for
-//         FP32 matrices: the batched accuracy target 5e-6 N sigma_1 is met and
-//         the FP64 pipe is 64x slower on this GPU).
-//     Groups synchronise with named barriers (bar.sync id, g).
+//  2. persistent kernel (one block of 16 warps per SM): each block takes units of work from an
+//     atomic counter; a unit is one matrix for all 16 warps, two for 8 warps each, four for 4,
+//     or sixteen for one warp each, by the classes below.
+//
+// A matrix (or its transpose, M >= N) lives in the registers of its warps: lane l of
+// warp w holds rows l, l + 32, ... of columns w, w + NW, ... .
+//   - M beyond the rows the registers hold: R of the QR factorisation first, by chunks of rows.
+//     R (packed, shared memory) and a chunk are reduced to the next R column by column; a column
+//     belongs to one warp, so a step is: the owner publishes column j, one barrier, every warp
+//     forms its dot products, reduces them over its lanes and updates its columns.
+//   - One-stage Householder bidiagonalisation of the register tile (band width 1: the band stage
+//     degenerates for these sizes): the left reflector as above; the right one needs each row's
+//     sum over the warps (two barriers).
+//   - The bidiagonal's values by multisection on Sturm counts (FP32; sturm.cuh), with all
+//     threads of the matrix.
+// Columns are taken in order k NW + w0 with k unrolled, so that register indices are
+// constants, finished columns and rows drop out of the loops, and the code of one k serves NW
+// columns.
+//
+// What bounds it: the chain of a column (one to three barriers and a reduction over the lanes,
+// about 700 cycles) for the small classes, multiply-add issue for the large ones.  Before, the
+// matrix lived in shared memory or, above 48K elements, in global memory, and every reflector
+// streamed it twice.
 #include <algorithm>
 #include <cstdlib>
-#include <cfloat>
-#include <vector>
+#include <utility>
 
 #include "../../include/nla.h"
 #include "common.cuh"
 #include "kernels.cuh"
+#include "sturm.cuh"
 #include "trace.h"
 #include "tuned.h"
 
 namespace {
 
-constexpr int kBThreads = 256;
-constexpr int kBSmemElems = 48 * 1024;      // floats of shared memory for matrices per block (192 KiB)
-constexpr int kSortMax = 16384;             // batches up to this size are sorted
-constexpr int kBuckets = 5;
-// Buckets by element count m*n: <= 1/8, 1/4, 1/2, 1 of the block's matrix shared memory, or more
-// (global scratch).  A bucket-b matrix fits one group's share when g >= kMinGroup[b].
-// (the largest bucket runs in the large-matrix kernel, which takes 128 or 256)
-const int kMinGroup[kBuckets] = {32, 64, 128, 256, 128};
+constexpr int kWarps = 16, kThreads = 32 * kWarps;
+constexpr int kBuckets = 5;      // size buckets of the tuned table, by element count
+constexpr int kBucketElems = 48 * 1024;
+constexpr int kClasses = 5;      // 0: N <= 256, 1: N <= 192 (16 warps), 2: N <= 128 (8), 3: N <= 64 (4), 4: N <= 32 (1)
+constexpr int kCostBins = 128;   // per class, eighths of a power of two of the cost
 
+// Least threads per matrix for each size bucket (the tuned table's group sizes): a matrix is
+// given to the smallest class that holds its N and has as many threads.
 struct BatchCfg {
-    int group[kBuckets];  // threads per matrix for each bucket
+    int group[kBuckets];
 };
-
-__device__ int bucket_of(long elems) {
-    int b = 0;
-    while (b < kBuckets - 1 && elems > (long)kBSmemElems >> (kBuckets - 2 - b)) ++b;
-    return b;
-}
 
 nla_status berr(nla_status s, const char *m) {
     nla_set_last_error(m);
     return s;
 }
 
+__host__ __device__ inline int class_warps(int c) { return c <= 1 ? 16 : c == 2 ? 8 : c == 3 ? 4 : 1; }
+
+__device__ int class_of(long m, long n, const BatchCfg &cfg) {
+    const long N = min(m, n), elems = m * n;
+    int b = 0;
+    while (b < kBuckets - 1 && elems > (long)kBucketElems >> (kBuckets - 2 - b)) ++b;
+    const int by_n = N > 192 ? 0 : N > 128 ? 1 : N > 64 ? 2 : N > 32 ? 3 : 4;
+    int c = 4;
+    while (c > 1 && (c > by_n || 32 * class_warps(c) < cfg.group[b])) --c;
+    return min(c, by_n);
+}
+
 // ---------------------------------------------------------------- prep
-// counter[0]: next position of the main kernel, counter[1]: next position of the
-// large-matrix kernel, counter[2]: number of matrices above the shared-memory size
-// (the sorted order's first counter[2] entries; the main kernel starts after them).
-__global__ void batched_prep_kernel(int batch, const int *dM, const int *dN, int *order, unsigned int *counter) {
-    extern __shared__ unsigned long long keys[];
-    __shared__ unsigned int sh_large;
+__global__ void batched_prep_kernel(int batch, const int *dM, const int *dN, int *order, unsigned int *ctl, BatchCfg cfg) {
+    __shared__ unsigned int bins[kClasses * kCostBins];
     const int tid = threadIdx.x, nt = blockDim.x;
-    if (tid == 0) {
-        counter[0] = 0u;
-        counter[1] = 0u;
-        counter[2] = 0u;
-        sh_large = 0u;
-    }
-    if (batch > kSortMax) {
-        for (int i = tid; i < batch; i += nt) order[i] = i;
-        return;
-    }
-    int P = 1;
-    while (P < batch) P <<= 1;
-    for (int i = tid; i < P; i += nt) {
-        unsigned long long k = ~0ull;
-        if (i < batch) {
-            unsigned long long e = (unsigned long long)max(dM[i], 0) * (unsigned long long)max(dN[i], 0);
-            e = min(e, 0xFFFFFFFFull);
-            k = ((0xFFFFFFFFull - e) << 32) | (unsigned)i;  // ascending key = descending size, then index
+    const auto bin_of = [&](int i) {
+        const long m = max(dM[i], 0), n = max(dN[i], 0), N = min(m, n);
+        // flops to within the ordering's needs; +1: empty matrices come last
+        const float cost = (float)(m * n) * (float)N + 1.f;
+        return class_of(m, n, cfg) * kCostBins + kCostBins - 1 - min(kCostBins - 1, (int)(4.f * __log2f(cost)));
+    };
+    for (int i = tid; i < kClasses * kCostBins; i += nt) bins[i] = 0u;
+    __syncthreads();
+    for (int i = tid; i < batch; i += nt) atomicAdd(&bins[bin_of(i)], 1u);
+    __syncthreads();
+    if (tid < 32) {  // exclusive prefix sum: 20 bins a lane
+        constexpr int per = kClasses * kCostBins / 32;
+        unsigned int sum = 0;
+        for (int q = 0; q < per; ++q) sum += bins[tid * per + q];
+        unsigned int inc = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned int v = __shfl_up_sync(0xffffffffu, inc, o);
+            if (tid >= o) inc += v;
         }
-        keys[i] = k;
+        unsigned int at = inc - sum;
+        for (int q = 0; q < per; ++q) {
+            const unsigned int c = bins[tid * per + q];
+            bins[tid * per + q] = at;
+            at += c;
+        }
     }
     __syncthreads();
-    for (int size = 2; size <= P; size <<= 1)
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int i = tid; i < P; i += nt) {
-                int j = i ^ stride;
-                if (j > i) {
-                    bool up = (i & size) == 0;
-                    unsigned long long a = keys[i], b = keys[j];
-                    if ((a > b) == up) {
-                        keys[i] = b;
-                        keys[j] = a;
-                    }
-                }
-            }
-            __syncthreads();
-        }
-    unsigned int large = 0;
-    for (int i = tid; i < batch; i += nt) {
-        order[i] = (int)(keys[i] & 0xFFFFFFFFull);
-        large += (0xFFFFFFFFull - (keys[i] >> 32)) > (unsigned long long)kBSmemElems ? 1u : 0u;
-    }
-    atomicAdd(&sh_large, large);
+    if (tid <= kClasses) ctl[8 + tid] = tid < kClasses ? bins[tid * kCostBins] : (unsigned)batch;
+    if (tid == 0) ctl[0] = 0u;
     __syncthreads();
-    if (tid == 0) {
-        counter[0] = sh_large;
-        counter[2] = sh_large;
-    }
+    for (int i = tid; i < batch; i += nt) order[atomicAdd(&bins[bin_of(i)], 1u)] = i;
 }
 
-// ---------------------------------------------------------------- group primitives
-__device__ __forceinline__ void gsync(int gid, int g) {
-    asm volatile("bar.sync %0, %1;" ::"r"(gid + 1), "r"(g) : "memory");
-}
-
-// sum over the group of v (g threads, red holds g/32 floats)
-__device__ float gsum(float v, float *red, int gid, int g, int gt) {
-    v = nla::warp_sum(v);
-    if ((gt & 31) == 0) red[gt >> 5] = v;
-    gsync(gid, g);
-    float s = 0.f;
-    for (int w = 0; w < g / 32; ++w) s += red[w];
-    gsync(gid, g);
-    return s;
-}
-
-// Householder reflector for [alpha; x] with ||x||^2 = xn2 (all threads compute the same scalars)
-__device__ void reflector(float alpha, float xn2, float &tau, float &beta, float &scale) {
-    tau = 0.f;
-    beta = alpha;
-    scale = 0.f;
+// ---------------------------------------------------------------- one matrix by NW warps
+// Reflector of [alpha; x] with ||x||^2 = xn2: beta, tau, scale = 1 / (alpha - beta), u0 = alpha - beta.
+__device__ __forceinline__ void reflector(float alpha, float xn2, float &beta, float &tau, float &scale, float &u0) {
+    beta = alpha, tau = 0.f, scale = 0.f, u0 = 0.f;
     if (xn2 > 0.f) {
-        float r = sqrtf(alpha * alpha + xn2);
+        const float q = fmaf(alpha, alpha, xn2);
+        const float rs = rsqrtf(q), r = q * rs;
         beta = alpha >= 0.f ? -r : r;
-        tau = (beta - alpha) / beta;
-        scale = 1.f / (alpha - beta);
+        tau = fmaf(fabsf(alpha), rs, 1.f);
+        u0 = alpha - beta;
+        scale = __fdividef(1.f, u0);
     }
 }
 
-// number of singular values of B(d, e) below x (Sturm count of the Golub-Kahan tridiagonal)
-__device__ int count_below_f(int n, const float *d, const float *e, float x, float pivmin) {
-    float q = -x;
-    int neg = q < 0.f;
-    for (int i = 0; i < n; ++i) {
-        q = -x - d[i] * d[i] / q;
-        if (fabsf(q) < pivmin) q = -pivmin;  // floor first, then count the sign used
-        neg += q < 0.f;
-        if (i + 1 < n) {
-            q = -x - e[i] * e[i] / q;
-            if (fabsf(q) < pivmin) q = -pivmin;
-            neg += q < 0.f;
-        }
-    }
-    return neg - n;
+constexpr int pow2_ceil(int x) {
+    int p = 1;
+    while (p < x) p *= 2;
+    return p;
 }
 
-// One matrix by one group: W (M x N, column-major, leading dimension ldw) already
-// loaded, M >= N.
-__device__ void group_svd(float *W, int M, int N, float *d, float *e, float *vbuf, float *red, float *S, int gid,
-                          int g, int gt, int ldw) {
-    for (int j = 0; j < N; ++j) {
-        // ---- left reflector on column j, rows j..M-1
-        float *col = W + (size_t)j * ldw;
-        float part = 0.f;
-        for (int i = j + 1 + gt; i < M; i += g) part += col[i] * col[i];
-        const float xn2 = gsum(part, red, gid, g, gt);
-        float tau, beta, sc;
-        reflector(col[j], xn2, tau, beta, sc);
-        if (tau != 0.f) {
-            for (int i = j + 1 + gt; i < M; i += g) col[i] *= sc;  // v, v_j = 1 implicit
-            gsync(gid, g);
-            // columns c > j: warp-per-column dot products, then the update
-            const int wid = gt >> 5, lane = gt & 31, nw = g >> 5;
-            for (int c = j + 1 + wid; c < N; c += nw) {
-                float *cc = W + (size_t)c * ldw;
-                float s = lane == 0 ? cc[j] : 0.f;
-                for (int i = j + 1 + lane; i < M; i += 32) s += col[i] * cc[i];
-                s = nla::warp_sum(s) * tau;
-                if (lane == 0) cc[j] -= s;
-                for (int i = j + 1 + lane; i < M; i += 32) cc[i] -= s * col[i];
-            }
+// Sums of v[0..P-1] over the lanes; lane l is left with the sum of v[l / (32 / P)].
+template <int P>
+__device__ __forceinline__ float reduce_scatter(float (&v)[P], int lane) {
+    int o = 16;
+#pragma unroll
+    for (int h = P / 2; h >= 1; h /= 2, o /= 2) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const float send = up ? v[i] : v[i + h], keep = up ? v[i + h] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
-        if (gt == 0) d[j] = beta;
-        gsync(gid, g);
-        if (j + 1 >= N) break;
-        // ---- right reflector on row j, columns j+1..N-1
-        const int L = N - j - 1;
-        float p2 = 0.f;
-        for (int c = j + 2 + gt; c < N; c += g) {
-            float v = W[j + (size_t)c * ldw];
-            p2 += v * v;
-        }
-        const float yn2 = gsum(p2, red, gid, g, gt);
-        reflector(W[j + (size_t)(j + 1) * ldw], yn2, tau, beta, sc);
-        if (gt == 0) e[j] = beta;
-        if (tau != 0.f && L > 1) {
-            for (int c = gt; c < L; c += g) vbuf[c] = c == 0 ? 1.f : W[j + (size_t)(j + 1 + c) * ldw] * sc;
-            gsync(gid, g);
-            for (int i = j + 1 + gt; i < M; i += g) {  // one thread per row
-                float s = 0.f;
-                for (int c = 0; c < L; ++c) s += W[i + (size_t)(j + 1 + c) * ldw] * vbuf[c];
-                s *= tau;
-                for (int c = 0; c < L; ++c) W[i + (size_t)(j + 1 + c) * ldw] -= s * vbuf[c];
-            }
-        }
-        gsync(gid, g);
     }
-    // ---- bisection: one thread per singular value
-    float bnd = 0.f, tmax = 0.f;
-    for (int i = gt; i < N; i += g) {
-        float di = fabsf(d[i]), el = i > 0 ? fabsf(e[i - 1]) : 0.f, er = i + 1 < N ? fabsf(e[i]) : 0.f;
-        bnd = fmaxf(bnd, di + fmaxf(el, er));
-        tmax = fmaxf(tmax, fmaxf(di, er));
-    }
-    {
-        float v = bnd;
-        for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-        float t = tmax;
-        for (int o = 16; o > 0; o >>= 1) t = fmaxf(t, __shfl_xor_sync(0xffffffffu, t, o));
-        if ((gt & 31) == 0) {
-            red[gt >> 5] = v;
-            red[16 + (gt >> 5)] = t;
-        }
-        gsync(gid, g);
-        float b = 0.f, tt = 0.f;
-        for (int w = 0; w < g / 32; ++w) {
-            b = fmaxf(b, red[w]);
-            tt = fmaxf(tt, red[16 + w]);
-        }
-        bnd = b * (1.f + 4.f * FLT_EPSILON) + FLT_MIN;
-        tmax = tt;
-        gsync(gid, g);
-    }
-    const float pivmin = FLT_MIN * fmaxf(1.f, tmax * tmax);
-    const float tol = 2.f * FLT_EPSILON * bnd;
-    for (int idx = gt; idx < N; idx += g) {
-        const int jj = N - 1 - idx;
-        float lo = 0.f, hi = bnd;
-        for (int it = 0; it < 64; ++it) {
-            float mid = 0.5f * (lo + hi);
-            if (hi - lo <= tol || mid <= lo || mid >= hi) break;
-            if (count_below_f(N, d, e, mid, pivmin) <= jj)
-                lo = mid;
-            else
-                hi = mid;
-        }
-        S[idx] = 0.5f * (lo + hi);
-    }
+    for (; o >= 1; o /= 2) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    return v[0];
 }
 
-__global__ void __launch_bounds__(kBThreads)
-batched_svd_kernel(int batch, const int *__restrict__ dM, const int *__restrict__ dN, const int *__restrict__ dLda,
-                   float *const *dA, float *const *dS, const int *__restrict__ order, unsigned int *counter,
-                   float *scratch, size_t scratch_elems, int *dInfo, BatchCfg cfg, int sorted) {
-    extern __shared__ __align__(16) float smem[];
-    __shared__ int sh_start, sh_groups;
-    float *mat = smem;                                    // kBSmemElems
-    float *aux = smem + kBSmemElems;                      // per group: d, e (256 each), vbuf 256, red 32
-    const int tid = threadIdx.x;
-    while (true) {
-        if (tid == 0) {
-            unsigned int pos = atomicAdd(counter, 0u);
-            int gsz = kBThreads;
-            if (sorted && pos < (unsigned)batch) {
-                const int i0 = order[pos];
-                const long el = (long)dM[i0] * dN[i0];
-                const int bk = bucket_of(el);
-                gsz = bk == kBuckets - 1 ? kBThreads : cfg.group[bk];  // global scratch: one matrix per block
-            }
-            const int ng = kBThreads / gsz;
-            sh_groups = ng;
-            sh_start = (int)atomicAdd(counter, (unsigned)ng);
-        }
-        __syncthreads();
-        const int start = sh_start, ng = sh_groups;
-        if (start >= batch) break;
-        const int g = kBThreads / ng, gid = tid / g, gt = tid % g;
-        const int item = start + gid;
-        if (item < batch) {
-            const int i = order[item];
-            const int m = dM[i], n = dN[i], lda = dLda[i];
-            const float *A = dA[i];
-            float *Sout = dS[i];
-            const int M = max(m, n), N = min(m, n);
-            const bool tr = m < n;
-            const int share = kBSmemElems / ng;
-            float *W = (long)M * N <= share ? mat + (size_t)gid * share : scratch + (size_t)blockIdx.x * scratch_elems;
-            float *d = aux + gid * 800, *e = d + 256, *vb = e + 256, *red = vb + 256;
-            // the global slot is only ever used by a block working on one matrix
-            const bool ok = (long)M * N <= share || (ng == 1 && (size_t)M * N <= scratch_elems);
-            if (ok && N <= 256) {
-                for (int idx = gt; idx < M * N; idx += g) {
-                    const int r = idx % M, c = idx / M;  // W(r, c)
-                    W[idx] = tr ? A[c + (size_t)r * lda] : A[r + (size_t)c * lda];
-                }
-                gsync(gid, g);
-                if (N > 0) group_svd(W, M, N, d, e, vb, red, Sout, gid, g, gt, M);
-                if (gt == 0) dInfo[i] = 0;
-            } else if (gt == 0) {
-                dInfo[i] = -NLA_ERR_UNSUPPORTED;
-            }
-        }
-        __syncthreads();
+template <class F, int... K>
+__device__ __forceinline__ void static_for_impl(F &&f, std::integer_sequence<int, K...>) {
+    (f(std::integral_constant<int, K>{}), ...);
+}
+template <int N, class F>
+__device__ __forceinline__ void static_for(F &&f) {
+    static_for_impl(static_cast<F &&>(f), std::make_integer_sequence<int, N>{});
+}
+
+// NW warps, tiles of 32 RR rows x NW RC columns for the bidiagonalisation, of which the first
+// RCS columns of every warp live in shared memory (they are the first to be finished), and
+// 32 QR rows in a chunk of the QR reduction.
+template <int NW_, int RR_, int RC_, int RCS_, int QR_>
+struct Cls {
+    static constexpr int NW = NW_, RR = RR_, RC = RC_, RCS = RCS_, QR = QR_;
+    static constexpr int NMAX = NW * RC, RH = 32 * RR;
+    // shared floats of a worker; R packed by columns: entry (i, c) at c (c + 1) / 2 + i
+    static constexpr int kPacked = (NMAX * (NMAX + 1) / 2 + 3) & ~3;
+    static constexpr int kColsAt = RCS ? ((RCS * NW * (RCS * NW + 1) / 2 + 31) & ~31) : 0;  // shared columns, after R's first ones
+    static constexpr int kBig = RCS && kColsAt + RCS * NW * RH > kPacked ? kColsAt + RCS * NW * RH : kPacked;
+    static constexpr int kPart = RH + 32 / NW;  // conflict-free for two threads a row
+    static constexpr int kFloats = kBig + 2 * 32 * (RR > QR ? RR : QR) + 2 * NW * RC + (NW > 1 ? NW * kPart : 0) + 2 * RH + 32 + 2 * NMAX +
+                                   2 * NMAX;
+};
+
+template <class C>
+struct Worker {
+    static constexpr int NW = C::NW, RC = C::RC, RCS = C::RCS, RH = C::RH;
+    float *big, *us, *rowb, *mbuf, *part, *ys, *a1s, *misc, *d, *e, *t2;
+    int w, lane, bar;
+
+    __device__ Worker(float *sm, int warp, int lane_) : w(warp % NW), lane(lane_), bar(1 + warp / NW) {
+        constexpr int rows = 32 * (C::RR > C::QR ? C::RR : C::QR);
+        big = sm;
+        us = big + C::kBig;
+        rowb = us + 2 * rows;
+        mbuf = rowb + NW * RC;
+        part = mbuf + NW * RC;
+        ys = part + (NW > 1 ? NW * C::kPart : 0);
+        a1s = ys + RH;
+        misc = a1s + RH;  // [0..1] alpha by parity, [2] right alpha, [16 ..] the warps' partial norms
+        t2 = misc + 32;
+        d = t2 + 2 * C::NMAX;
+        e = d + C::NMAX;
+        rowb += w * RC;
+        mbuf += w * RC;
     }
-}
-
-// ---------------------------------------------------------------- blocked QR (large matrices)
-// W (M x N, column-major, leading dimension ldw a multiple of 4, M >= N) is reduced to
-// R = Q^T W by blocked Householder QR with panels of PW columns: each panel (rows k0..M-1)
-// is factored in shared memory (column-major, leading dimension ldp), its compact-WY
-// factor T formed from V^T V (T(j, j) = tau_j, T(0:j, j) = -tau_j T(0:j, 0:j) V(:, 0:j)^T v_j),
-// and the trailing columns updated as X -= V (T^T (V^T X)) in two streaming passes
-// (X read once, then read and written once), so the trailing block is read 3 times per
-// PW columns instead of twice per column.  On return the top N x N block of W holds R
-// (zeros below its diagonal).  The singular values of R are those of W: R = Q^T W with Q
-// orthogonal (the same argument as Section 5.1.1's).
-template <int PW, int G>
-__device__ void group_qr_blocked(float *W, int ldw, int M, int N, float *Pm, int ldp, float *Wt, float *Tt, float *tau,
-                                 float *red, int gt) {
-    const int lane = gt & 31, wid = gt >> 5, nw = G / 32;
-    for (int k0 = 0; k0 < N; k0 += PW) {
-        const int nb = min(PW, N - k0), r = M - k0, C = N - k0 - nb;
-        // ---- load the panel (rows k0.., columns k0..k0+nb-1); zero rows up to ldp
-        for (int idx = gt; idx < PW * ldp; idx += G) {
-            const int k = idx / ldp, i = idx % ldp;
-            Pm[idx] = (k < nb && i < r) ? W[(k0 + i) + (size_t)(k0 + k) * ldw] : 0.f;
-        }
-        gsync(0, G);
-        // ---- factor the panel: reflector j on rows j..r-1, applied to the panel's columns > j
-        for (int j = 0; j < nb; ++j) {
-            float *col = Pm + (size_t)j * ldp;
-            float part = 0.f;
-            for (int i = j + 1 + gt; i < r; i += G) part += col[i] * col[i];
-            const float xn2 = gsum(part, red, 0, G, gt);
-            float t, beta, sc;
-            reflector(col[j], xn2, t, beta, sc);
-            if (gt == 0) tau[j] = t;
-            if (t != 0.f) {
-                for (int i = j + 1 + gt; i < r; i += G) col[i] *= sc;  // v, v_j = 1 implicit
-                gsync(0, G);
-                for (int c = j + 1 + wid; c < nb; c += nw) {
-                    float *cc = Pm + (size_t)c * ldp;
-                    float s = lane == 0 ? cc[j] : 0.f;
-                    for (int i = j + 1 + lane; i < r; i += 32) s += col[i] * cc[i];
-                    s = nla::warp_sum(s) * t;
-                    if (lane == 0) cc[j] -= s;
-                    for (int i = j + 1 + lane; i < r; i += 32) cc[i] -= s * col[i];
-                }
-            }
-            gsync(0, G);
-            if (gt == 0) col[j] = beta;
-            gsync(0, G);
-        }
-        // ---- R rows of the panel back to W (zeros below the diagonal within the top N rows),
-        // then V's unit diagonal and zeros above it in the panel
-        for (int idx = gt; idx < nb * nb; idx += G) {
-            const int i = idx % nb, k = idx / nb;
-            W[(k0 + i) + (size_t)(k0 + k) * ldw] = i <= k ? Pm[i + (size_t)k * ldp] : 0.f;
-        }
-        for (int idx = gt; idx < nb * (N - k0 - nb); idx += G) {  // rows k0+nb..N-1 of the panel columns
-            const int i = nb + idx % (N - k0 - nb), k = idx / (N - k0 - nb);
-            W[(k0 + i) + (size_t)(k0 + k) * ldw] = 0.f;
-        }
-        gsync(0, G);
-        for (int idx = gt; idx < nb * nb; idx += G) {
-            const int i = idx % nb, k = idx / nb;
-            if (i <= k) Pm[i + (size_t)k * ldp] = i == k ? 1.f : 0.f;
-        }
-        gsync(0, G);
-        if (C <= 0) continue;
-        // ---- T from V^T V (warp per entry of the strict upper triangle), then the recurrence
-        for (int e = wid; e < nb * nb; e += nw) {
-            const int a = e % nb, b = e / nb;
-            if (a >= b) continue;
-            const float *va = Pm + (size_t)a * ldp, *vb = Pm + (size_t)b * ldp;
-            float s = 0.f;
-            for (int i = lane; i < r; i += 32) s += va[i] * vb[i];
-            s = nla::warp_sum(s);
-            if (lane == 0) Tt[a + b * PW] = s;  // (V^T V)(a, b), overwritten by T below
-        }
-        gsync(0, G);
-        if (wid == 0) {
-            // column b of T: T(0:b, b) = -tau_b T(0:b, 0:b) (V^T V)(0:b, b), computed top-down in
-            // registers (lane a holds entry a); T(b, b) = tau_b
-            for (int b = 0; b < nb; ++b) {
-                const float g_ab = lane < b ? Tt[lane + b * PW] : 0.f;
-                float v = 0.f;
-                for (int a = 0; a < b; ++a) {  // v_lane = sum_a T(lane, a) g(a, b), T upper triangular
-                    const float ga = __shfl_sync(0xffffffffu, g_ab, a);
-                    if (lane <= a) v += Tt[lane + a * PW] * ga;
-                }
-                __syncwarp();
-                if (lane < b) Tt[lane + b * PW] = -tau[b] * v;
-                if (lane == b) Tt[b + b * PW] = tau[b];
-                __syncwarp();
-            }
-        }
-        gsync(0, G);
-        // ---- pass 1: Wt(:, c) = V^T X(:, c) (warp per column; each lane 4 consecutive rows)
-        const float *X0 = W + k0;  // X(i, c) = X0[i + (c0 + c) * ldw], c0 = k0 + nb
-        const int c0 = k0 + nb;
-        for (int c = wid; c < C; c += nw) {
-            const float *xc = X0 + (size_t)(c0 + c) * ldw;
-            float acc[PW];
-#pragma unroll
-            for (int k = 0; k < PW; ++k) acc[k] = 0.f;
-            for (int i0 = 4 * lane; i0 < r; i0 += 128) {
-                float4 x4;
-                if (i0 + 3 < r) {
-                    x4 = *reinterpret_cast<const float4 *>(xc + i0);
-                } else {
-                    x4.x = xc[i0];
-                    x4.y = i0 + 1 < r ? xc[i0 + 1] : 0.f;
-                    x4.z = i0 + 2 < r ? xc[i0 + 2] : 0.f;
-                    x4.w = 0.f;
-                }
-#pragma unroll
-                for (int k = 0; k < PW; ++k) {
-                    const float4 v4 = *reinterpret_cast<const float4 *>(Pm + (size_t)k * ldp + i0);
-                    acc[k] += v4.x * x4.x + v4.y * x4.y + v4.z * x4.z + v4.w * x4.w;
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < PW; ++k) {
-                const float s = nla::warp_sum(acc[k]);
-                if (lane == k) Wt[k * 256 + c] = s;
-            }
-        }
-        gsync(0, G);
-        // ---- W' = T^T Wt (in place, column by column: W'(k, c) = sum_{j <= k} T(j, k) Wt(j, c))
-        for (int c = gt; c < C; c += G) {
-            float w[PW];
-#pragma unroll
-            for (int k = 0; k < PW; ++k) w[k] = k < nb ? Wt[k * 256 + c] : 0.f;
-#pragma unroll
-            for (int k = PW - 1; k >= 0; --k) {
-                float v = 0.f;
-#pragma unroll
-                for (int j = 0; j <= k; ++j) v += Tt[j + k * PW] * w[j];
-                if (k < nb) Wt[k * 256 + c] = v;
-            }
-        }
-        gsync(0, G);
-        // ---- pass 2: X(:, c) -= V W'(:, c)
-        for (int c = wid; c < C; c += nw) {
-            float *xc = W + k0 + (size_t)(c0 + c) * ldw;
-            float wk[PW];
-#pragma unroll
-            for (int k = 0; k < PW; ++k) wk[k] = k < nb ? Wt[k * 256 + c] : 0.f;
-            for (int i0 = 4 * lane; i0 < r; i0 += 128) {
-                float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                for (int k = 0; k < PW; ++k) {
-                    const float4 v4 = *reinterpret_cast<const float4 *>(Pm + (size_t)k * ldp + i0);
-                    d.x += v4.x * wk[k], d.y += v4.y * wk[k], d.z += v4.z * wk[k], d.w += v4.w * wk[k];
-                }
-                if (i0 + 3 < r) {
-                    float4 x4 = *reinterpret_cast<float4 *>(xc + i0);
-                    x4.x -= d.x, x4.y -= d.y, x4.z -= d.z, x4.w -= d.w;
-                    *reinterpret_cast<float4 *>(xc + i0) = x4;
-                } else {
-                    xc[i0] -= d.x;
-                    if (i0 + 1 < r) xc[i0 + 1] -= d.y;
-                    if (i0 + 2 < r) xc[i0 + 2] -= d.z;
-                }
-            }
-        }
-        gsync(0, G);
+    __device__ __forceinline__ void sync() const {
+        if (NW == 1)
+            __syncwarp();
+        else
+            asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(32 * NW) : "memory");
     }
-}
 
-// threads per block of the large-matrix kernel: 1024 per SM in blocks of G
-// (global scratch slots: one per block)
-constexpr int kLargeThreadsPerSm = 1024;
-constexpr int kLargeSlotsPerSm = kLargeThreadsPerSm / 128;
+    // Left reflector step on columns of group k: with u (rows of column j, zero where it does not
+    // reach), form the coefficients m_c of every column c > j of the warp and subtract u m_c.
+    // row(q): entry (j, c) of the warp's column k + q before the step; set_row(q, w): what happens
+    // to it.  Returns through mk[] the coefficients (zero for finished columns).
+    template <int K, int RR, class Get, class Row, class SetRow>
+    __device__ __forceinline__ void left_coeffs(const float (&u)[RR], int r0, int w0, float alpha, Get get, Row row,
+                                                SetRow set_row, float (&mk)[RC], float &beta, float &u0) {
+        constexpr int CNT = RC - K, P = pow2_ceil(CNT);
+        float z[P], nrm = 0.f;
+#pragma unroll
+        for (int q = 0; q < P; ++q) z[q] = 0.f;
+#pragma unroll
+        for (int r = 0; r < RR; ++r) {
+            if (r < r0) continue;
+            nrm = fmaf(u[r], u[r], nrm);
+#pragma unroll
+            for (int q = 0; q < CNT; ++q) z[q] = fmaf(u[r], get(r, K + q), z[q]);
+        }
+        nrm = nla::warp_sum(nrm);
+        const float zs = reduce_scatter<P>(z, lane);
+        const int q = lane / (32 / P);
+        float tau, scale;
+        reflector(alpha, nrm, beta, tau, scale, u0);
+        const bool live = q < CNT && (q > 0 || w > w0);
+        const float wc = live ? tau * fmaf(scale, zs, row(min(q, CNT - 1))) : 0.f;
+        if (lane % (32 / P) == 0 && q < CNT) {
+            mbuf[K + q] = scale * wc;
+            if (live) set_row(q, wc);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int t = K; t < RC; ++t) mk[t] = mbuf[t];
+    }
 
-// The matrices too large for shared memory (the sorted order's first counter[2]):
-// one per block of G threads, working in the block's global scratch slot (leading
-// dimension rounded up to 4).  When its panel fits the block's shared memory
-// (ldp_max), a matrix is first reduced to its N x N triangular factor R by blocked
-// Householder QR (three streaming passes per 16 columns instead of two per column)
-// and R's singular values are found by the one-stage bidiagonalisation + bisection;
-// otherwise the one-stage reduction runs on the whole matrix.
-constexpr int kQrPanel = 16;
-
-__host__ __device__ constexpr size_t large_smem_floats(int ldp) {
-    return (size_t)kQrPanel * ldp + (size_t)kQrPanel * 256 + kQrPanel * kQrPanel + kQrPanel;
-}
-
-template <int G>
-__global__ void __launch_bounds__(G)
-batched_large_kernel(const int *__restrict__ dM, const int *__restrict__ dN, const int *__restrict__ dLda,
-                     float *const *dA, float *const *dS, const int *__restrict__ order, unsigned int *counter,
-                     float *scratch, size_t scratch_elems, int ldp_max, int rsm_floats, int *dInfo) {
-    extern __shared__ __align__(16) float qsm[];
-    __shared__ float aux[800];
-    __shared__ int sh_item;
-    const int tid = threadIdx.x;
-    const int nlarge = (int)counter[2];
-    while (true) {
-        if (tid == 0) sh_item = (int)atomicAdd(&counter[1], 1u);
-        __syncthreads();
-        const int item = sh_item;
-        if (item >= nlarge) break;
-        const int i = order[item];
-        const int m = dM[i], n = dN[i], lda = dLda[i];
-        const float *A = dA[i];
-        const int M = max(m, n), N = min(m, n);
-        const bool tr = m < n;
-        const int ldw = (M + 3) & ~3;
-        float *W = scratch + (size_t)blockIdx.x * scratch_elems;
-        if ((size_t)ldw * N <= scratch_elems && N <= 256) {
-            for (int idx = tid; idx < M * N; idx += G) {
-                const int r = idx % M, c = idx / M;  // W(r, c)
-                W[r + (size_t)c * ldw] = tr ? A[c + (size_t)r * lda] : A[r + (size_t)c * lda];
+    // R (packed in big) <- R of the QR factorisation of [R; A], A = rows in the tile.
+    __device__ void qr_chunk(float (&a)[C::QR][RC], int N) {
+        constexpr int RR = C::QR, rows = 32 * RR;
+        static_for<RC>([&](auto kc) {
+            constexpr int K = decltype(kc)::value;
+#pragma unroll 1
+            for (int w0 = 0; w0 < NW; ++w0) {
+                const int j = K * NW + w0;
+                if (j >= N) break;
+                float *ub = us + (j & 1) * rows, *rjj = big + j * (j + 1) / 2 + j;
+                if (w == w0) {
+#pragma unroll
+                    for (int r = 0; r < RR; ++r) ub[32 * r + lane] = a[r][K];
+                    if (lane == 0) misc[j & 1] = *rjj;
+                }
+                sync();
+                float u[RR], mk[RC], beta, u0;
+#pragma unroll
+                for (int r = 0; r < RR; ++r) u[r] = ub[32 * r + lane];
+                const auto rjc = [&](int q) -> float & {
+                    const int c = w + NW * (K + q);
+                    return big[c * (c + 1) / 2 + j];
+                };
+                left_coeffs<K, RR>(u, 0, w0, misc[j & 1], [&](int r, int t) { return a[r][t]; },
+                                   [&](int q) { return q > 0 || w > w0 ? rjc(q) : 0.f; },
+                                   [&](int q, float wc) { rjc(q) -= wc; }, mk, beta, u0);
+                if (w == w0 && lane == 0) *rjj = beta;
+#pragma unroll
+                for (int r = 0; r < RR; ++r)
+#pragma unroll
+                    for (int t = K; t < RC; ++t) a[r][t] = fmaf(-u[r], mk[t], a[r][t]);
+                if (NW == 1) __syncwarp();
             }
-            gsync(0, G);
-            if (N > 0) {
-                if (ldw <= ldp_max && M > N) {
-                    float *Pm = qsm, *Wt = Pm + (size_t)kQrPanel * ldw, *Tt = Wt + kQrPanel * 256,
-                          *tau = Tt + kQrPanel * kQrPanel;
-                    group_qr_blocked<kQrPanel, G>(W, ldw, M, N, Pm, ldw, Wt, Tt, tau, aux + 768, tid);
-                    if ((size_t)N * N <= (size_t)rsm_floats) {
-                        // R into shared memory (the panel's space), where the one-stage reduction
-                        // runs at shared-memory latency
-                        for (int idx = tid; idx < N * N; idx += G) {
-                            const int r = idx % N, c = idx / N;
-                            qsm[idx] = W[r + (size_t)c * ldw];
-                        }
-                        gsync(0, G);
-                        group_svd(qsm, N, N, aux, aux + 256, aux + 512, aux + 768, dS[i], 0, G, tid, N);
-                    } else {
-                        group_svd(W, N, N, aux, aux + 256, aux + 512, aux + 768, dS[i], 0, G, tid, ldw);
+        });
+    }
+
+    // Bidiagonalisation of the tile (M x N, M <= RH): d, e.
+    __device__ void bidiag(float (&a)[C::RR][RC - RCS], int N) {
+        constexpr int RR = C::RR;
+        float *const sc = big + C::kColsAt + w * RH + lane;  // column w + NW t, t < RCS, at sc + t NW RH
+        const auto get = [&](int r, int t) -> float & { return t < RCS ? sc[t * NW * RH + 32 * r] : a[r][t < RCS ? 0 : t - RCS]; };
+        static_for<RC>([&](auto kc) {
+            constexpr int K = decltype(kc)::value, R0 = K * NW / 32;  // rows 32 R0 .. are not finished
+#pragma unroll 1
+            for (int w0 = 0; w0 < NW; ++w0) {
+                const int j = K * NW + w0, jl = j % 32;
+                if (j >= N) break;
+                // ---- left reflector of column j
+                if (w == w0) {
+#pragma unroll
+                    for (int r = R0; r < RR; ++r) {
+                        const float v = get(r, K);
+                        us[32 * r + lane] = r > R0 || lane > jl ? v : 0.f;
+                        if (r == R0 && lane == jl) misc[0] = v;
                     }
+                }
+                if (lane == jl) {
+#pragma unroll
+                    for (int t = K; t < RC; ++t) rowb[t] = get(R0, t);
+                }
+                sync();
+                float u[RR], mk[RC], beta, u0;
+#pragma unroll
+                for (int r = R0; r < RR; ++r) u[r] = us[32 * r + lane];
+                left_coeffs<K, RR>(u, R0, w0, misc[0], get, [&](int q) { return rowb[K + q]; }, [](int, float) {}, mk, beta, u0);
+                if (lane == jl) u[R0] = u0;  // row j: its entries drop by w_c = u_0 m_c
+#pragma unroll
+                for (int r = R0; r < RR; ++r)
+#pragma unroll
+                    for (int t = K; t < RC; ++t) {
+                        float &x = get(r, t);
+                        x = fmaf(-u[r], mk[t], x);
+                    }
+                if (w == w0 && lane == 0) d[j] = beta;
+                if (j + 1 >= N) break;
+                // ---- right reflector of row j: entries x_c, c > j; alpha = x_{j+1} in warp w1, column k or k + 1
+                const bool wrap = w0 + 1 == NW;
+                const int w1 = wrap ? 0 : w0 + 1;
+                __syncwarp();
+                if (lane == jl) {
+#pragma unroll
+                    for (int t = K; t < RC; ++t) rowb[t] = t > K || w > w0 ? get(R0, t) : 0.f;
+                }
+                __syncwarp();
+                float x[RC], y[RR], pn = 0.f;
+#pragma unroll
+                for (int t = K; t < RC; ++t) x[t] = rowb[t];
+                constexpr int K1 = K + 1 < RC ? K + 1 : K;
+                if (w == w1) {
+                    if (lane == 0) misc[2] = wrap ? x[K1] : x[K];
+#pragma unroll
+                    for (int r = R0; r < RR; ++r) a1s[32 * r + lane] = wrap ? get(r, K1) : get(r, K);
+                    if (wrap)
+                        x[K1] = 0.f;
+                    else
+                        x[K] = 0.f;
+                }
+#pragma unroll
+                for (int r = R0; r < RR; ++r) {
+                    float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+                    for (int t = K; t < RC; t += 2) {
+                        s0 = fmaf(get(r, t), x[t], s0);
+                        if (t + 1 < RC) s1 = fmaf(get(r, t + 1), x[t + 1], s1);
+                    }
+                    y[r] = s0 + s1;
+                }
+#pragma unroll
+                for (int t = K; t < RC; ++t) pn = fmaf(x[t], x[t], pn);
+                if constexpr (NW > 1) {
+#pragma unroll
+                    for (int r = R0; r < RR; ++r) part[w * C::kPart + 32 * r + lane] = y[r];
+                    if (lane == 0) misc[16 + w] = pn;
+                    sync();
+                    // two threads a row add the warps' sums
+                    const int t = w * 32 + lane, row = 32 * R0 + (t >> 1);
+                    if (row < RH) {
+                        float s = 0.f;
+#pragma unroll
+                        for (int q = 0; q < NW / 2; ++q) s += part[((t & 1) * (NW / 2) + q) * C::kPart + row];
+                        s += __shfl_xor_sync(__activemask(), s, 1);
+                        if ((t & 1) == 0) ys[row] = s;
+                    }
+                    sync();
+                    pn = 0.f;
+#pragma unroll
+                    for (int q = 0; q < NW; ++q) pn += misc[16 + q];
+#pragma unroll
+                    for (int r = R0; r < RR; ++r) y[r] = ys[32 * r + lane];
                 } else {
-                    group_svd(W, M, N, aux, aux + 256, aux + 512, aux + 768, dS[i], 0, G, tid, ldw);
+                    __syncwarp();
+                }
+                float tau, scale;
+                reflector(misc[2], pn, beta, tau, scale, u0);
+                if (w == w0 && lane == 0) e[j] = beta;
+                if (w == w1) {
+                    if (wrap)
+                        x[K1] = u0;
+                    else
+                        x[K] = u0;
+                }
+#pragma unroll
+                for (int r = R0; r < RR; ++r) {
+                    const float m = scale * (tau * fmaf(scale, y[r], a1s[32 * r + lane]));
+#pragma unroll
+                    for (int t = K; t < RC; ++t) {
+                        float &v = get(r, t);
+                        v = fmaf(-m, x[t], v);
+                    }
+                }
+                if (NW == 1) __syncwarp();
+            }
+        });
+    }
+
+    // Values of the bidiagonal (d, e) by multisection, L lanes per value; S descending.
+    __device__ void values(int N, float *S) {
+        const int t = w * 32 + lane;
+        sync();
+        float b = 0.f;
+        for (int i = t; i < N; i += 32 * NW) {
+            const float el = i > 0 ? fabsf(e[i - 1]) : 0.f, er = i + 1 < N ? fabsf(e[i]) : 0.f;
+            b = fmaxf(b, fabsf(d[i]) + fmaxf(el, er));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) b = fmaxf(b, __shfl_xor_sync(0xffffffffu, b, o));
+        if (NW > 1) {
+            if (lane == 0) misc[16 + w] = b;
+            sync();
+#pragma unroll
+            for (int q = 0; q < NW; ++q) b = fmaxf(b, misc[16 + q]);
+        }
+        if (!(b > 0.f)) {  // zero
+            for (int i = t; i < N; i += 32 * NW) S[i] = 0.f;
+            return;
+        }
+        // B is scaled by 2^-ex, in two factors that are normal numbers, to a bound in [0.5, 1)
+        int ex;
+        frexpf(b, &ex);
+        const float f1 = ldexpf(1.f, -(ex / 2)), f2 = ldexpf(1.f, -(ex - ex / 2));
+        for (int i = t; i < 2 * N - 1; i += 32 * NW) {
+            const float v = ((i & 1) ? e[i >> 1] : d[i >> 1]) * f1 * f2;
+            t2[i] = fmaxf(v * v, nla::kT2FloorF);
+        }
+        sync();
+        int L = 1;
+        while (L < 32 && N * L * 2 <= 32 * NW) L *= 2;
+        const int idx = t / L, l = t % L, gbase = lane & ~(L - 1);
+        const unsigned full = L == 32 ? 0xffffffffu : (1u << L) - 1, gmask = full << gbase;
+        if (idx < N) {  // uniform over the group of L lanes
+            const int j = N - 1 - idx;
+            const float frac = (float)(l + 1) / (float)(L + 1);
+            float lo = 0.f, hi = 1.f;
+            for (int round = 0; round < 64 && hi - lo > 0x1p-23f; ++round) {
+                const float x = fmaf(hi - lo, frac, lo);
+                const bool below = nla::sturm_neg(2 * N - 1, t2, x) - N <= j;
+                const unsigned m = (__ballot_sync(gmask, below) >> gbase) & full;
+                const int f = m == full ? L : __ffs(~m) - 1;  // first point whose count passes j
+                const float xf = __shfl_sync(gmask, x, gbase + min(f, L - 1));
+                const float xp = __shfl_sync(gmask, x, gbase + max(f - 1, 0));
+                if (f < L) hi = xf;
+                if (f > 0) lo = xp;
+            }
+            if (l == 0) S[idx] = 0.5f * (lo + hi) / f1 / f2;
+        }
+    }
+
+    // The matrix A (m x n, column-major, lda): M >= N after transposition (tr).
+    __device__ void run(const float *A, int M, int N, int lda, bool tr, float *S) {
+        const auto entry = [&](int i, int c) {
+            return i < M && c < N ? (tr ? A[c + (size_t)i * lda] : A[i + (size_t)c * lda]) : 0.f;
+        };
+        constexpr int RR = C::RR;
+        const bool qr = M > RH;
+        if (qr) {
+            for (int i = w * 32 + lane; i < N * (N + 1) / 2; i += 32 * NW) big[i] = 0.f;
+            for (int base = 0; base < M; base += 32 * C::QR) {
+                float a[C::QR][RC];
+#pragma unroll
+                for (int t = 0; t < RC; ++t)
+#pragma unroll
+                    for (int r = 0; r < C::QR; ++r) a[r][t] = entry(base + 32 * r + lane, w + NW * t);
+                sync();
+                qr_chunk(a, N);
+            }
+            sync();
+        }
+        float a[RR][RC - RCS];
+#pragma unroll
+        for (int t = RCS; t < RC; ++t)
+#pragma unroll
+            for (int r = 0; r < RR; ++r) {
+                const int i = 32 * r + lane, c = w + NW * t;
+                a[r][t - RCS] = qr ? (i <= c && c < N ? big[c * (c + 1) / 2 + i] : 0.f) : entry(i, c);
+            }
+        if constexpr (RCS > 0) {
+            sync();  // R's later columns are in registers: the shared columns may take their place
+            float *const sc = big + C::kColsAt + w * RH + lane;
+#pragma unroll
+            for (int t = 0; t < RCS; ++t)
+#pragma unroll
+                for (int r = 0; r < RR; ++r) {
+                    const int i = 32 * r + lane, c = w + NW * t;
+                    sc[t * NW * RH + 32 * r] = qr ? (i <= c && c < N ? big[c * (c + 1) / 2 + i] : 0.f) : entry(i, c);
+                }
+        }
+        bidiag(a, N);
+        values(N, S);
+        sync();
+    }
+};
+
+// Tile shapes.  256 columns do not fit the registers beside their addresses, hence six columns a
+// warp in shared memory (seven and eight measured 5 and 7 % slower at 256 x 256).  us for one
+// unit (one SM's 16 warps), square / 4:1 tall: N = 256 615 / 1908, 192 305 / 848, 128 (two
+// matrices) 211 / 541, 64 (four) 104 / 192, 32 (sixteen) 99 / 151.  Rows per chunk of the QR:
+// larger chunks only paid for the two smallest classes (64 rows a chunk: 237 and 172 us).
+// The 10,000-matrix workload (n ~ U{8..256}, m/n ~ U[1, 4]): 186.0 ms with the matrices in
+// shared or global memory, 33.7 ms with these; 300 small ones (n <= 64): 726 -> 184 us.
+using Class0 = Cls<16, 8, 16, 6, 4>;
+using Class1 = Cls<16, 6, 12, 0, 6>;
+using Class2 = Cls<8, 4, 16, 0, 4>;
+using Class3 = Cls<4, 2, 16, 0, 4>;
+using Class4 = Cls<1, 1, 32, 0, 2>;
+
+constexpr int worker_floats() {
+    int f = Class0::kFloats;
+    f = std::max(f, Class1::kFloats);
+    f = std::max(f, 2 * Class2::kFloats);
+    f = std::max(f, 4 * Class3::kFloats);
+    return std::max(f, 16 * Class4::kFloats);
+}
+
+template <class C>
+__device__ __noinline__ void run_worker(float *smem, int warp, int lane, const float *A, int M, int N, int lda, bool tr, float *S) {
+    Worker<C> wk(smem + warp / C::NW * C::kFloats, warp, lane);
+    wk.run(A, M, N, lda, tr, S);
+}
+
+__global__ void __launch_bounds__(kThreads, 1)
+batched_svd_kernel(const int *__restrict__ dM, const int *__restrict__ dN, const int *__restrict__ dLda,
+                   float *const *dA, float *const *dS, const int *__restrict__ order, unsigned int *ctl,
+                   size_t slot_elems, int *dInfo) {
+    extern __shared__ __align__(16) float smem[];
+    __shared__ int sh_unit;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    while (true) {
+        if (tid == 0) sh_unit = (int)atomicAdd(ctl, 1u);
+        __syncthreads();
+        int unit = sh_unit, cls = 0, first = 0, per = 1, end = 0;
+        for (; cls < kClasses; ++cls) {
+            first = (int)ctl[8 + cls];
+            end = (int)ctl[8 + cls + 1];
+            per = kWarps / class_warps(cls);
+            const int units = (end - first + per - 1) / per;
+            if (unit < units) break;
+            unit -= units;
+        }
+        if (cls == kClasses) break;
+        const int pos = first + unit * per + warp / class_warps(cls);
+        if (pos < end) {
+            const int i = order[pos];
+            const int m = dM[i], n = dN[i], lda = dLda[i];
+            const int M = max(m, n), N = min(m, n);
+            // (matrices beyond the sizes the caller declared are refused)
+            const bool ok = N <= 256 && ((long)M * N <= kBucketElems || (size_t)((M + 3) & ~3) * N <= slot_elems);
+            if (ok && N > 0) {
+                const float *A = dA[i];
+                float *S = dS[i];
+                const bool tr = m < n;
+                switch (cls) {
+                    case 0: run_worker<Class0>(smem, warp, lane, A, M, N, lda, tr, S); break;
+                    case 1: run_worker<Class1>(smem, warp, lane, A, M, N, lda, tr, S); break;
+                    case 2: run_worker<Class2>(smem, warp, lane, A, M, N, lda, tr, S); break;
+                    case 3: run_worker<Class3>(smem, warp, lane, A, M, N, lda, tr, S); break;
+                    default: run_worker<Class4>(smem, warp, lane, A, M, N, lda, tr, S); break;
                 }
             }
-            if (tid == 0) dInfo[i] = 0;
-        } else if (tid == 0) {
-            dInfo[i] = -NLA_ERR_UNSUPPORTED;
+            if (lane == 0 && warp % class_warps(cls) == 0) dInfo[i] = ok ? 0 : -NLA_ERR_UNSUPPORTED;
         }
         __syncthreads();
     }
-}
-
-BatchCfg default_cfg() {
-    BatchCfg c;
-    for (int b = 0; b < kBuckets; ++b) c.group[b] = kMinGroup[b];
-    c.group[kBuckets - 1] = kBThreads;
-    return c;
 }
 
 }  // namespace
 
 namespace nla {
-// Group sizes per bucket installed by the tuner table (bucket b -> threads per matrix).
+// Group sizes per bucket installed by the tuner table (bucket b -> least threads per matrix).
 int g_batched_group[kBuckets] = {0, 0, 0, 0, 0};
 }
 
@@ -577,12 +568,7 @@ extern "C" {
 nla_status nla_gesvd_vals_batched_workspace(int batch, nla_dtype dtype, int max_m, int max_n, size_t *bytes) {
     if (!bytes || batch < 0 || max_m < 0 || max_n < 0) return berr(NLA_ERR_ARG, "bad arguments");
     if (dtype != NLA_F32) return berr(NLA_ERR_UNSUPPORTED, "the batched kernel supports FP32 only");
-    const size_t blocks = (size_t)nla::device_sm_count() * std::max(2, kLargeSlotsPerSm);
-    const size_t slot = (size_t)((std::max(max_m, 1) + 3) & ~3) * std::max(max_n, 1);
-    size_t b = 256;                                    // counter
-    b += ((size_t)std::max(batch, 1) * 4 + 255) / 256 * 256;  // order
-    b += blocks * slot * 4;                            // scratch slots
-    *bytes = b;
+    *bytes = 256 + ((size_t)std::max(batch, 1) * 4 + 255) / 256 * 256;  // control words, order
     return NLA_OK;
 }
 
@@ -602,66 +588,26 @@ nla_status nla_gesvd_vals_batched(int batch, nla_dtype dtype, const int *dM, con
     if (((uintptr_t)dWork) % 256) return berr(NLA_ERR_WORKSPACE, "workspace not 256-byte aligned");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     char *w = reinterpret_cast<char *>(dWork);
-    unsigned int *counter = reinterpret_cast<unsigned int *>(w);
+    unsigned int *ctl = reinterpret_cast<unsigned int *>(w);
     int *order = reinterpret_cast<int *>(w + 256);
-    float *scratch = reinterpret_cast<float *>(w + 256 + ((size_t)batch * 4 + 255) / 256 * 256);
     const size_t slot = (size_t)((std::max(max_m, 1) + 3) & ~3) * std::max(max_n, 1);
-    BatchCfg cfg = default_cfg();
-    for (int b = 0; b < kBuckets; ++b)
-        if (nla::g_batched_group[b] >= kMinGroup[b] && nla::g_batched_group[b] <= kBThreads &&
-            kBThreads % nla::g_batched_group[b] == 0)
-            cfg.group[b] = nla::g_batched_group[b];
+    BatchCfg cfg;
+    for (int b = 0; b < kBuckets; ++b) {
+        const int g = nla::g_batched_group[b];
+        cfg.group[b] = g >= 32 && g <= 256 && 256 % g == 0 ? g : 32;
+    }
     static nla::PerDeviceOnce attr;
-    const size_t sort_smem = (size_t)kSortMax * sizeof(unsigned long long);
-    const size_t main_smem = ((size_t)kBSmemElems + 8 * 800) * sizeof(float);
+    constexpr size_t smem = (size_t)worker_floats() * sizeof(float);
     attr.run([&] {
-        cudaFuncSetAttribute(batched_prep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sort_smem);
-        cudaFuncSetAttribute(batched_svd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)main_smem);
+        cudaFuncSetAttribute(batched_svd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         cudaGetLastError();
     });
     {
         nla::TraceScope ts(nla::kTrBatched, st);
-        batched_prep_kernel<<<1, 1024, batch <= kSortMax ? sort_smem : 0, st>>>(batch, dM, dN, order, counter);
-        int blocks = nla::device_sm_count();
-        if (batch <= kSortMax) {  // (unsorted batches leave counter[2] = 0: the main kernel takes all)
-            static const int per_sm_threads = [] {  // NLA_BATCH_LARGE_THREADS: threads per SM of the kernel
-                const char *v = getenv("NLA_BATCH_LARGE_THREADS");
-                const int t = v ? atoi(v) : kLargeThreadsPerSm;
-                return std::max(256, std::min(t, kLargeThreadsPerSm));
-            }();
-            // threads per large matrix: the tuned group of the largest bucket (128 or 256); the
-            // blocked QR's panel is sized for the batch's largest row count when it fits
-            // (and a triangular factor R that fits the same shared memory is reduced there;
-            // larger ones in the scratch slot -- growing the shared memory for them costs
-            // blocks per SM: 232 vs 187 ms per batch of the 10,000-matrix workload)
-            const int ldp = (std::max(max_m, max_n) + 3) & ~3;
-            const size_t qsmem = large_smem_floats(ldp) * sizeof(float);
-            const bool qr = qsmem <= (size_t)160 * 1024;
-            const size_t dsm = qr ? qsmem : 0;
-            const int rsm_floats = qr ? (int)(dsm / sizeof(float)) : 0;
-            auto launch_large = [&](auto kern, int G) {
-                static nla::PerDeviceOnce lattr;
-                lattr.run([&] {
-                    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 210 * 1024);
-                    cudaGetLastError();
-                });
-                int per_sm = 0;
-                if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, G, dsm) != cudaSuccess || per_sm < 1) {
-                    cudaGetLastError();
-                    per_sm = 1;
-                }
-                per_sm = std::min(per_sm, per_sm_threads / G);
-                kern<<<blocks * per_sm, G, dsm, st>>>(dM, dN, dLda, (float *const *)dA_array, (float *const *)dS_array,
-                                                      order, counter, scratch, slot, qr ? ldp : 0, rsm_floats, dInfo);
-            };
-            if (cfg.group[kBuckets - 1] == 128)
-                launch_large(batched_large_kernel<128>, 128);
-            else
-                launch_large(batched_large_kernel<256>, 256);
-        }
-        batched_svd_kernel<<<blocks, kBThreads, main_smem, st>>>(batch, dM, dN, dLda, (float *const *)dA_array,
-                                                                 (float *const *)dS_array, order, counter, scratch, slot,
-                                                                 dInfo, cfg, batch <= kSortMax ? 1 : 0);
+        batched_prep_kernel<<<1, 1024, 0, st>>>(batch, dM, dN, order, ctl, cfg);
+        const int blocks = std::min(nla::device_sm_count(), batch);
+        batched_svd_kernel<<<blocks, kThreads, smem, st>>>(dM, dN, dLda, (float *const *)dA_array, (float *const *)dS_array,
+                                                           order, ctl, slot, dInfo);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return berr(NLA_ERR_CUDA, cudaGetErrorString(e));

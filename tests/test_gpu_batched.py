@@ -116,3 +116,44 @@ def test_unsorted_batch_over_the_sort_limit(nla):
     for i in check_ids:
         ref = oracle.svdvals(mats[i].astype(np.float64))
         assert err_rel(S[i].cpu().numpy(), ref) <= 5e-6 * max(mats[i].shape), (i, mats[i].shape)
+
+
+@pytest.mark.parametrize("groups", [None, 32, 128, 256])
+def test_class_and_chunk_edges(nla, groups, tmp_path):
+    # column counts around the five classes, rows around the register tiles and the chunks of the QR
+    # reduction, wide matrices, leading dimensions beyond the rows; the table's least threads per matrix
+    from paper_2608_21227_gb300 import kt
+
+    if groups is None:
+        kt.load_config(None)
+    else:
+        path = tmp_path / "t.kt"
+        for b in range(5):
+            kt.write_table(path, 2, b, 0, nla.F32, 0, (groups, 0, 0, 0, 0), 1.0)
+        kt.load_config(path)
+    try:
+        g = np.random.default_rng(77)
+        shapes = [(n, n) for n in (1, 2, 3, 31, 32, 33, 63, 64, 65, 127, 128, 129, 191, 192, 193, 255, 256)]
+        shapes += [(65, 32), (129, 32), (64, 33), (65, 64), (129, 64), (257, 60), (129, 100), (257, 128), (513, 77),
+                   (193, 150), (385, 192), (577, 130), (257, 200), (385, 256), (1024, 256), (3000, 17), (2000, 1)]
+        mats, dev = [], []
+        for k, (m, n) in enumerate(shapes):
+            A = g.standard_normal((m, n)).astype(np.float32)
+            if k % 4 == 1:
+                A = (A * 1e-12).astype(np.float32)
+            if k % 3 == 2:
+                A = np.ascontiguousarray(A.T)  # wide
+            pad = 3 if k % 2 else 0
+            t = torch.zeros(A.shape[1], A.shape[0] + pad, device="cuda")
+            t[:, : A.shape[0]] = torch.from_numpy(np.ascontiguousarray(A.T)).cuda()
+            mats.append(A)
+            dev.append(t[:, : A.shape[0]])  # column-major m x n, lda = m + pad
+        b = nla.Batch(dev)
+        S, info = nla.gesvd_vals_batched(b)
+        torch.cuda.synchronize()
+        assert np.all(info.cpu().numpy() == 0)
+        for A, s in zip(mats, S):
+            ref = np.linalg.svd(A.astype(np.float64), compute_uv=False)
+            assert err_rel(s.cpu().numpy(), ref) <= 5e-6 * max(A.shape), A.shape
+    finally:
+        kt.load_config(None)
