@@ -34,6 +34,7 @@
 
 #include "../../include/nla.h"
 #include "common.cuh"
+#include "house.cuh"
 #include "kernels.cuh"
 #include "sturm.cuh"
 #include "trace.h"
@@ -112,12 +113,12 @@ __global__ void batched_prep_kernel(int batch, const int *dM, const int *dN, int
 __device__ __forceinline__ void reflector(float alpha, float xn2, float &beta, float &tau, float &scale, float &u0) {
     beta = alpha, tau = 0.f, scale = 0.f, u0 = 0.f;
     if (xn2 > 0.f) {
-        const float q = fmaf(alpha, alpha, xn2);
-        const float rs = rsqrtf(q), r = q * rs;
+        float r, rs;
+        nla::sqrt_and_inverse(fmaf(alpha, alpha, xn2), r, rs);
         beta = alpha >= 0.f ? -r : r;
         tau = fmaf(fabsf(alpha), rs, 1.f);
         u0 = alpha - beta;
-        scale = __fdividef(1.f, u0);
+        scale = nla::inverse(u0);
     }
 }
 

@@ -576,11 +576,11 @@ constexpr int kRegWarps = 15;  // row warps per block at most (with the extra on
 
 // beta, tau and the scale 1 / (alpha - beta) of the reflector of [alpha; x], xn2 = ||x||^2 > 0.
 NLA_DEV void panel_scalars(float alpha, float xn2, float &beta, float &tau, float &scale) {
-    const float q = fmaf(alpha, alpha, xn2);
-    const float rs = rsqrtf(q), r = q * rs;
+    float r, rs;
+    sqrt_and_inverse(fmaf(alpha, alpha, xn2), r, rs);
     beta = alpha >= 0.f ? -r : r;
     tau = fmaf(fabsf(alpha), rs, 1.f);
-    scale = __fdividef(1.f, alpha - beta);
+    scale = inverse(alpha - beta);
 }
 NLA_DEV void panel_scalars(double alpha, double xn2, double &beta, double &tau, double &scale) {
     double u0, g, one;
