@@ -291,13 +291,16 @@ qr_proj_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
 // ------------------------------------------------------------------ qr_proj on the tensor cores
 // W^T (128 strip columns x NB) = X_strip^T V accumulated in TMEM by tcgen05.mma
 // (kind::tf32, M = 128, K = 8 per instruction) over 32-row stages of X.
-// FP32 accuracy from TF32 operands by the three-term split x = hi + lo,
-// hi = x with the low 13 mantissa bits cleared (what the tensor core reads of an
-// FP32 word), lo = x - hi (exact): x . v ~ hi_x hi_v + hi_x lo_v + lo_x hi_v, the
-// dropped lo_x lo_v term and the truncation of lo are below 2^-21 relative.  The
+// FP32 accuracy from TF32 operands by the three-term split x = hi + lo: of X, hi = x with the
+// low 13 mantissa bits cleared (what the tensor core reads of an FP32 word); of V, hi is x
+// rounded to TF32, so that the dropped lo_x lo_v has no preferred sign; lo = x - hi (exact)
+// rounded to TF32: x . v ~ hi_x hi_v + hi_x lo_v + lo_x hi_v to 2^-22 relative.  The
 // first two products are one MMA against [V_hi; V_lo] (N = 2 NB, the hi copy of X
-// read once), the third a second MMA (N = NB) into its own accumulator; the
-// epilogue adds the three parts.
+// read once), the third a second MMA (N = NB) onto the columns of the other small product.
+// The tensor core rounds its accumulator toward zero, which shrinks W in proportion to the
+// number of MMAs summed one after another and with it, over the steps, every singular value
+// (-2.7e-8 of sigma_1 per MMA in the chain, 3.5e-6 at 8,192 rows).  So the K steps take turns on
+// as many accumulators as two blocks' TMEM holds, and the epilogue adds them in FP32.
 // Roles: warp 0 issues the TMA loads of X and V (128-byte-swizzled boxes, which
 // are the canonical K-major operand layout); warps 2..5 write the lo copies and
 // mask V's unit diagonal; warp 1 owns TMEM and one lane issues the MMAs, each
@@ -306,6 +309,9 @@ qr_proj_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
 constexpr int kTcWarps = 6;
 
 NLA_DEV float tf32_hi(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
+NLA_DEV float tf32_rn(float x) { return __uint_as_float(tc::to_tf32(x)); }
+// x - hi for the tensor core, which drops the low 13 bits: half a TF32 unit first makes that a rounding
+NLA_DEV float tf32_lo(float x, float hi) { return __uint_as_float(__float_as_uint(x - hi) + 0x1000u); }
 
 template <int NB>
 __global__ void __launch_bounds__(32 * kTcWarps, 1)
@@ -314,8 +320,8 @@ qr_proj_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
                   int *info) {
     pdl_wait();
     pdl_trigger();
-    // TMEM: D1 = hi x [V_hi | V_lo] (2 NB columns), D2 = lo x V_hi (NB columns)
-    constexpr uint32_t kCols = 3 * NB <= 32 ? 32 : 3 * NB <= 64 ? 64 : 3 * NB <= 128 ? 128 : 256;
+    // TMEM: kSets accumulators of 2 NB columns: hi x V_hi | hi x V_lo + lo x V_hi
+    constexpr uint32_t kCols = 256, kSets = kCols / (2 * NB);
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full[kMaxStages], conv[kMaxStages], empty[kMaxStages], accdone;
     __shared__ uint32_t tmem_base;
@@ -386,9 +392,9 @@ qr_proj_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
                 const uint32_t bh = tc::smem_u32(vhi(st));
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {  // 8 TF32 = 32 bytes of K per instruction
-                    const uint32_t off = kk * 32, acc = (t > 0 || kk > 0) ? 1u : 0u;
-                    tc::mma_tf32(tbase, tc::sdesc_sw128(ah + off), tc::sdesc_sw128(bh + off), id2, acc);
-                    tc::mma_tf32(tbase + 2 * NB, tc::sdesc_sw128(al + off), tc::sdesc_sw128(bh + off), id1, acc);
+                    const uint32_t off = kk * 32, step = 4 * t + kk, d = tbase + step % kSets * 2 * NB;
+                    tc::mma_tf32(d, tc::sdesc_sw128(ah + off), tc::sdesc_sw128(bh + off), id2, step >= kSets ? 1u : 0u);
+                    tc::mma_tf32(d + NB, tc::sdesc_sw128(al + off), tc::sdesc_sw128(bh + off), id1, 1u);
                 }
                 tc::mma_commit(&empty[st]);  // the stage is free once these MMAs have read it
             }
@@ -420,13 +426,15 @@ qr_proj_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
 #pragma unroll 4
             for (int e = ct; e < xbytes / 16; e += 128) {
                 const float4 v = xs[e];
-                xl[e] = make_float4(v.x - tf32_hi(v.x), v.y - tf32_hi(v.y), v.z - tf32_hi(v.z), v.w - tf32_hi(v.w));
+                xl[e] = make_float4(tf32_lo(v.x, tf32_hi(v.x)), tf32_lo(v.y, tf32_hi(v.y)), tf32_lo(v.z, tf32_hi(v.z)),
+                                    tf32_lo(v.w, tf32_hi(v.w)));
             }
-            const float4 *vs = reinterpret_cast<const float4 *>(vh);
+            float4 *vs = reinterpret_cast<float4 *>(vh);
             float4 *vl = reinterpret_cast<float4 *>(vlo(st));
             for (int e = ct; e < vbytes / 16; e += 128) {
-                const float4 v = vs[e];
-                vl[e] = make_float4(v.x - tf32_hi(v.x), v.y - tf32_hi(v.y), v.z - tf32_hi(v.z), v.w - tf32_hi(v.w));
+                const float4 v = vs[e], h = make_float4(tf32_rn(v.x), tf32_rn(v.y), tf32_rn(v.z), tf32_rn(v.w));
+                vs[e] = h;
+                vl[e] = make_float4(tf32_lo(v.x, h.x), tf32_lo(v.y, h.y), tf32_lo(v.z, h.z), tf32_lo(v.w, h.w));
             }
             tc::fence_async_smem();  // the lo copies -> visible to the tensor core
             __syncwarp();
@@ -440,15 +448,22 @@ qr_proj_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
         if (ok && !*(volatile int *)&sh_abort) {
 #pragma unroll
             for (int c = 0; c < NB; c += 16) {
-                float w[16], wl[16], w2[16];  // hi.hi, hi.lo, lo.hi
+                float w[16], small[16];  // hi.hi, hi.lo + lo.hi
                 const uint32_t lb = tbase + ((uint32_t)(32 * q) << 16) + (uint32_t)c;
                 tc::tmem_ld16(lb, w);
-                tc::tmem_ld16(lb + NB, wl);
-                tc::tmem_ld16(lb + 2 * NB, w2);
+                tc::tmem_ld16(lb + NB, small);
                 tc::tmem_wait_ld();
+                for (uint32_t set = 1; set < min(kSets, (uint32_t)(4 * nt)); ++set) {  // (warp-uniform)
+                    float a[16], b[16];
+                    tc::tmem_ld16(lb + set * 2 * NB, a);
+                    tc::tmem_ld16(lb + set * 2 * NB + NB, b);
+                    tc::tmem_wait_ld();
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) w[k] += a[k], small[k] += b[k];
+                }
                 if (col < wc) {
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) part[((size_t)sp * NB + c + k) * N + c0 + col] = w[k] + (wl[k] + w2[k]);
+                    for (int k = 0; k < 16; ++k) part[((size_t)sp * NB + c + k) * N + c0 + col] = w[k] + small[k];
                 }
             }
         }
@@ -673,13 +688,21 @@ lq_proj_tm_kernel(const __grid_constant__ CUtensorMap tmX, int M, int N, const f
     constexpr int H = 128;                            // rows per block = the MMA's M
     constexpr int kX = 4 * kLqXBox;                   // the stage's 128 rows
     constexpr int kB = NB * 128;                      // V^T of the stage's 32 columns (hi or lo)
-    // At NB = 16 the accumulator is split like qr_proj_tc's (D1 = A_hi [V_hi; V_lo], 2 NB
-    // columns; D2 = A_lo V_hi, NB columns: two MMAs per K step); the wider forms keep one
-    // accumulator and three MMAs (the split one would not leave room for three slots).
+    // At NB = 16 the accumulators are laid out like qr_proj_tc's (A_hi [V_hi; V_lo] and A_lo V_hi
+    // onto its second half: two MMAs per K step); the wider forms take three MMAs onto NB columns
+    // (the split one would not leave room for three slots).  Against the accumulator's rounding
+    // (qr_proj_tc) only two accumulators fit beside the slots, so blocks of kBlk stages take turns on
+    // them and the converters add a finished block's to FP32 sums in registers: its MMAs are known to
+    // have completed when they get the operand slot of the stage two after it, and the next block
+    // on the same accumulator cannot start before they have passed that stage.  NB = 64 has room
+    // for one accumulator only.
     constexpr bool kStack = NB == 16;
     constexpr uint32_t kD = kStack ? 64 : (NB < 32 ? 32 : NB);  // TMEM columns of the accumulator(s)
-    constexpr uint32_t kCols = 256;
-    static_assert(kD + 64 * kLqStages <= 256, "TMEM budget: two blocks per SM");
+    constexpr uint32_t kCols = 256, kSets = NB <= 32 ? 2 : 1;
+    constexpr int kBlk = kSets == 2 ? 4 : 1 << 28;  // >= kLqStages
+    constexpr uint32_t kSetStep = kStack ? 2 * NB : kD + 64 * kLqStages;  // to the second accumulator
+    static_assert(kD + 64 * kLqStages + (NB == 32 ? NB : 0) <= 256, "TMEM budget: two blocks per SM");
+    static_assert(kLqStages == 3, "the stage at which a block is known to be finished");
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t xfull[kMaxStages], xfree[kMaxStages], conv[kLqStages], ofree[kLqStages], accdone;
     __shared__ uint32_t tmem_base;
@@ -748,14 +771,15 @@ lq_proj_tm_kernel(const __grid_constant__ CUtensorMap tmX, int M, int N, const f
                 const uint32_t bh = tc::smem_u32(bhi(o)), bl = tc::smem_u32(blo(o));
 #pragma unroll
                 for (int kk = 0; kk < kLqCols / 8; ++kk) {  // 8 columns per instruction
-                    const uint32_t off = kk * 32, acc = (t > 0 || kk > 0) ? 1u : 0u;
+                    const uint32_t off = kk * 32, acc = t % kBlk > 0 || kk > 0 ? 1u : 0u;
+                    const uint32_t d = tbase + (uint32_t)(t / kBlk) % kSets * kSetStep;
                     if constexpr (kStack) {  // B lo lies right after B hi: [V_hi; V_lo] is one operand
-                        tc::mma_tf32_tmem_a(tbase, ah + 8 * kk, tc::sdesc_sw128(bh + off), id2, acc);
-                        tc::mma_tf32_tmem_a(tbase + 2 * NB, al + 8 * kk, tc::sdesc_sw128(bh + off), id, acc);
+                        tc::mma_tf32_tmem_a(d, ah + 8 * kk, tc::sdesc_sw128(bh + off), id2, acc);
+                        tc::mma_tf32_tmem_a(d + NB, al + 8 * kk, tc::sdesc_sw128(bh + off), id, 1u);
                     } else {
-                        tc::mma_tf32_tmem_a(tbase, ah + 8 * kk, tc::sdesc_sw128(bh + off), id, acc);
-                        tc::mma_tf32_tmem_a(tbase, ah + 8 * kk, tc::sdesc_sw128(bl + off), id, 1u);
-                        tc::mma_tf32_tmem_a(tbase, al + 8 * kk, tc::sdesc_sw128(bh + off), id, 1u);
+                        tc::mma_tf32_tmem_a(d, ah + 8 * kk, tc::sdesc_sw128(bh + off), id, acc);
+                        tc::mma_tf32_tmem_a(d, ah + 8 * kk, tc::sdesc_sw128(bl + off), id, 1u);
+                        tc::mma_tf32_tmem_a(d, al + 8 * kk, tc::sdesc_sw128(bh + off), id, 1u);
                     }
                 }
                 tc::mma_commit(&ofree[o]);  // the operand slot is free once these MMAs have read it
@@ -768,6 +792,21 @@ lq_proj_tm_kernel(const __grid_constant__ CUtensorMap tmX, int M, int N, const f
         const int q = warp & 3, ct = tid - 64;
         constexpr int kVe = NB * kLqCols / 128;  // V entries per thread and stage
         const uint32_t lane_base = tbase + ((uint32_t)(32 * q) << 16);
+        float ysum[NB];
+#pragma unroll
+        for (int k = 0; k < NB; ++k) ysum[k] = 0.f;
+        auto drain = [&](int blk) {  // (warp-uniform)
+            const uint32_t at = lane_base + (uint32_t)blk % kSets * kSetStep;
+#pragma unroll
+            for (int c = 0; c < NB; c += 16) {
+                float a[16], small[16];
+                tc::tmem_ld16(at + (uint32_t)c, a);
+                if constexpr (kStack) tc::tmem_ld16(at + (uint32_t)(NB + c), small);
+                tc::tmem_wait_ld();
+#pragma unroll
+                for (int k = 0; k < 16; ++k) ysum[c + k] += kStack ? a[k] + small[k] : a[k];  // hi.hi + (hi.lo + lo.hi)
+            }
+        };
         // V of stage t, loaded a stage ahead (its L2 latency hides behind the previous stage):
         // entry (k, j) = V(cb + j, k), the address clamped into the split, the value masked to
         // the unit lower form after the load (no branch per load)
@@ -808,10 +847,11 @@ lq_proj_tm_kernel(const __grid_constant__ CUtensorMap tmX, int M, int N, const f
                 break;
             }
             tc::fence_after_sync();
+            if (t >= kBlk + 2 && (t - 2) % kBlk == 0) drain((t - 2) / kBlk - 1);
 #pragma unroll
             for (int c = 0; c < kLqCols; ++c) {
                 h[c] = tf32_hi(x[c]);
-                x[c] -= h[c];
+                x[c] = tf32_lo(x[c], h[c]);
             }
             tc::tmem_st32(lane_base + acol(o), h);
             tc::tmem_st32(lane_base + acol(o) + 32, x);
@@ -821,8 +861,9 @@ lq_proj_tm_kernel(const __grid_constant__ CUtensorMap tmX, int M, int N, const f
             for (int u = 0; u < kVe; ++u) {  // row k, 16-byte chunk (j/4) ^ (k & 7), word j % 4
                 const int e = ct + 128 * u, j = e / NB, k = e % NB;
                 const int w = k * 32 + (((j >> 2) ^ (k & 7)) << 2) + (j & 3);
-                vh[w] = v[u];
-                vl[w] = v[u] - tf32_hi(v[u]);
+                const float h = tf32_rn(v[u]);
+                vh[w] = h;
+                vl[w] = tf32_lo(v[u], h);
             }
             tc::tmem_wait_st();
             tc::fence_async_smem();  // the B copies -> visible to the tensor core
@@ -835,23 +876,10 @@ lq_proj_tm_kernel(const __grid_constant__ CUtensorMap tmX, int M, int N, const f
         tc::fence_after_sync();
         const int i = 32 * q + lane;
         if (ok && !*(volatile int *)&sh_abort) {
+            for (int blk = nt >= 3 ? (nt - 3) / kBlk : 0; blk * kBlk < nt; ++blk) drain(blk);
+            if (i < hr) {
 #pragma unroll
-            for (int c = 0; c < NB; c += 16) {
-                float y[16], yl[16], y2[16];
-                tc::tmem_ld16(lane_base + (uint32_t)c, y);
-                if constexpr (kStack) {  // hi.hi + (hi.lo + lo.hi)
-                    tc::tmem_ld16(lane_base + (uint32_t)(NB + c), yl);
-                    tc::tmem_ld16(lane_base + (uint32_t)(2 * NB + c), y2);
-                }
-                tc::tmem_wait_ld();
-                if constexpr (kStack) {
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) y[k] += yl[k] + y2[k];
-                }
-                if (i < hr) {
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) part[((size_t)s * NB + c + k) * M + i0 + i] = y[k];
-                }
+                for (int k = 0; k < NB; ++k) part[((size_t)s * NB + k) * M + i0 + i] = ysum[k];
             }
         }
     }
