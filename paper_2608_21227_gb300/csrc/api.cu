@@ -96,6 +96,7 @@ struct Stage1Plan {
     // per-step configurations: the tuned table's entry for each step's trailing block
     // (set when the caller fixed no update parameters and a table is installed)
     bool adaptive = false;
+    bool strips = false;  // the caller fixed no update parameters: small blocks take the one-launch update
     nla_dtype dt = NLA_F64;
 };
 
@@ -140,6 +141,17 @@ nla_status check_upd(const Stage1Plan &p, int elem) {
 
 void step_cfgs(const Stage1Plan &p, int Mt, int Nt, nla::UpdCfg &l, nla::UpdCfg &r);
 
+// The FP32 trailing update of one side (0 = QR, 1 = LQ).
+cudaError_t trail_f32(int side, float *X, long ldx, int M, int N, const float *V, long ldv, int nb, const float *Tm,
+                      const Stage1Plan &p, const nla::UpdCfg &c, const nla::UpdScratch &sc, cudaStream_t st) {
+    if (p.strips) {
+        const cudaError_t e = nla::trail_strip(side, X, ldx, M, N, V, ldv, nb, Tm, st);
+        if (e != cudaErrorNotSupported) return e;
+    }
+    return side == 0 ? nla::trail_left<float>(X, ldx, M, N, V, ldv, nb, Tm, c, sc, st)
+                     : nla::trail_right<float>(X, ldx, M, N, V, ldv, nb, Tm, c, sc, st);
+}
+
 template <typename T>
 nla_status run_stage1(T *X, long ldx, int M, int N, const Stage1Plan &p, const Stage1Bufs &bufs,
                       T *tauq_all, T *taup_all, int *dInfo, cudaStream_t st) {
@@ -170,7 +182,7 @@ nla_status run_stage1(T *X, long ldx, int M, int N, const Stage1Plan &p, const S
                          "QR trailing update");
             }
         } else {
-            NLA_LAUNCH(nla::kTrTrailLeft, st, nla::trail_left<T>(X + kb + (long)c0 * ldx, ldx, M - kb, N - c0, panel, ldx, nb, Tq, cfl,
+            NLA_LAUNCH(nla::kTrTrailLeft, st, trail_f32(0, X + kb + (long)c0 * ldx, ldx, M - kb, N - c0, panel, ldx, nb, Tq, p, cfl,
                                         usc, st),
                      "QR trailing update");
         }
@@ -186,8 +198,12 @@ nla_status run_stage1(T *X, long ldx, int M, int N, const Stage1Plan &p, const S
                     continue;
                 }
             }
-            NLA_LAUNCH(nla::kTrTrailRight, st, nla::trail_right<T>(Xr, ldx, M - c0, N - c0, rowp, ldx, nb, Tp, cfr, usc, st),
-                     "LQ trailing update");
+            if constexpr (sizeof(T) == 8)
+                NLA_LAUNCH(nla::kTrTrailRight, st, nla::trail_right<T>(Xr, ldx, M - c0, N - c0, rowp, ldx, nb, Tp, cfr, usc, st),
+                         "LQ trailing update");
+            else
+                NLA_LAUNCH(nla::kTrTrailRight, st, trail_f32(1, Xr, ldx, M - c0, N - c0, rowp, ldx, nb, Tp, p, cfr, usc, st),
+                         "LQ trailing update");
         }
     }
     return NLA_OK;
@@ -230,6 +246,7 @@ Stage1Plan make_plan(int M, int N, nla_dtype dt, const nla_opts *opts, int band_
         const int es = (int)elem_size(dt);
         p.left = fallback_upd(0, es, p.b, p.left);
         p.right = fallback_upd(1, es, p.b, p.right);
+        p.strips = dt == NLA_F32;
         nla_cfg probe;
         p.adaptive = p.update == NLA_UPD_NATIVE && nla_tuned_lookup(M, N, (int)dt, 0, 0, &probe);
         p.dt = dt;

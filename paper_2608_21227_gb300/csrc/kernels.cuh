@@ -66,6 +66,10 @@ size_t tma_cfg_smem(int nb, const UpdCfg &c);
 bool trail_tma_eligible(const float *X, long ldx, const float *V, long ldv, int nb, const UpdScratch &sc);
 cudaError_t trail_tma(int side, float *X, long ldx, int M, int N, const float *V, long ldv, int nb, const float *Tm,
                       const UpdCfg &c, const UpdScratch &sc, cudaStream_t st);
+// update_strip.cu: the whole FP32 update of a small trailing block in one launch (band widths 16
+// and 32, any alignment); cudaErrorNotSupported where the two-kernel path is the better one.
+cudaError_t trail_strip(int side, float *X, long ldx, int M, int N, const float *V, long ldv, int nb, const float *Tm,
+                        cudaStream_t st);
 // The same in two parts: the projection (step 1 + T, into the scratch) and the
 // update of rows [off, off + len) (side 0) / columns [off, off + len) (side 1) of
 // the M x N block; off a multiple of 4.

@@ -179,3 +179,22 @@ def test_stage1_panel_row_limits(nla, dt, m, n, b):
     torch.cuda.synchronize()
     assert int(info.item()) == 0 and int(info2.item()) == 0
     assert err_rel(oracle.bdsvd(d.cpu().numpy(), e.cpu().numpy()), np.linalg.svd(A, compute_uv=False)) <= tol_for(dt, m)
+
+
+@pytest.mark.parametrize("m,n,b,pad", [(17, 17, 16, 0), (40, 37, 16, 1), (513, 513, 16, 0), (515, 130, 16, 1),
+                                       (1030, 600, 16, 2), (2500, 60, 16, 0), (700, 650, 32, 0), (1537, 200, 32, 3),
+                                       (2433, 300, 16, 3)])
+def test_stage1_one_launch_update(nla, m, n, b, pad):
+    # the FP32 update that keeps a strip of lines in a block: ragged strips, long dimensions around its
+    # chunks (512 and 256), every lines-per-strip choice, with and without 16-byte alignment; against
+    # the two-kernel path (which explicit update parameters select) and the values themselves
+    A = np.random.default_rng(3 * m + n).standard_normal((m, n)).astype(np.float32)
+    buf = torch.zeros(n, m + pad, device="cuda")
+    buf[:, :m] = torch.from_numpy(np.ascontiguousarray(A.T)).cuda()
+    ref = np.linalg.svd(A.astype(np.float64), compute_uv=False)
+    cfg = nla.Cfg.make(band=b, tile=32, threads=128, cols_per_block=2, unroll=1)
+    for c in (nla.Cfg.make(band=b), cfg):
+        S, info = nla.gesvd_vals(buf[:, :m].clone() if pad == 0 else buf.clone()[:, :m], cfg=c)
+        torch.cuda.synchronize()
+        assert int(info.item()) == 0
+        assert err_rel(S.double().cpu().numpy(), ref) <= tol_for(1, m)
