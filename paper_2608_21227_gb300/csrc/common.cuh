@@ -103,7 +103,7 @@ NLA_DEV float ld_cg(const float *p) { return __ldcg(p); }
 NLA_DEV void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 NLA_DEV void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// NLA_PDL=1 adds the attribute (default: plain stream order).
+// NLA_PDL=0 drops the attribute (plain stream order).
 bool pdl_enabled();
 
 template <typename... KArgs, typename... Args>

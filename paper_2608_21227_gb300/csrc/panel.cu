@@ -65,12 +65,13 @@ int device_sm_count() {
 
 int panel_max_ctas() { return device_sm_count(); }
 
-// Off by default: at 8192 it measured 182.8 vs 181.9 ms per SVD (the launch gaps
-// between the stage-1 kernels are not where the time goes); NLA_PDL=1 enables it.
+// NLA_PDL=0: plain stream order.  With the panels and the small updates down to 8 to 20 us the
+// launch gaps show (ms per FP32 SVD, off / on: 1024 5.28 / 4.66, 3001 x 1537 10.7 / 9.8, 8192
+// 114.5 / 109.2).
 bool pdl_enabled() {
     static const bool on = [] {
         const char *v = getenv("NLA_PDL");
-        return v && atoi(v) != 0;
+        return !v || atoi(v) != 0;
     }();
     return on;
 }

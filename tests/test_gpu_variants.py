@@ -53,3 +53,38 @@ def test_variant_matches_oracle(name):
     for rec in json.loads(r.stdout.strip().splitlines()[-1]):
         assert rec["info"] == 0, rec
         assert rec["err"] <= rec["tol"], rec
+
+
+@pytest.mark.parametrize("env", [{}, {"NLA_PDL": "0"}])
+def test_whole_svd_captured_and_replayed(env):
+    # programmatic dependent launch is on by default: plain, captured in a graph and replayed on new
+    # data, and with it off, the values agree with the reference
+    child = r"""
+import sys
+import numpy as np, torch
+sys.path.insert(0, sys.argv[1]); sys.path.insert(0, sys.argv[1] + "/tests")
+from paper_2608_21227_gb300 import nla
+from _util import err_rel, tol_for
+for (m, n, dt) in [(700, 500, torch.float32), (2500, 300, torch.float32), (260, 200, torch.float64)]:
+    code = 1 if dt == torch.float32 else 0
+    g = torch.Generator(device="cuda"); g.manual_seed(m)
+    A = torch.randn(n, m, generator=g, device="cuda", dtype=dt)
+    work = nla.workspace(nla.gesvd_vals_workspace(m, n, code, preserve_a=True))
+    S = torch.empty(n, dtype=dt, device="cuda"); info = torch.zeros(1, dtype=torch.int32, device="cuda")
+    run = lambda: nla.gesvd_vals(A, preserve_a=True, work=work, S=S, info=info)
+    run(); torch.cuda.synchronize()
+    st = torch.cuda.Stream(); gr = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(st):
+        with torch.cuda.graph(gr, stream=st):
+            run()
+    for _ in range(2):
+        A.copy_(torch.randn(n, m, generator=g, device="cuda", dtype=dt))
+        S.fill_(float("nan"))
+        gr.replay(); torch.cuda.synchronize()
+        ref = np.linalg.svd(A.double().cpu().numpy(), compute_uv=False)
+        assert int(info.item()) == 0 and err_rel(S.double().cpu().numpy(), ref) <= tol_for(code, m)
+print("ok")
+"""
+    r = subprocess.run([sys.executable, "-c", child, ROOT], env=dict(os.environ, **env), capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0 and r.stdout.strip().endswith("ok"), r.stderr[-2000:]
