@@ -112,7 +112,10 @@ nla_status nla_gesvd_vals_workspace(int m, int n, nla_dtype dtype, const nla_opt
  * Algorithm 2 for its trailing updates).
  * dS receives min(m, n) values in descending order, in dtype.  dA is
  * overwritten unless opts->preserve_a (or m < n, where A^T is formed in the
- * workspace and dA is left intact).  dWork: >= nla_gesvd_vals_workspace bytes,
+ * workspace and dA is left intact).  An FP32 matrix with min(m, n) <= 256 whose
+ * configuration is left open (opts->cfg NULL or all zero) is reduced in one
+ * block's registers where that is faster (the batched kernel's method; dA is
+ * then left intact).  dWork: >= nla_gesvd_vals_workspace bytes,
  * 256-byte aligned.  dInfo: one device int (see conventions). */
 nla_status nla_gesvd_vals(int m, int n, nla_dtype dtype, void *dA, int lda, void *dS,
                           void *dWork, size_t work_bytes, int *dInfo,

@@ -388,6 +388,13 @@ nla_status nla_gesvd_vals(int m, int n, nla_dtype dtype, void *dA, int lda, void
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (dtype == NLA_F64)
         return gesvd_impl<double>(m, n, dtype, (double *)dA, lda, (double *)dS, L, p, opts, dInfo, st);
+    // a small matrix whose configuration the caller left open: in one block's registers
+    const nla_cfg *u = opts ? opts->cfg : nullptr;
+    const bool open = !u || (u->band <= 0 && u->tile <= 0 && u->threads <= 0 && u->cols_per_block <= 0 && u->unroll <= 0);
+    if (open && nla::small_svd_pays(m, n)) {
+        NLA_LAUNCH(nla::kTrBatched, st, nla::small_svd((const float *)dA, m, n, lda, (float *)dS, dInfo, st), "small matrix");
+        return NLA_OK;
+    }
     return gesvd_impl<float>(m, n, dtype, (float *)dA, lda, (float *)dS, L, p, opts, dInfo, st);
 }
 

@@ -29,6 +29,7 @@
 // matrix lived in shared memory or, above 48K elements, in global memory, and every reflector
 // streamed it twice.
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 #include <utility>
 
@@ -512,6 +513,27 @@ __device__ __noinline__ void run_worker(float *smem, int warp, int lane, const f
     wk.run(A, M, N, lda, tr, S);
 }
 
+// One matrix by one block of C::NW warps.
+template <class C>
+__global__ void __launch_bounds__(32 * C::NW, 1)
+one_svd_kernel(const float *A, int M, int N, int lda, int tr, float *S, int *info) {
+    extern __shared__ __align__(16) float smem[];
+    run_worker<C>(smem, threadIdx.x >> 5, threadIdx.x & 31, A, M, N, lda, tr != 0, S);
+    if (threadIdx.x == 0) *info = 0;
+}
+
+template <class C>
+cudaError_t one_launch(const float *A, int M, int N, int lda, bool tr, float *S, int *info, cudaStream_t st) {
+    static nla::PerDeviceOnce attr;
+    constexpr int smem = C::kFloats * (int)sizeof(float);
+    attr.run([] {
+        cudaFuncSetAttribute(one_svd_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaGetLastError();
+    });
+    one_svd_kernel<C><<<1, 32 * C::NW, smem, st>>>(A, M, N, lda, tr ? 1 : 0, S, info);
+    return cudaGetLastError();
+}
+
 __global__ void __launch_bounds__(kThreads, 1)
 batched_svd_kernel(const int *__restrict__ dM, const int *__restrict__ dN, const int *__restrict__ dLda,
                    float *const *dA, float *const *dS, const int *__restrict__ order, unsigned int *ctl,
@@ -560,6 +582,32 @@ batched_svd_kernel(const int *__restrict__ dM, const int *__restrict__ dN, const
 }  // namespace
 
 namespace nla {
+
+// us on GB300, fitted to N = 16 .. 256 and M / N = 1 .. 64: this file's one-block form against the
+// two-stage reduction of a whole GPU, whose chains of steps cost about 3.4 us a column however
+// small the matrix is (N = 64, M = 64: 80 against 209; M = 1,024: 465 against 245; N = 256: 610
+// against 965 square, 1,244 against 1,004 at 512 rows).
+bool small_svd_pays(int m, int n) {
+    const float M = (float)std::max(m, n), N = (float)std::min(m, n);
+    if (N > 256.f || M > 65536.f) return false;
+    const auto chunks = [&](float tile, float rows) { return M > tile ? ceilf(M / rows) : 0.f; };
+    const float one = N <= 64.f    ? 1.3f + 0.8f * chunks(64.f, 128.f)
+                      : N <= 128.f ? 1.3f + 0.55f * chunks(128.f, 128.f)
+                      : N <= 192.f ? 1.65f + 0.7f * chunks(192.f, 192.f)
+                                   : 2.4f + 0.62f * chunks(256.f, 128.f);
+    return one * N < 0.9f * (3.35f * N + 0.0016f * N * N + 0.00035f * M * N);
+}
+
+// Singular values of the column-major m x n matrix (read only), min(m, n) <= 256.
+cudaError_t small_svd(const float *A, int m, int n, int lda, float *S, int *info, cudaStream_t st) {
+    const int M = std::max(m, n), N = std::min(m, n);
+    const bool tr = m < n;
+    if (N > 192) return one_launch<Class0>(A, M, N, lda, tr, S, info, st);
+    if (N > 128) return one_launch<Class1>(A, M, N, lda, tr, S, info, st);
+    if (N > 64) return one_launch<Class2>(A, M, N, lda, tr, S, info, st);
+    return one_launch<Class3>(A, M, N, lda, tr, S, info, st);  // (one warp alone is slower up to 32, too: 82 against 41 us)
+}
+
 // Group sizes per bucket installed by the tuner table (bucket b -> least threads per matrix).
 int g_batched_group[kBuckets] = {0, 0, 0, 0, 0};
 }

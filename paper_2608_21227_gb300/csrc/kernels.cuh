@@ -125,6 +125,10 @@ template <typename T>
 cudaError_t bdsvd_bisect(int n, const double *d, const double *e, T *S, void *scratch, int *info,
                          cudaStream_t st);
 
+// batched.cu: one FP32 matrix with min(m, n) <= 256 by one block, and whether that is the faster way.
+bool small_svd_pays(int m, int n);
+cudaError_t small_svd(const float *A, int m, int n, int lda, float *S, int *info, cudaStream_t st);
+
 int device_sm_count();
 
 }  // namespace nla

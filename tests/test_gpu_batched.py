@@ -157,3 +157,20 @@ def test_class_and_chunk_edges(nla, groups, tmp_path):
             assert err_rel(s.cpu().numpy(), ref) <= 5e-6 * max(A.shape), A.shape
     finally:
         kt.load_config(None)
+
+
+@pytest.mark.parametrize("m,n", [(1, 1), (3, 1), (1, 9), (32, 32), (33, 33), (96, 64), (64, 96), (128, 129), (192, 192),
+                                 (250, 200), (256, 256), (257, 256), (300, 40), (40, 700), (2000, 30), (3000, 250)])
+def test_single_small_matrix(nla, m, n):
+    # nla_gesvd_vals on both sides of the small-matrix rule, padded leading dimension, A left as it was
+    # when asked; the configuration given explicitly takes the two-stage path
+    A = np.random.default_rng(5 * m + n).standard_normal((m, n)).astype(np.float32)
+    t = torch.zeros(n, m + 2, device="cuda")
+    t[:, :m] = torch.from_numpy(np.ascontiguousarray(A.T)).cuda()
+    keep = t.clone()
+    ref = np.linalg.svd(A.astype(np.float64), compute_uv=False)
+    for kw in ({}, {"cfg": nla.Cfg.make(band=16)}):
+        S, info = nla.gesvd_vals(t[:, :m], preserve_a=True, **kw)
+        torch.cuda.synchronize()
+        assert int(info.item()) == 0 and torch.equal(t, keep)
+        assert err_rel(S.cpu().numpy(), ref) <= 5e-6 * max(m, n)
