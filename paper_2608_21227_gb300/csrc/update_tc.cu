@@ -5,10 +5,10 @@
 // mixed-precision form of the contraction).
 //
 // Two launches per side (as in the SIMT path): step 1 on a grid of
-// (128-wide strips) x (splits of the reduction dimension), the last block of a
+// (32-wide strips) x (splits of the reduction dimension), the last block of a
 // strip applying T; step 3 on a 2-D grid of 128 x 128 output tiles.
-// QR side (strips of 128 columns of X):
-//   1. W^T (128 x nbp) = X_strip^T V, accumulated over 32-row tiles.  Each tile
+// QR side (strips of 32 columns of X in step 1, 128 in step 3):
+//   1. W^T (32 x nbp) = X_strip^T V, accumulated over 32-row tiles.  Each tile
 //      of X is scaled per column by 2^-e (e = exponent of the column's largest
 //      magnitude in that tile), rounded to TF32/BF16 and multiplied on the
 //      tensor cores into one of two TMEM accumulators; the previous tile's
@@ -18,7 +18,7 @@
 //   3. For each 128-row tile: D = V_tile W' on the tensor cores, then the
 //      epilogue reads D from TMEM row by row and subtracts it, rescaled, from
 //      X in FP64 (coalesced: one thread per row).
-// LQ side (one block per 128-row strip): the same with rows and columns
+// LQ side (strips of rows): the same with rows and columns
 // exchanged (Y = X_strip V, Y' = Y T, X_strip -= Y' V^T), scaling per row.
 //
 // Panel factorisation, T and the matrix stay FP64; only the two products are
@@ -47,7 +47,8 @@ size_t trail_tc_scratch_bytes(int M, int N, int nb) {
 namespace {
 
 constexpr int kTcThreads = 256;   // 8 warps
-constexpr int kStrip = 128;       // strip width = UMMA M
+constexpr int kStrip = 128;       // UMMA M; step 3's strip width
+constexpr int kLines = 32;        // step 1's strip width
 constexpr int kKt = 32;           // rows (QR) / columns (LQ) of X per step-1 tile
 constexpr int kTmemCols = 256;    // self-test accumulator columns
 
@@ -67,6 +68,10 @@ struct Prec<NLA_UPD_TF32> {
     NLA_DEV static void put(unsigned char *base, uint32_t off, float v) {
         *reinterpret_cast<uint32_t *>(base + off) = tc::to_tf32(v);
     }
+    NLA_DEV static void put4(unsigned char *p, const float *v) {
+        *reinterpret_cast<uint4 *>(p) =
+            make_uint4(tc::to_tf32(v[0]), tc::to_tf32(v[1]), tc::to_tf32(v[2]), tc::to_tf32(v[3]));
+    }
     NLA_DEV static void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) { tc::mma_tf32(d, a, b, id, acc); }
 };
 template <>
@@ -77,6 +82,10 @@ struct Prec<NLA_UPD_BF16> {
     NLA_DEV static float round(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
     NLA_DEV static void put(unsigned char *base, uint32_t off, float v) {
         *reinterpret_cast<uint16_t *>(base + off) = tc::to_bf16(v);
+    }
+    NLA_DEV static void put4(unsigned char *p, const float *v) {
+        *reinterpret_cast<uint2 *>(p) = make_uint2((uint32_t)tc::to_bf16(v[0]) | (uint32_t)tc::to_bf16(v[1]) << 16,
+                                                   (uint32_t)tc::to_bf16(v[2]) | (uint32_t)tc::to_bf16(v[3]) << 16);
     }
     NLA_DEV static void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) { tc::mma_bf16(d, a, b, id, acc); }
 };
@@ -96,6 +105,19 @@ NLA_DEV void put_op(unsigned char *hi, unsigned char *lo, uint32_t off, float v)
     using P = Prec<PREC>;
     P::put(hi, off, v);
     if constexpr (P::split) P::put(lo, off, v - P::round(v));
+}
+
+// Four consecutive K entries of one row (the first a multiple of 4) by one store.
+template <int PREC>
+NLA_DEV void put_op4(unsigned char *hi, unsigned char *lo, uint32_t off, const float *v) {
+    using P = Prec<PREC>;
+    P::put4(hi + off, v);
+    if constexpr (P::split) {
+        float l[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) l[i] = v[i] - P::round(v[i]);
+        P::put4(lo + off, l);
+    }
 }
 
 // power-of-two scale exponent: x * 2^-e lies in [0.5, 1) for the largest |x|
@@ -241,36 +263,45 @@ __global__ void __launch_bounds__(128) tc_selftest_kernel(const float *A, const 
 
 // ---------------------------------------------------------------- step 1 (both sides)
 // Block (strip, split) accumulates the partial W^T (QR side: strip columns x
-// reflectors, reduction over rows [sbeg, send)) or Y (LQ side: strip rows x
+// reflectors, reduction over rows [kbeg, kend)) or Y (LQ side: strip rows x
 // reflectors, reduction over columns) from 32-wide tiles scaled per strip
 // line by 2^-e, rounded and multiplied on the tensor cores; the previous
 // tile's TMEM accumulator is read back (unscaled) into FP32 registers while
 // the next multiply runs.  The last block of the strip (atomic ticket) sums
 // the partials and applies T (QR: W' = T^T W; LQ: Y' = Y T), storing FP32.
+//
+// Bound: the conversions.  A block's tiles follow one another (each adds to the running sum, and
+// the splits are fixed by the order of the sums), so a launch lasts as long as one block converts
+// its split.  A strip therefore has 32 lines, not the MMA's 128: the tensor cores idle anyway, and
+// the other rows of the tile are not written and their products not read.  The tiles are loaded
+// one ahead; K entries are shared out so that a warp's stores to the K-major tile meet in at most
+// two banks' turns (lanes along K met 8 ways).  X 4096 x 1024, nb 16, TF32: 152 -> 48 us (QR), 91 ->
+// 57 us (LQ); 64 lines 1.2x, 128 lines 1.9x as long, at 5120 x 5120 0.95x and 1.09x.
 template <int PREC, int SIDE>
-__global__ void __launch_bounds__(kTcThreads)
+__global__ void __launch_bounds__(kTcThreads, 2)
 tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *__restrict__ V, long ldv, int nb,
             int nbp, const double *__restrict__ Tm, int Ls, float *part, int *pexp, float *fin, int *finexp,
             unsigned int *tickets, int *info) {
     using P = Prec<PREC>;
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ int sh_last;
-    const int es = P::es, rb1 = kKt * es;
+    constexpr int es = P::es, rb1 = kKt * es;
+    constexpr int kWarps = kTcThreads / 32;
     constexpr int nsp = P::split ? 2 : 1;                    // hi (and lo) copies of each tile
     unsigned char *A1 = sm;                                  // 2 x [128 x kKt]  X tile (strip line x K)
     unsigned char *B1 = A1 + 2 * kStrip * rb1;               // 2 x [64 x kKt]   V tile (reflector x K)
     unsigned char *A1l = B1 + 2 * 64 * rb1;                  // lo copies (compensated forms)
     unsigned char *B1l = A1l + (nsp - 1) * 2 * kStrip * rb1;
-    int *ex1 = reinterpret_cast<int *>(B1l + (nsp - 1) * 2 * 64 * rb1);  // 2 x 128
-    int *lmax = ex1 + 2 * kStrip;                            // 2 x 128 biased exponents
-    TcShared *sh = reinterpret_cast<TcShared *>(lmax + 2 * kStrip);
-    float *Wsh = reinterpret_cast<float *>(sm);              // reused after the MMAs: nbp x 128
+    int *ex1 = reinterpret_cast<int *>(B1l + (nsp - 1) * 2 * 64 * rb1);  // 2 x kLines
+    int *lmax = ex1 + 2 * kLines;                                // kWarps x kLines biased exponents (LQ)
+    TcShared *sh = reinterpret_cast<TcShared *>(lmax + kWarps * kLines);
+    float *Wsh = reinterpret_cast<float *>(sm);              // reused after the MMAs: nbp x kLines
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int q = warp & 3, hh = warp >> 2;
     // strip lines: QR -> columns of X, LQ -> rows of X; reduction dimension: the other one
-    const int L0 = blockIdx.x * kStrip;
+    const int L0 = blockIdx.x * kLines;
     const int Lext = SIDE == 0 ? N : M, Kext = SIDE == 0 ? M : N;
-    const int lw = min(kStrip, Lext - L0);
+    const int lw = min(kLines, Lext - L0);
     const int s = blockIdx.y, S = gridDim.y;
     const int kbeg = s * Ls, kend = min(Kext, kbeg + Ls);
     if (warp == 0) {
@@ -289,80 +320,79 @@ tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *
     const uint32_t tbase = sh->tmem_base;
     const uint32_t id1 = tc::idesc(P::fmt, 128, nbp);
     const int half = nbp / 2;
+    const bool reader = q == 0;  // warps 0 and 4 hold the strip's lines (TMEM lanes 0 .. 31), half the reflectors each
     float acc[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) acc[i] = 0.f;
     int erun = kNoExp;  // acc holds the line's partial W scaled by 2^-erun
-    const int m = tid & (kStrip - 1), h = tid >> 7;  // loader: strip line m, K entries h*16 .. h*16+15
+    // Loader: four K entries per thread of one line in every 32 (X) and of one reflector in every
+    // 32 (V).  QR (K contiguous in memory): 8 lanes along K, 4 lines a warp; LQ (lines
+    // contiguous): lanes along the lines, four neighbouring K a warp.
+    const int lr = SIDE == 0 ? warp * 4 + (lane >> 3) : lane;
+    const int kq = SIDE == 0 ? (lane & 7) : warp * 4;
+    constexpr int kStep = SIDE == 0 ? 8 : 1;
     const int ntiles = (kend - kbeg + kKt - 1) / kKt;
+    double xv[4], vv[2][4];
+    const auto load_tile = [&](int t) {
+        const int k0 = kbeg + t * kKt + kq;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int g = k0 + i * kStep;
+            const bool in = g < kend;
+            xv[i] = in && lr < lw ? (SIDE == 0 ? X[g + (long)(L0 + lr) * ldx] : X[(L0 + lr) + (long)g * ldx]) : 0.0;
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int n = 32 * u + lr;
+                vv[u][i] = in && n < nb && g > n ? (SIDE == 0 ? V[g + (long)n * ldv] : V[n + (long)g * ldv])
+                           : in && n < nb && g == n ? 1.0
+                                                    : 0.0;
+            }
+        }
+    };
+    // four converted entries of one row to the hi (and lo) tile
+    const auto put_row = [&](unsigned char *hi, unsigned char *lo, int row, const double *x, int e) {
+        float f[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) f[i] = f64_scaled_to_f32(x[i], e);
+        if (SIDE == 1) {
+            put_op4<PREC>(hi, lo, tc::kmajor_off(row, kq, es, rb1), f);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) put_op<PREC>(hi, lo, tc::kmajor_off(row, kq + i * kStep, es, rb1), f[i]);
+        }
+    };
+    if (ntiles > 0) load_tile(0);
     for (int t = 0; t <= ntiles; ++t) {
         const int buf = t & 1;
         if (t < ntiles) {
-            const int k0 = kbeg + t * kKt;
-            double xv[16];
-            if (SIDE == 0) {
-                // lanes over the tile's 32 rows, warp w over strip columns 16w .. 16w+15:
-                // coalesced column segments; the column's scale from a warp-wide max
-                const int kk = k0 + lane;
-#pragma unroll
-                for (int c = 0; c < 16; ++c) {
-                    const int mc = warp * 16 + c;
-                    xv[c] = (mc < lw && kk < kend) ? X[kk + (long)(L0 + mc) * ldx] : 0.0;
-                }
-            } else {
-                int emx = 0;
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const int kk = k0 + h * 16 + i;
-                    const double v = (m < lw && kk < kend) ? X[(L0 + m) + (long)kk * ldx] : 0.0;
-                    xv[i] = v;
-                    emx = max(emx, f64_biased_exp(v));
-                }
-                lmax[h * kStrip + m] = emx;
-            }
-            for (int idx = tid; idx < nbp * kKt; idx += blockDim.x) {
-                int n, k;
-                if (SIDE == 0) {
-                    k = idx % kKt, n = idx / kKt;
-                } else {
-                    n = idx % nbp, k = idx / nbp;
-                }
-                const int g = k0 + k;
-                double v = 0.0;
-                if (n < nb && g < kend) {
-                    if (SIDE == 0)
-                        v = g > n ? V[g + (long)n * ldv] : (g == n ? 1.0 : 0.0);
-                    else
-                        v = g > n ? V[n + (long)g * ldv] : (g == n ? 1.0 : 0.0);
-                }
-                put_op<PREC>(B1 + buf * 64 * rb1, B1l + buf * 64 * rb1, tc::kmajor_off(n, k, es, rb1),
-                             f64_scaled_to_f32(v, 0));
-            }
+            unsigned char *const At = A1 + buf * kStrip * rb1, *const Atl = A1l + buf * kStrip * rb1;
+            unsigned char *const Bt = B1 + buf * 64 * rb1, *const Btl = B1l + buf * 64 * rb1;
+            int emx = max(max(f64_biased_exp(xv[0]), f64_biased_exp(xv[1])),
+                          max(f64_biased_exp(xv[2]), f64_biased_exp(xv[3])));
             if (SIDE == 0) {
 #pragma unroll
-                for (int c = 0; c < 16; ++c) {
-                    const int mc = warp * 16 + c;
-                    const int e = tile_exp_from_biased(__reduce_max_sync(0xffffffffu, f64_biased_exp(xv[c])));
-                    if (lane == 0) ex1[buf * kStrip + mc] = e;
-                    put_op<PREC>(A1 + buf * kStrip * rb1, A1l + buf * kStrip * rb1, tc::kmajor_off(mc, lane, es, rb1),
-                                 f64_scaled_to_f32(xv[c], e));
-                }
+                for (int o = 1; o < 8; o <<= 1) emx = max(emx, __shfl_xor_sync(0xffffffffu, emx, o));
             } else {
+                lmax[warp * kLines + lane] = emx;
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+                if (32 * u < nbp) put_row(Bt, Btl, 32 * u + lr, vv[u], 0);
+            if (SIDE == 1) {
                 __syncthreads();
-                const int e = tile_exp_from_biased(max(lmax[m], lmax[kStrip + m]));
-                if (h == 0) ex1[buf * kStrip + m] = e;
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    put_op<PREC>(A1 + buf * kStrip * rb1, A1l + buf * kStrip * rb1,
-                                 tc::kmajor_off(m, h * 16 + i, es, rb1), f64_scaled_to_f32(xv[i], e));
+                for (int w = 0; w < kWarps; ++w) emx = max(emx, lmax[w * kLines + lane]);
             }
+            const int e = tile_exp_from_biased(emx);
+            if (SIDE == 0 ? (lane & 7) == 0 : warp == 0) ex1[buf * kLines + lr] = e;
+            put_row(At, Atl, lr, xv, e);
+            if (t + 1 < ntiles) load_tile(t + 1);
             tc::fence_async_smem();
             tc::fence_before_sync();
             __syncthreads();
             tc::fence_after_sync();
             if (tid == 0) {
-                issue<PREC>(tbase + buf * 64, A1 + buf * kStrip * rb1, A1l + buf * kStrip * rb1, rb1,
-                            B1 + buf * 64 * rb1, B1l + buf * 64 * rb1, rb1, rb1, id1, false);
+                issue<PREC>(tbase + buf * 64, At, Atl, rb1, Bt, Btl, rb1, rb1, id1, false);
                 tc::mma_commit(&sh->mbar[buf]);
                 sh->last_bar = buf;
                 sh->last_parity = (t >> 1) & 1;
@@ -376,10 +406,10 @@ tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *
             // the tile's product is scaled by 2^-et per line; the running sum is kept
             // scaled by 2^-erun (erun = the largest et so far), so no factor leaves
             // FP32's range whatever the exponents of X
-            // (ok is warp-uniform: the TMEM loads below are warp-collective, so every lane
-            // executes them; a line whose tile is all zero adds its product with factor 0)
-            const int et = ex1[pb * kStrip + 32 * q + lane];
-            if (ok) {
+            // (ok and reader are warp-uniform: the TMEM loads below are warp-collective, so every
+            // lane executes them; a line whose tile is all zero adds its product with factor 0)
+            if (ok && reader) {
+                const int et = ex1[pb * kLines + lane];
                 float sc = 0.f;
                 if (et != kNoExp) {
                     if (et > erun) {
@@ -390,9 +420,11 @@ tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *
                     }
                     sc = exp2_nonpos(et - erun);
                 }
-                for (int c = 0; c < half; c += 16) {
+#pragma unroll
+                for (int c = 0; c < 32; c += 16) {
+                    if (c >= half) break;
                     float v[16];
-                    tc::tmem_ld16(tbase + pb * 64 + hh * half + c + ((uint32_t)(32 * q) << 16), v);
+                    tc::tmem_ld16(tbase + pb * 64 + hh * half + c, v);
                     tc::tmem_wait_ld();
 #pragma unroll
                     for (int i = 0; i < 16; ++i) acc[c + i] += v[i] * sc;
@@ -410,10 +442,12 @@ tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *
     if (warp == 0) tc::tmem_dealloc(tbase, 128);
     if (sh->fail) return;
     // ---- partial of this split; the last block of the strip finishes
-    const int line = 32 * q + lane;
-    for (int i = 0; i < half; ++i)
-        if (line < lw) part[((size_t)s * nbp + hh * half + i) * Lext + L0 + line] = acc[i];
-    if (hh == 0 && line < lw) pexp[(size_t)s * Lext + L0 + line] = erun;
+    if (reader && lane < lw) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (i < half) part[((size_t)s * nbp + hh * half + i) * Lext + L0 + lane] = acc[i];
+        if (hh == 0) pexp[(size_t)s * Lext + L0 + lane] = erun;
+    }
     __threadfence();
     __syncthreads();
     if (tid == 0) sh_last = atomicAdd(&tickets[blockIdx.x], 1u) == (unsigned)(S - 1);
@@ -421,8 +455,10 @@ tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *
     if (!sh_last) return;
     __threadfence();
     // the line's common exponent: the largest of its splits' (kNoExp: all zero)
-    int *lexp = reinterpret_cast<int *>(Wsh + (size_t)nbp * kStrip);
-    if (tid < kStrip) {
+    int *lexp = reinterpret_cast<int *>(Wsh + (size_t)nbp * kLines);
+    float *Tf = reinterpret_cast<float *>(lexp + kLines);  // T in FP32, nb x nb
+    for (int i = tid; i < nb * nb; i += blockDim.x) Tf[i] = (float)Tm[i];
+    if (tid < kLines) {
         int em = kNoExp;
 #pragma unroll
         for (int qq = 0; qq < 8; ++qq)
@@ -431,8 +467,8 @@ tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *
         if (tid < lw) finexp[L0 + tid] = em == kNoExp ? 0 : em;
     }
     __syncthreads();
-    for (int idx = tid; idx < nbp * kStrip; idx += blockDim.x) {
-        const int l = idx % kStrip, k = idx / kStrip;
+    for (int idx = tid; idx < nbp * kLines; idx += blockDim.x) {
+        const int l = idx % kLines, k = idx / kLines;
         float sum = 0.f;
         if (l < lw && lexp[l] != kNoExp)
 #pragma unroll
@@ -442,16 +478,16 @@ tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *
                     if (es_ != kNoExp)
                         sum += __ldcg(part + ((size_t)qq * nbp + k) * Lext + L0 + l) * exp2_nonpos(es_ - lexp[l]);
                 }
-        Wsh[k * kStrip + l] = sum;
+        Wsh[k * kLines + l] = sum;
     }
     __syncthreads();
-    for (int i = 0; i < half; ++i) {
-        const int kk = hh * half + i;
+    for (int idx = tid; idx < nbp * kLines; idx += blockDim.x) {
+        const int l = idx % kLines, kk = idx / kLines;
         float v = 0.f;
         // QR: W'(kk) = sum_{k <= kk} T(k, kk) W(k);  LQ: Y'(kk) = sum_{k <= kk} Y(k) T(k, kk) -- same form
         if (kk < nb)
-            for (int k = 0; k <= kk; ++k) v += (float)Tm[k + (long)kk * nb] * Wsh[k * kStrip + line];
-        if (line < lw) fin[(size_t)kk * Lext + L0 + line] = v;
+            for (int k = 0; k <= kk; ++k) v += Tf[k + kk * nb] * Wsh[k * kLines + l];
+        if (l < lw) fin[(size_t)kk * Lext + L0 + l] = v;
     }
     if (tid == 0) tickets[blockIdx.x] = 0u;
 }
@@ -461,16 +497,20 @@ tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *
 // subtracts it from X in FP64.  QR: D = V(rows) W'(strip columns); LQ:
 // D = Y'(strip rows) V(columns)^T.  W' / Y' are scaled per strip line by a
 // power of two before rounding; the scale is undone in the epilogue.
-template <int PREC, int SIDE>
-__global__ void __launch_bounds__(kTcThreads)
-tc_x_kernel(double *__restrict__ X, long ldx, int M, int N, const double *__restrict__ V, long ldv, int nb, int nbp,
+//
+// Bound: the latency of its few dependent phases (operands, MMA, X), so each phase has all its
+// loads in flight at once and two blocks share an SM.  X 4096 x 1024, nb 16, TF32: 36 -> 21 us (QR),
+// 44 -> 20 us (LQ), 3.2 TB/s through X, which the L2 holds.
+template <int PREC, int SIDE, int NBP>
+__global__ void __launch_bounds__(kTcThreads, 2)
+tc_x_kernel(double *__restrict__ X, long ldx, int M, int N, const double *__restrict__ V, long ldv, int nb,
             const float *__restrict__ fin, const int *__restrict__ finexp, int *info) {
     using P = Prec<PREC>;
     extern __shared__ __align__(1024) unsigned char sm[];
-    const int es = P::es, rb3 = nbp * es;
+    constexpr int es = P::es, rb3 = NBP * es;
     constexpr int nsp = P::split ? 2 : 1;
-    unsigned char *Aop = sm;                         // [128 x nbp]
-    unsigned char *Bop = Aop + kStrip * rb3;         // [128 x nbp]
+    unsigned char *Aop = sm;                         // [128 x NBP]
+    unsigned char *Bop = Aop + kStrip * rb3;         // [128 x NBP]
     unsigned char *Aopl = Bop + kStrip * rb3;        // lo copies (compensated forms)
     unsigned char *Bopl = Aopl + (nsp - 1) * kStrip * rb3;
     int *exs = reinterpret_cast<int *>(Bopl + (nsp - 1) * kStrip * rb3);  // 128 strip-line exponents
@@ -491,11 +531,55 @@ tc_x_kernel(double *__restrict__ X, long ldx, int M, int N, const double *__rest
         sh->fail = 0;
         sh->last_bar = -1;
     }
-    // W' / Y' strip block: line l, reflector k; scale per line
+    // V block of this tile: QR -> rows T0.. of V (A operand); LQ -> V(T0 + n, k) (B operand).
+    // QR (rows contiguous in memory): one row and half the reflectors a thread; LQ (reflectors
+    // contiguous): 8 lanes along the reflectors, 4 rows a warp.  All loads of a part in flight at once.
     {
-        const int l = tid & (kStrip - 1), hf = tid >> 7;
-        float mx = 0.f;
-        for (int k = hf; k < nbp; k += 2) mx = fmaxf(mx, fabsf(l < lw && k < nb ? fin[(size_t)k * Lext + L0 + l] : 0.f));
+        unsigned char *const dst = SIDE == 0 ? Aop : Bop, *const dstl = SIDE == 0 ? Aopl : Bopl;
+        if (SIDE == 0) {
+            const int r = tid & (kStrip - 1), g = T0 + r;
+#pragma unroll
+            for (int c = 0; c < NBP / 2; c += 16) {
+                const int kb = (tid >> 7) * (NBP / 2) + c;
+                double v[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    v[i] = kb + i < nb && r < tw && g > kb + i ? V[g + (long)(kb + i) * ldv]
+                           : kb + i < nb && r < tw && g == kb + i ? 1.0
+                                                                  : 0.0;
+#pragma unroll
+                for (int i = 0; i < 16; i += 4) {
+                    float f[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) f[j] = f64_scaled_to_f32(v[i + j], 0);
+                    put_op4<PREC>(dst, dstl, tc::kmajor_off(r, kb + i, es, rb3), f);
+                }
+            }
+        } else {
+#pragma unroll
+            for (int c = 0; c < NBP; c += 32) {
+                double v[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    const int k = c + (i & 3) * 8 + (lane & 7), r = (i >> 2) * 32 + warp * 4 + (lane >> 3), g = T0 + r;
+                    v[i] = k < nb && r < tw && g > k ? V[k + (long)g * ldv] : k < nb && r < tw && g == k ? 1.0 : 0.0;
+                }
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    const int k = c + (i & 3) * 8 + (lane & 7), r = (i >> 2) * 32 + warp * 4 + (lane >> 3);
+                    put_op<PREC>(dst, dstl, tc::kmajor_off(r, k, es, rb3), f64_scaled_to_f32(v[i], 0));
+                }
+            }
+        }
+    }
+    // W' / Y' strip block: line l, half of the reflectors; scale per line
+    {
+        const int l = tid & (kStrip - 1), hf = tid >> 7, kb = hf * (NBP / 2);
+        float w[NBP / 2], mx = 0.f;
+#pragma unroll
+        for (int i = 0; i < NBP / 2; ++i) w[i] = l < lw && kb + i < nb ? fin[(size_t)(kb + i) * Lext + L0 + l] : 0.f;
+#pragma unroll
+        for (int i = 0; i < NBP / 2; ++i) mx = fmaxf(mx, fabsf(w[i]));
         lmax[hf * kStrip + l] = mx;
         __syncthreads();
         // fin holds W' / Y' scaled by 2^-finexp per line (step 1); rescaled here so the
@@ -503,31 +587,14 @@ tc_x_kernel(double *__restrict__ X, long ldx, int M, int N, const double *__rest
         const int e = scale_exp((double)fmaxf(lmax[l], lmax[kStrip + l]));
         if (hf == 0) exs[l] = e + (l < lw ? finexp[L0 + l] : 0);
         // QR: B operand rows = strip columns (N dim), K = reflectors; LQ: A operand rows = strip rows
-        unsigned char *dst = SIDE == 0 ? Bop : Aop;
-        unsigned char *dstl = SIDE == 0 ? Bopl : Aopl;
-        for (int k = hf; k < nbp; k += 2) {
-            const float v = (l < lw && k < nb) ? fin[(size_t)k * Lext + L0 + l] : 0.f;
-            put_op<PREC>(dst, dstl, tc::kmajor_off(l, k, es, rb3), ldexpf(v, -e));
+        unsigned char *const dst = SIDE == 0 ? Bop : Aop, *const dstl = SIDE == 0 ? Bopl : Aopl;
+#pragma unroll
+        for (int i = 0; i < NBP / 2; i += 4) {
+            float f[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) f[j] = ldexpf(w[i + j], -e);
+            put_op4<PREC>(dst, dstl, tc::kmajor_off(l, kb + i, es, rb3), f);
         }
-    }
-    // V block of this tile: QR -> rows T0.. of V (A operand); LQ -> V(T0 + n, k) (B operand)
-    for (int idx = tid; idx < kStrip * nbp; idx += blockDim.x) {
-        int r, k;
-        if (SIDE == 0) {
-            r = idx % kStrip, k = idx / kStrip;
-        } else {
-            k = idx % nbp, r = idx / nbp;
-        }
-        const int g = T0 + r;
-        double v = 0.0;
-        if (k < nb && r < tw) {
-            if (SIDE == 0)
-                v = g > k ? V[g + (long)k * ldv] : (g == k ? 1.0 : 0.0);
-            else
-                v = g > k ? V[k + (long)g * ldv] : (g == k ? 1.0 : 0.0);
-        }
-        put_op<PREC>(SIDE == 0 ? Aop : Bop, SIDE == 0 ? Aopl : Bopl, tc::kmajor_off(r, k, es, rb3),
-                     f64_scaled_to_f32(v, 0));
     }
     tc::fence_async_smem();
     tc::fence_before_sync();
@@ -540,30 +607,38 @@ tc_x_kernel(double *__restrict__ X, long ldx, int M, int N, const double *__rest
         sh->last_bar = 0;
         sh->last_parity = 0;
     }
+    // D row = MMA row (QR: X row T0 + row; LQ: strip row L0 + row); D column = MMA column.  X is read
+    // 16 columns at a time, the first while the MMAs run, the next before the stores of the last
+    // (a load after each store waits out the memory latency 64 times).
+    const int row = 32 * q + lane;
+    const int rlim = SIDE == 0 ? tw : lw, clim = SIDE == 0 ? lw : tw;
+    double *const Xd = SIDE == 0 ? X + T0 + (long)L0 * ldx : X + L0 + (long)T0 * ldx;
+    double xc[16];
+    const auto load16 = [&](int c) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int col = hh * 64 + c + i;
+            xc[i] = row < rlim && col < clim ? Xd[row + (long)col * ldx] : 0.0;
+        }
+    };
+    load16(0);
     const bool ok = tc::mbar_wait_warp(&sh->mbar[0], 0, info);
     if (!ok && lane == 0) sh->fail = 1;
     tc::fence_after_sync();
     if (ok) {
-        // D row = MMA row (QR: X row T0 + row; LQ: strip row L0 + row); D column = MMA column
-        const int row = 32 * q + lane;
+#pragma unroll 1
         for (int c = 0; c < 64; c += 16) {
             float v[16];
             tc::tmem_ld16(tbase + hh * 64 + c + ((uint32_t)(32 * q) << 16), v);
             tc::tmem_wait_ld();
+            double xo[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) xo[i] = xc[i] - f32_scaled_to_f64(v[i], exs[SIDE == 0 ? hh * 64 + c + i : row]);
+            if (c + 16 < 64) load16(c + 16);
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
                 const int col = hh * 64 + c + i;
-                if (SIDE == 0) {
-                    if (row < tw && col < lw) {
-                        double *px = X + (T0 + row) + (long)(L0 + col) * ldx;
-                        *px -= f32_scaled_to_f64(v[i], exs[col]);
-                    }
-                } else {
-                    if (row < lw && col < tw) {
-                        double *px = X + (L0 + row) + (long)(T0 + col) * ldx;
-                        *px -= f32_scaled_to_f64(v[i], exs[row]);
-                    }
-                }
+                if (row < rlim && col < clim) Xd[row + (long)col * ldx] = xo[i];
             }
         }
     }
@@ -576,22 +651,43 @@ tc_x_kernel(double *__restrict__ X, long ldx, int M, int N, const double *__rest
 
 size_t tc_w_smem(int es, int nsp) {
     const size_t rb1 = (size_t)kKt * es;
-    return std::max((size_t)nsp * (2 * kStrip * rb1 + 2 * 64 * rb1) + 2 * kStrip * 4 + 2 * kStrip * 8 +
+    return std::max((size_t)nsp * (2 * kStrip * rb1 + 2 * 64 * rb1) + (size_t)(2 + kTcThreads / 32) * kLines * 4 +
                         sizeof(TcShared) + 64,
-                    (size_t)64 * kStrip * 4 + kStrip * 4 + 64);
+                    (size_t)64 * kLines * 4 + kLines * 4 + (size_t)64 * 64 * 4 + 64);
 }
 size_t tc_x_smem(int es, int nbp, int nsp) {
     return (size_t)nsp * 2 * kStrip * nbp * es + kStrip * 4 + 2 * kStrip * 4 + sizeof(TcShared) + 64;
 }
 
 template <int PREC, int SIDE>
+cudaError_t launch_tc_w(const double *X, long ldx, int M, int N, const double *V, long ldv, int nb, int nbp,
+                        const double *Tm, int S, int Ls, float *part, int *pexp, float *fin, int *finexp,
+                        const UpdScratch &sc, int *info, cudaStream_t st) {
+    static PerDeviceOnce once;
+    allow_max_smem(tc_w_kernel<PREC, SIDE>, once);
+    const int Lext = SIDE == 0 ? N : M;
+    tc_w_kernel<PREC, SIDE><<<dim3((Lext + kLines - 1) / kLines, S), kTcThreads,
+                                  tc_w_smem(Prec<PREC>::es, Prec<PREC>::split ? 2 : 1), st>>>(
+        X, ldx, M, N, V, ldv, nb, nbp, Tm, Ls, part, pexp, fin, finexp, sc.tickets, info);
+    return cudaGetLastError();
+}
+
+template <int PREC, int SIDE, int NBP>
+cudaError_t launch_tc_x(double *X, long ldx, int M, int N, const double *V, long ldv, int nb, const float *fin,
+                        const int *finexp, int *info, cudaStream_t st) {
+    static PerDeviceOnce once;
+    allow_max_smem(tc_x_kernel<PREC, SIDE, NBP>, once);
+    const int Lext = SIDE == 0 ? N : M, Text = SIDE == 0 ? M : N;
+    tc_x_kernel<PREC, SIDE, NBP><<<dim3((Lext + kStrip - 1) / kStrip, (Text + kStrip - 1) / kStrip), kTcThreads,
+                                   tc_x_smem(Prec<PREC>::es, NBP, Prec<PREC>::split ? 2 : 1), st>>>(
+        X, ldx, M, N, V, ldv, nb, fin, finexp, info);
+    return cudaGetLastError();
+}
+
+template <int PREC, int SIDE>
 cudaError_t launch_tc(double *X, long ldx, int M, int N, const double *V, long ldv, int nb, const double *Tm,
                       const UpdScratch &sc, int *info, cudaStream_t st) {
     const int nbp = nb <= 32 ? 32 : 64;
-    const int es = Prec<PREC>::es, nsp = Prec<PREC>::split ? 2 : 1;
-    static PerDeviceOnce a1, a3;
-    allow_max_smem(tc_w_kernel<PREC, SIDE>, a1);
-    allow_max_smem(tc_x_kernel<PREC, SIDE>, a3);
     const int Lext = SIDE == 0 ? N : M, Kext = SIDE == 0 ? M : N;
     const int nblk = (Lext + kStrip - 1) / kStrip;
     int S = (3 * device_sm_count() + nblk - 1) / nblk;
@@ -605,14 +701,11 @@ cudaError_t launch_tc(double *X, long ldx, int M, int N, const double *V, long l
     float *fin = part + (size_t)8 * 64 * L;
     int *pexp = reinterpret_cast<int *>(fin + (size_t)64 * L);
     int *finexp = pexp + (size_t)8 * L;
-    tc_w_kernel<PREC, SIDE><<<dim3(nblk, S), kTcThreads, tc_w_smem(es, nsp), st>>>(X, ldx, M, N, V, ldv, nb, nbp, Tm, Ls,
-                                                                             part, pexp, fin, finexp, sc.tickets, info);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e =
+        launch_tc_w<PREC, SIDE>(X, ldx, M, N, V, ldv, nb, nbp, Tm, S, Ls, part, pexp, fin, finexp, sc, info, st);
     if (e != cudaSuccess) return e;
-    const int Text = SIDE == 0 ? M : N;
-    tc_x_kernel<PREC, SIDE><<<dim3(nblk, (Text + kStrip - 1) / kStrip), kTcThreads, tc_x_smem(es, nbp, nsp), st>>>(
-        X, ldx, M, N, V, ldv, nb, nbp, fin, finexp, info);
-    return cudaGetLastError();
+    return nbp == 32 ? launch_tc_x<PREC, SIDE, 32>(X, ldx, M, N, V, ldv, nb, fin, finexp, info, st)
+                     : launch_tc_x<PREC, SIDE, 64>(X, ldx, M, N, V, ldv, nb, fin, finexp, info, st);
 }
 
 // Element-wise check of the two conversions (nla_scale_selftest).

@@ -224,3 +224,14 @@ def test_mixed_stage1_keeps_sigma(nla, prec, m, n, b):
     i, j = np.indices(D.shape)
     assert np.all(D[(j - i < 0) | (j - i > b)] == 0)
     assert err_rel(oracle.svdvals(D), oracle.svdvals(A)) <= 10 * U_OF[prec] * math.sqrt(m / b)
+
+
+@pytest.mark.parametrize("prec", [1, 2, 3, 4])
+@pytest.mark.parametrize("m,n,b", [(33, 32, 16), (97, 65, 32), (31, 129, 16), (289, 95, 64), (1060, 40, 32)])
+def test_mixed_update_edges(nla, prec, m, n, b):
+    # strips of 32 lines, tiles of 32 and splits of the reduction dimension with one line or
+    # entry more or less than full; the bound is the first-order model of the mixed form
+    k = min(m, n)
+    A = inputs.prescribed(m, n, inputs.geometric_sigma(k, 1e4), seed=m + n)
+    err = err_rel(mixed_run(nla, A, prec, b), oracle.svdvals(A))
+    assert err <= 10 * U_OF[prec] * math.sqrt(max(m, n) / b)
