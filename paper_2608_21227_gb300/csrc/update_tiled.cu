@@ -8,14 +8,14 @@
 //   Step 1: for every staged row (column) of X the thread does R x 4 FMAs from
 //           one 128-bit shared load of X and R reflector values that the whole
 //           warp shares (broadcast).
-//   Step 3: the thread updates sub-blocks of 4 x 4 entries of the staged X
-//           tile; per reflector one 128-bit load of W' and one broadcast
-//           128-bit load of V (stored k-major) feed 16 FMAs.
+//   Step 3: the thread updates sub-blocks of A x 4 entries of the staged X
+//           tile (A = 4; 2 or 1 where FP64 needs more warps); per reflector
+//           one 128-bit load of W' and one broadcast load of V (128-bit for
+//           A = 4; stored k-major) feed 4 A FMAs.
 //
-// Two launches per side keep every SM busy: step 1 runs on a grid of
-// (strips) x (splits of the long dimension, about three waves in all) and the
-// last block of each strip -- chosen by an atomic ticket, so nothing waits --
-// reduces the partial sums and applies T (step 2); step 3 runs on a full 2-D
+// Two launches per side keep every SM busy: step 1 runs on a grid of (strips) x
+// (splits of the long dimension) and the last block of each strip -- chosen by
+// an atomic ticket, so nothing waits -- reduces the partial sums and applies T (step 2); step 3 runs on a full 2-D
 // grid of (tile x strip) blocks.
 //
 // QR side: X tiles are staged row-major with an XOR swizzle of the 4-column
@@ -56,9 +56,16 @@ struct Vec4<double> {
 // Swizzled position of X(r, c) in a row-major tile with w columns.
 NLA_DEV int swz(int r, int c, int w) { return r * w + ((((c >> 2) ^ (r & 7))) << 2) + (c & 3); }
 
+constexpr int kMaxSplit = 8;
+
 size_t tiled_smem(int side, int elem, int nb, int th, int w) {
     (void)side;
     return (size_t)elem * ((size_t)th * w + (size_t)th * (nb + 4) + (size_t)nb * w);
+}
+// Step 1: elements before W (nb x w): the X and V tiles, later T.
+__host__ NLA_DEV int tiled_w_offset(int nb, int th, int w) {
+    const int tiles = th * (w + nb + 4), t = (nb * nb + 3) / 4 * 4;
+    return tiles > t ? tiles : t;
 }
 
 // R = reflectors per thread, or 0 if (nb, threads, cpb, tile, unroll) do not tile.
@@ -91,7 +98,7 @@ __global__ void left_w_kernel(const T *__restrict__ X, long ldx, int M, int N, c
     const int ldv_s = nb + 4;
     T *Xs = reinterpret_cast<T *>(smem_raw);  // th x w, swizzled
     T *Vs = Xs + (size_t)th * w;             // th x (nb+4) row-major
-    T *Ws = Vs + (size_t)th * ldv_s;         // nb x w row-major
+    T *Ws = reinterpret_cast<T *>(smem_raw) + tiled_w_offset(nb, th, w);  // nb x w row-major
     const int tid = threadIdx.x, nt = blockDim.x;
     const int ncg = w >> 2, cg = tid % ncg, rg = tid / ncg;
     const int c0 = blockIdx.x * w, wc = min(w, N - c0);
@@ -149,43 +156,44 @@ __global__ void left_w_kernel(const T *__restrict__ X, long ldx, int M, int N, c
     __syncthreads();
     if (!sh_last) return;
     __threadfence();
-    // ---- step 2 (last block of the strip): W = sum of partials; W' = T^T W
+    // ---- step 2 (last block of the strip): sum of the partials, times T.  A sum's S loads are in
+    // flight together and T waits in shared memory.
+    T *const Ts = reinterpret_cast<T *>(smem_raw);  // nb x nb, where the tiles were
+#pragma unroll 1
+    for (int idx = tid; idx < nb * w; idx += nt) {
+        const int c = idx % w, k = idx / w;
+        T p[kMaxSplit], sum = T(0);
 #pragma unroll
-    for (int i = 0; i < R; ++i)
+        for (int q = 0; q < kMaxSplit; ++q)
+            p[q] = q < S && c < wc ? __ldcg(part + ((size_t)q * nb + k) * N + c0 + c) : T(0);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int c = 4 * cg + j;
-            T sum = T(0);
-            if (c < wc)
-                for (int q = 0; q < S; ++q) sum += __ldcg(part + ((size_t)q * nb + R * rg + i) * N + c0 + c);
-            acc[i][j] = sum;
-        }
-#pragma unroll
-    for (int i = 0; i < R; ++i) Vec4<T>::st(Ws + (R * rg + i) * w + 4 * cg, acc[i]);
+        for (int q = 0; q < kMaxSplit; ++q) sum += p[q];
+        Ws[k * w + c] = sum;
+    }
+    for (int idx = tid; idx < nb * nb; idx += nt) Ts[idx] = Tm[idx];
     __syncthreads();
+    const int nrg = nt / ncg;
 #pragma unroll
     for (int i = 0; i < R; ++i) {
-        const int kk = R * rg + i;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
+        const int kk = rg + nrg * i;  // (interleaved: term counts grow with kk)
+        T a[4] = {};
+#pragma unroll 2
         for (int k = 0; k <= kk; ++k) {
-            const T t = Tm[k + (long)kk * nb];
+            const T t = Ts[k + kk * nb];
             T wv[4];
             Vec4<T>::ld(Ws + k * w + 4 * cg, wv);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] += t * wv[j];
+            for (int j = 0; j < 4; ++j) a[j] += t * wv[j];
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int c = 4 * cg + j;
-            if (c < wc) fin[(size_t)kk * N + c0 + c] = acc[i][j];
-        }
+        for (int j = 0; j < 4; ++j)
+            if (4 * cg + j < wc) fin[(size_t)kk * N + c0 + 4 * cg + j] = a[j];
     }
     if (tid == 0) tickets[blockIdx.x] = 0u;  // ready for the next launch
 }
 
 // Step 3: block (cb, rb) updates the th x w tile X(rb, cb) -= V(rb, :) W'(:, cb).
-template <typename T, int U>
+template <typename T, int U, int A>
 __global__ void left_x_kernel(T *__restrict__ X, long ldx, int M, int N, const T *__restrict__ V, long ldv, int nb,
                               int th, int w, const T *__restrict__ fin) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -211,25 +219,30 @@ __global__ void left_x_kernel(T *__restrict__ X, long ldx, int M, int N, const T
         Ws[k * w + c] = c < wc ? fin[(size_t)k * N + c0 + c] : T(0);
     }
     __syncthreads();
-    const int rpt = th / nrg;  // rows per thread, a multiple of 4
-    for (int rb = rg * rpt; rb < rg * rpt + rpt; rb += 4) {
-        T sacc[4][4];
+    const int rpt = th / nrg;  // rows per thread, a multiple of A
+    for (int rb = rg * rpt; rb < rg * rpt + rpt; rb += A) {
+        T sacc[A][4];
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+        for (int a = 0; a < A; ++a)
 #pragma unroll
             for (int j = 0; j < 4; ++j) sacc[a][j] = T(0);
 #pragma unroll U
         for (int k = 0; k < nb; ++k) {
-            T v[4], wv[4];
-            Vec4<T>::ld(Vs + k * th + rb, v);
+            T v[A], wv[4];
+            if constexpr (A == 4) {
+                Vec4<T>::ld(Vs + k * th + rb, v);
+            } else {
+#pragma unroll
+                for (int a = 0; a < A; ++a) v[a] = Vs[k * th + rb + a];
+            }
             Vec4<T>::ld(Ws + k * w + 4 * cg, wv);
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
+            for (int a = 0; a < A; ++a)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) sacc[a][j] += v[a] * wv[j];
         }
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
+        for (int a = 0; a < A; ++a) {
             T *p = Xs + swz(rb + a, 4 * cg, w);
             T x[4];
             Vec4<T>::ld(p, x);
@@ -257,7 +270,7 @@ __global__ void right_w_kernel(const T *__restrict__ X, long ldx, int M, int N, 
     const int ldv_s = nb + 4;
     T *Xs = reinterpret_cast<T *>(smem_raw);  // th columns x h rows, column-major
     T *Vs = Xs + (size_t)th * h;             // th x (nb+4): row c = V(c, :)
-    T *Ys = Vs + (size_t)th * ldv_s;         // nb x h
+    T *Ys = reinterpret_cast<T *>(smem_raw) + tiled_w_offset(nb, th, h);  // nb x h
     const int tid = threadIdx.x, nt = blockDim.x;
     const int ncg = h >> 2, cg = tid % ncg, rg = tid / ncg;
     const int i0 = blockIdx.x * h, hr = min(h, M - i0);
@@ -314,42 +327,44 @@ __global__ void right_w_kernel(const T *__restrict__ X, long ldx, int M, int N, 
     __syncthreads();
     if (!sh_last) return;
     __threadfence();
+    // ---- step 2 (last block of the strip): sum of the partials, times T.  A sum's S loads are in
+    // flight together and T waits in shared memory.
+    T *const Ts = reinterpret_cast<T *>(smem_raw);  // nb x nb, where the tiles were
+#pragma unroll 1
+    for (int idx = tid; idx < nb * h; idx += nt) {
+        const int c = idx % h, k = idx / h;
+        T p[kMaxSplit], sum = T(0);
 #pragma unroll
-    for (int i = 0; i < R; ++i)
+        for (int q = 0; q < kMaxSplit; ++q)
+            p[q] = q < S && c < hr ? __ldcg(part + ((size_t)q * nb + k) * M + i0 + c) : T(0);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int r = 4 * cg + j;
-            T sum = T(0);
-            if (r < hr)
-                for (int q = 0; q < S; ++q) sum += __ldcg(part + ((size_t)q * nb + R * rg + i) * M + i0 + r);
-            acc[i][j] = sum;
-        }
-#pragma unroll
-    for (int i = 0; i < R; ++i) Vec4<T>::st(Ys + (R * rg + i) * h + 4 * cg, acc[i]);
+        for (int q = 0; q < kMaxSplit; ++q) sum += p[q];
+        Ys[k * h + c] = sum;
+    }
+    for (int idx = tid; idx < nb * nb; idx += nt) Ts[idx] = Tm[idx];
     __syncthreads();
+    const int nrg = nt / ncg;
 #pragma unroll
     for (int i = 0; i < R; ++i) {
-        const int kk = R * rg + i;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
+        const int kk = rg + nrg * i;  // (interleaved: term counts grow with kk)
+        T a[4] = {};
+#pragma unroll 2
         for (int k = 0; k <= kk; ++k) {
-            const T t = Tm[k + (long)kk * nb];
+            const T t = Ts[k + kk * nb];
             T yv[4];
             Vec4<T>::ld(Ys + k * h + 4 * cg, yv);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] += t * yv[j];
+            for (int j = 0; j < 4; ++j) a[j] += t * yv[j];
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int r = 4 * cg + j;
-            if (r < hr) fin[(size_t)kk * M + i0 + r] = acc[i][j];
-        }
+        for (int j = 0; j < 4; ++j)
+            if (4 * cg + j < hr) fin[(size_t)kk * M + i0 + 4 * cg + j] = a[j];
     }
     if (tid == 0) tickets[blockIdx.x] = 0u;
 }
 
 // Step 3: block (rb, cbk) updates the h x th tile X(rb, cbk) -= Y'(rb, :) V(cbk, :)^T.
-template <typename T, int U>
+template <typename T, int U, int A>
 __global__ void right_x_kernel(T *__restrict__ X, long ldx, int M, int N, const T *__restrict__ Vt, long ldvt, int nb,
                                int th, int h, const T *__restrict__ fin) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -376,24 +391,29 @@ __global__ void right_x_kernel(T *__restrict__ X, long ldx, int M, int N, const 
     }
     __syncthreads();
     const int cpt = th / nrg;
-    for (int cbl = rg * cpt; cbl < rg * cpt + cpt; cbl += 4) {
-        T sacc[4][4];  // [column a][row j]
+    for (int cbl = rg * cpt; cbl < rg * cpt + cpt; cbl += A) {
+        T sacc[A][4];  // [column a][row j]
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+        for (int a = 0; a < A; ++a)
 #pragma unroll
             for (int j = 0; j < 4; ++j) sacc[a][j] = T(0);
 #pragma unroll U
         for (int k = 0; k < nb; ++k) {
-            T v[4], yv[4];
-            Vec4<T>::ld(Vs + k * th + cbl, v);
+            T v[A], yv[4];
+            if constexpr (A == 4) {
+                Vec4<T>::ld(Vs + k * th + cbl, v);
+            } else {
+#pragma unroll
+                for (int a = 0; a < A; ++a) v[a] = Vs[k * th + cbl + a];
+            }
             Vec4<T>::ld(Ys + k * h + 4 * cg, yv);
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
+            for (int a = 0; a < A; ++a)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) sacc[a][j] += v[a] * yv[j];
         }
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
+        for (int a = 0; a < A; ++a) {
             T *p = Xs + (cbl + a) * h + 4 * cg;
             T x[4];
             Vec4<T>::ld(p, x);
@@ -410,8 +430,6 @@ __global__ void right_x_kernel(T *__restrict__ X, long ldx, int M, int N, const 
 }
 
 // -------------------------------------------------------------------- dispatch
-constexpr int kMaxSplit = 8;
-
 // partial slabs, the projection's W' / Y', and room for the mixed path's line exponents
 size_t tiled_scratch_elems(int M, int N) { return (size_t)(kMaxSplit + 2) * 64 * (size_t)std::max(std::max(M, N), 1); }
 size_t tiled_tickets(int M, int N) { return (size_t)std::max(M, N) / 32 + 2; }
@@ -423,52 +441,116 @@ static int split_count(int L, int th, int nblk) {
     return S;
 }
 
-template <typename T, int R, int U>
-static cudaError_t run_tiled(int side, T *X, long ldx, int M, int N, const T *V, long ldv, int nb, const T *Tm,
-                             const UpdCfg &c, size_t smem, const UpdScratch &sc, cudaStream_t st) {
-    const int w = 32 * c.cpb, th = c.tile;
-    T *part = reinterpret_cast<T *>(sc.work);
-    T *fin = part + (size_t)kMaxSplit * 64 * std::max(M, N);
-    if (side == 0) {
-        static PerDeviceOnce a1, a3;
-        allow_max_smem(left_w_kernel<T, R, U>, a1);
-        allow_max_smem(left_x_kernel<T, U>, a3);
-        const int nblk = (N + w - 1) / w;
-        int S = split_count(M, th, nblk);
-        const int Ms = ((M + S - 1) / S + th - 1) / th * th;
-        S = (M + Ms - 1) / Ms;
-        left_w_kernel<T, R, U><<<dim3(nblk, S), c.threads, smem, st>>>(X, ldx, M, N, V, ldv, nb, Tm, th, w, Ms, part,
-                                                                       fin, sc.tickets);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        left_x_kernel<T, U><<<dim3(nblk, (M + th - 1) / th), c.threads, smem, st>>>(X, ldx, M, N, V, ldv, nb, th, w,
-                                                                                   fin);
-    } else {
-        static PerDeviceOnce a1, a3;
-        allow_max_smem(right_w_kernel<T, R, U>, a1);
-        allow_max_smem(right_x_kernel<T, U>, a3);
-        const int nblk = (M + w - 1) / w;
-        int S = split_count(N, th, nblk);
-        const int Ns = ((N + S - 1) / S + th - 1) / th * th;
-        S = (N + Ns - 1) / Ns;
-        right_w_kernel<T, R, U><<<dim3(nblk, S), c.threads, smem, st>>>(X, ldx, M, N, V, ldv, nb, Tm, th, w, Ns, part,
-                                                                        fin, sc.tickets);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        right_x_kernel<T, U><<<dim3(nblk, (N + th - 1) / th), c.threads, smem, st>>>(X, ldx, M, N, V, ldv, nb, th, w,
-                                                                                    fin);
+// The blocks of one launch: strips of w lines and tiles of th; step 1: R reflectors a thread and
+// S splits of Ms entries; step 3: A lines of the tile at a time a thread.
+struct Shape {
+    int threads, w, th, R, S, Ms, A;
+};
+
+// FP64: an SM's pipe (a warp's FMA holds a quarter of it for 64 cycles) is the bound, not memory,
+// so a launch lasts as long as the quarter with the most warps: ceil(blocks / SMs) blocks, their
+// warps over four quarters, and a warp's FMAs.  The configuration's block is the largest one; it is
+// halved along the strip (and, in step 3, along the tile), with all or half of its threads, where
+// this count says that more SMs or quarters work.  Step 1 takes the number of splits and their
+// length (whole 64-byte lines) by it too.  A halving has to win 2 %: smaller blocks stage V more
+// often.  FP32 is bound by memory and keeps its tuned blocks and splits.  Updates of a whole
+// reduction, 64 x 64 blocks with three waves of splits before: 2048 x 2048, band 16, 35.9 -> 30.4 ms
+// (21.6 at the pipe's rate); 256 x 256, band 32, 1.60 -> 0.70 ms.
+static double quarter_warps(long blocks, int threads) {
+    const long sm = device_sm_count();
+    return (double)(((blocks + sm - 1) / sm * (threads / 32) + 3) / 4);
+}
+
+template <typename T>
+static Shape step1_shape(int side, int nb, int R, const UpdCfg &c, int strip, int len) {
+    Shape best{c.threads, 32 * c.cpb, c.tile, R, 1, 0, 4};
+    if constexpr (sizeof(T) == 4) {
+        best.S = split_count(len, c.tile, (strip + best.w - 1) / best.w);
+        best.Ms = ((len + best.S - 1) / best.S + c.tile - 1) / c.tile * c.tile;
+        best.S = (len + best.Ms - 1) / best.Ms;
+        return best;
     }
+    double least = 0;
+    for (int h = 1; h <= 2; ++h)
+        for (int ht = 1; ht <= 2; ++ht) {
+            const int w = 32 * c.cpb / h, threads = c.threads / ht;
+            if (w < 32 || threads % 32 || threads % (w / 4) || nb % (threads / (w / 4))) continue;
+            const int r = nb / (threads / (w / 4));
+            if ((r != 1 && r != 2 && r != 4 && r != 8) || r > R || threads > tiled_max_threads(side, 8, r, c.unroll)) continue;
+            for (int S = 1; S <= kMaxSplit; ++S) {
+                const int Ms = ((len + S - 1) / S + 7) / 8 * 8, used = (len + Ms - 1) / Ms;
+                const double cost = quarter_warps((long)((strip + w - 1) / w) * used, threads) * Ms * r *
+                                    (1 + 0.02 * (h * ht - 1));
+                if (best.Ms == 0 || cost < least)
+                    best = Shape{threads, w, std::min(c.tile, Ms), r, used, Ms, 4}, least = cost;
+            }
+        }
+    return best;
+}
+
+template <typename T>
+static Shape step3_shape(const UpdCfg &c, int strip, int len) {
+    Shape best{c.threads, 32 * c.cpb, c.tile, 0, 0, 0, 4};
+    if constexpr (sizeof(T) == 4) return best;
+    double least = 0;
+    for (int hw = 1; hw <= 2; ++hw)
+        for (int ht = 1; ht <= 2; ++ht)
+            for (int hn = 1; hn <= hw * ht; hn *= 2) {
+                const int w = 32 * c.cpb / hw, th = c.tile / ht, threads = c.threads / hn;
+                if (w < 32 || c.tile % ht || threads % 32 || threads % (w / 4)) continue;
+                const int nrg = threads / (w / 4);
+                if (th % nrg || th / nrg > c.tile * 8 * c.cpb / c.threads) continue;
+                const int rpt = th / nrg, A = rpt % 4 == 0 ? 4 : rpt % 2 == 0 ? 2 : 1;
+                const long blocks = (long)((strip + w - 1) / w) * ((len + th - 1) / th);
+                const double cost = quarter_warps(blocks, threads) * rpt * (1 + 0.02 * (hw * ht - 1));
+                if (least == 0 || cost < least) best = Shape{threads, w, th, 0, 0, 0, A}, least = cost;
+            }
+    return best;
+}
+
+template <typename T, int U, int R>
+static cudaError_t run_step1(int side, const T *X, long ldx, int M, int N, const T *V, long ldv, int nb, const T *Tm,
+                             const Shape &a, T *part, T *fin, unsigned int *tickets, cudaStream_t st) {
+    const size_t smem = sizeof(T) * ((size_t)tiled_w_offset(nb, a.th, a.w) + (size_t)nb * a.w);
+    const dim3 grid(((side == 0 ? N : M) + a.w - 1) / a.w, a.S);
+    static PerDeviceOnce once[2];
+    const auto kern = side == 0 ? left_w_kernel<T, R, U> : right_w_kernel<T, R, U>;
+    allow_max_smem(kern, once[side]);
+    kern<<<grid, a.threads, smem, st>>>(X, ldx, M, N, V, ldv, nb, Tm, a.th, a.w, a.Ms, part, fin, tickets);
     return cudaGetLastError();
 }
 
-template <typename T, int R>
-static cudaError_t run_tiled_u(int side, T *X, long ldx, int M, int N, const T *V, long ldv, int nb, const T *Tm,
-                               const UpdCfg &c, size_t smem, const UpdScratch &sc, cudaStream_t st) {
-    switch (c.unroll) {
-        case 1: return run_tiled<T, R, 1>(side, X, ldx, M, N, V, ldv, nb, Tm, c, smem, sc, st);
-        case 2: return run_tiled<T, R, 2>(side, X, ldx, M, N, V, ldv, nb, Tm, c, smem, sc, st);
-        default: return run_tiled<T, R, 4>(side, X, ldx, M, N, V, ldv, nb, Tm, c, smem, sc, st);
+template <typename T, int U, int A>
+static cudaError_t run_step3(int side, T *X, long ldx, int M, int N, const T *V, long ldv, int nb, const Shape &b,
+                             const T *fin, cudaStream_t st) {
+    const int strip = side == 0 ? N : M, len = side == 0 ? M : N;
+    const dim3 grid((strip + b.w - 1) / b.w, (len + b.th - 1) / b.th);
+    static PerDeviceOnce once[2];
+    const auto kern = side == 0 ? left_x_kernel<T, U, A> : right_x_kernel<T, U, A>;
+    allow_max_smem(kern, once[side]);
+    kern<<<grid, b.threads, tiled_smem(side, (int)sizeof(T), nb, b.th, b.w), st>>>(X, ldx, M, N, V, ldv, nb, b.th, b.w,
+                                                                                   fin);
+    return cudaGetLastError();
+}
+
+template <typename T, int U>
+static cudaError_t run_tiled(int side, T *X, long ldx, int M, int N, const T *V, long ldv, int nb, const T *Tm, int R,
+                             const UpdCfg &c, const UpdScratch &sc, cudaStream_t st) {
+    T *part = reinterpret_cast<T *>(sc.work);
+    T *fin = part + (size_t)kMaxSplit * 64 * std::max(M, N);
+    const int strip = side == 0 ? N : M, len = side == 0 ? M : N;
+    const Shape a = step1_shape<T>(side, nb, R, c, strip, len), b = step3_shape<T>(c, strip, len);
+    const auto step1 = a.R == 1   ? run_step1<T, U, 1>
+                       : a.R == 2 ? run_step1<T, U, 2>
+                       : a.R == 4 ? run_step1<T, U, 4>
+                                  : run_step1<T, U, 8>;
+    cudaError_t e = step1(side, X, ldx, M, N, V, ldv, nb, Tm, a, part, fin, sc.tickets, st);
+    if (e != cudaSuccess) return e;
+    if constexpr (sizeof(T) == 8) {
+        if (b.A == 1) return run_step3<T, U, 1>(side, X, ldx, M, N, V, ldv, nb, b, fin, st);
+        if (b.A == 2) return run_step3<T, U, 2>(side, X, ldx, M, N, V, ldv, nb, b, fin, st);
     }
+    return run_step3<T, U, 4>(side, X, ldx, M, N, V, ldv, nb, b, fin, st);
 }
 
 template <typename T>
@@ -478,11 +560,10 @@ cudaError_t trail_tiled(int side, T *X, long ldx, int M, int N, const T *V, long
     if (!R || !sc.work || !sc.tickets) return cudaErrorInvalidConfiguration;
     const size_t smem = tiled_smem(side, (int)sizeof(T), nb, c.tile, 32 * c.cpb);
     if (smem > kTiledSmemLimit) return cudaErrorInvalidConfiguration;
-    switch (R) {
-        case 1: return run_tiled_u<T, 1>(side, X, ldx, M, N, V, ldv, nb, Tm, c, smem, sc, st);
-        case 2: return run_tiled_u<T, 2>(side, X, ldx, M, N, V, ldv, nb, Tm, c, smem, sc, st);
-        case 4: return run_tiled_u<T, 4>(side, X, ldx, M, N, V, ldv, nb, Tm, c, smem, sc, st);
-        default: return run_tiled_u<T, 8>(side, X, ldx, M, N, V, ldv, nb, Tm, c, smem, sc, st);
+    switch (c.unroll) {
+        case 1: return run_tiled<T, 1>(side, X, ldx, M, N, V, ldv, nb, Tm, R, c, sc, st);
+        case 2: return run_tiled<T, 2>(side, X, ldx, M, N, V, ldv, nb, Tm, R, c, sc, st);
+        default: return run_tiled<T, 4>(side, X, ldx, M, N, V, ldv, nb, Tm, R, c, sc, st);
     }
 }
 
@@ -501,9 +582,14 @@ static int kernel_max_threads(K kernel, bool &known) {
 
 template <typename T, int R, int U>
 static int max_threads_one(int side, bool &known) {
-    if (side == 0)
-        return std::min(kernel_max_threads(left_w_kernel<T, R, U>, known), kernel_max_threads(left_x_kernel<T, U>, known));
-    return std::min(kernel_max_threads(right_w_kernel<T, R, U>, known), kernel_max_threads(right_x_kernel<T, U>, known));
+    const auto w = side == 0 ? left_w_kernel<T, R, U> : right_w_kernel<T, R, U>;
+    int n = std::min(kernel_max_threads(w, known),
+                     kernel_max_threads(side == 0 ? left_x_kernel<T, U, 4> : right_x_kernel<T, U, 4>, known));
+    if constexpr (sizeof(T) == 8) {
+        n = std::min(n, kernel_max_threads(side == 0 ? left_x_kernel<T, U, 2> : right_x_kernel<T, U, 2>, known));
+        n = std::min(n, kernel_max_threads(side == 0 ? left_x_kernel<T, U, 1> : right_x_kernel<T, U, 1>, known));
+    }
+    return n;
 }
 
 template <typename T, int R>

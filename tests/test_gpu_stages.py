@@ -198,3 +198,20 @@ def test_stage1_one_launch_update(nla, m, n, b, pad):
         torch.cuda.synchronize()
         assert int(info.item()) == 0
         assert err_rel(S.double().cpu().numpy(), ref) <= tol_for(1, m)
+
+
+@pytest.mark.parametrize("cfg", [(16, 64, 256, 2, 4), (32, 64, 128, 2, 1), (64, 64, 256, 4, 2), (16, 128, 512, 4, 1),
+                                 (8, 32, 64, 1, 2), (32, 32, 32, 1, 4)])
+@pytest.mark.parametrize("m,n", [(70, 40), (300, 257), (1100, 90), (257, 300)])
+def test_fp64_update_shapes(nla, cfg, m, n):
+    # the FP64 update halves its blocks and splits its sums by the trailing size: 1, 2, 4 and 8
+    # reflectors a thread, tiles of 4, 2 and 1 lines, strips and splits that end raggedly
+    A = np.random.default_rng(m * n + cfg[0]).standard_normal((m, n))
+    if cfg[0] > min(m, n):  # the band is cut to 40, five reflectors a thread: refused
+        with pytest.raises(nla.NLAError):
+            nla.gesvd_vals(to_device_colmajor(A, torch.float64), cfg=nla.Cfg.make(*cfg))
+        return
+    S, info = nla.gesvd_vals(to_device_colmajor(A, torch.float64), cfg=nla.Cfg.make(*cfg))
+    torch.cuda.synchronize()
+    assert int(info.item()) == 0
+    assert err_rel(S.cpu().numpy(), np.linalg.svd(A, compute_uv=False)) <= tol_for(0, max(m, n))
