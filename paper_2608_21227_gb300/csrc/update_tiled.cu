@@ -53,6 +53,18 @@ struct Vec4<double> {
     }
 };
 
+// One element from global to shared memory, asynchronously.
+template <typename T>
+NLA_DEV void cp_async1(T *dst, const T *src) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(sizeof(T)) : "memory");
+}
+NLA_DEV void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+NLA_DEV void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // Swizzled position of X(r, c) in a row-major tile with w columns.
 NLA_DEV int swz(int r, int c, int w) { return r * w + ((((c >> 2) ^ (r & 7))) << 2) + (c & 3); }
 
@@ -62,9 +74,9 @@ size_t tiled_smem(int side, int elem, int nb, int th, int w) {
     (void)side;
     return (size_t)elem * ((size_t)th * w + (size_t)th * (nb + 4) + (size_t)nb * w);
 }
-// Step 1: elements before W (nb x w): the X and V tiles, later T.
+// Step 1: elements before W (nb x w): two X and V tiles, later T.
 __host__ NLA_DEV int tiled_w_offset(int nb, int th, int w) {
-    const int tiles = th * (w + nb + 4), t = (nb * nb + 3) / 4 * 4;
+    const int tiles = 2 * th * (w + nb + 4), t = (nb * nb + 3) / 4 * 4;
     return tiles > t ? tiles : t;
 }
 
@@ -97,7 +109,7 @@ __global__ void left_w_kernel(const T *__restrict__ X, long ldx, int M, int N, c
     __shared__ int sh_last;
     const int ldv_s = nb + 4;
     T *Xs = reinterpret_cast<T *>(smem_raw);  // th x w, swizzled
-    T *Vs = Xs + (size_t)th * w;             // th x (nb+4) row-major
+    T *Vs = Xs + (size_t)2 * th * w;             // th x (nb+4) row-major
     T *Ws = reinterpret_cast<T *>(smem_raw) + tiled_w_offset(nb, th, w);  // nb x w row-major
     const int tid = threadIdx.x, nt = blockDim.x;
     const int ncg = w >> 2, cg = tid % ncg, rg = tid / ncg;
@@ -110,24 +122,45 @@ __global__ void left_w_kernel(const T *__restrict__ X, long ldx, int M, int N, c
     for (int i = 0; i < R; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
-    for (int r0 = rbeg; r0 < rend; r0 += th) {
+    // two half tiles in the room of one: the next lands while this one is multiplied (one block
+    // often holds an SM; 2048 x 2048 FP64 SVD 65.6 -> 63.5 ms)
+    const auto stage = [&](int r0, int buf) {
         const int rows = min(th, rend - r0);
+        T *const xs = Xs + buf * th * w, *const vs = Vs + buf * th * ldv_s;
         for (int idx = tid; idx < th * w; idx += nt) {
-            int r = idx % th, c = idx / th;
-            Xs[swz(r, c, w)] = (r < rows && c < wc) ? X[(r0 + r) + (long)(c0 + c) * ldx] : T(0);
+            const int r = idx % th, c = idx / th;
+            T *const d = xs + swz(r, c, w);
+            if (r < rows && c < wc)
+                cp_async1(d, X + (r0 + r) + (long)(c0 + c) * ldx);
+            else
+                *d = T(0);
         }
         for (int idx = tid; idx < th * nb; idx += nt) {
-            int r = idx % th, k = idx / th, gr = r0 + r;
-            T v = T(0);
-            if (r < rows) v = gr > k ? V[gr + (long)k * ldv] : (gr == k ? T(1) : T(0));
-            Vs[r * ldv_s + k] = v;
+            const int r = idx % th, k = idx / th, gr = r0 + r;
+            T *const d = vs + r * ldv_s + k;
+            if (r < rows && gr > k)
+                cp_async1(d, V + gr + (long)k * ldv);
+            else
+                *d = r < rows && gr == k ? T(1) : T(0);
+        }
+        cp_async_commit();
+    };
+    if (rbeg < rend) stage(rbeg, 0);
+    for (int r0 = rbeg, buf = 0; r0 < rend; r0 += th, buf ^= 1) {
+        const int rows = min(th, rend - r0);
+        if (r0 + th < rend) {
+            stage(r0 + th, buf ^ 1);
+            cp_async_wait<1>();
+        } else {
+            cp_async_wait<0>();
         }
         __syncthreads();
+        const T *const xs = Xs + buf * th * w, *const vs = Vs + buf * th * ldv_s;
 #pragma unroll U
         for (int r = 0; r < rows; ++r) {
             T x[4], v[R];
-            Vec4<T>::ld(Xs + swz(r, 4 * cg, w), x);
-            const T *vr = Vs + r * ldv_s + R * rg;
+            Vec4<T>::ld(xs + swz(r, 4 * cg, w), x);
+            const T *vr = vs + r * ldv_s + R * rg;
             if constexpr (R % 4 == 0) {
 #pragma unroll
                 for (int i = 0; i < R; i += 4) Vec4<T>::ld(vr + i, v + i);
@@ -261,15 +294,17 @@ __global__ void left_x_kernel(T *__restrict__ X, long ldx, int M, int N, const T
 // -------------------------------------------------------------------- LQ side
 // Step 1 (+2): block (rb, s) accumulates Y = X V over columns [s*Ns, (s+1)*Ns)
 // of the h-row strip rb; the last block sums the partials and stores Y' = Y T.
+// (bounds: 64 lines / 4 times 64 reflectors / R, the widest block that a configuration may ask for)
 template <typename T, int R, int U>
-__global__ void right_w_kernel(const T *__restrict__ X, long ldx, int M, int N, const T *__restrict__ Vt, long ldvt,
+__global__ void __launch_bounds__(R < 8 ? 1024 : 512)
+    right_w_kernel(const T *__restrict__ X, long ldx, int M, int N, const T *__restrict__ Vt, long ldvt,
                                int nb, const T *__restrict__ Tm, int th, int h, int Ns, T *part, T *fin,
                                unsigned int *tickets) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int sh_last;
     const int ldv_s = nb + 4;
-    T *Xs = reinterpret_cast<T *>(smem_raw);  // th columns x h rows, column-major
-    T *Vs = Xs + (size_t)th * h;             // th x (nb+4): row c = V(c, :)
+    T *Xs = reinterpret_cast<T *>(smem_raw);  // 2 x th columns x h rows, column-major
+    T *Vs = Xs + (size_t)2 * th * h;             // 2 x th x (nb+4): row c = V(c, :)
     T *Ys = reinterpret_cast<T *>(smem_raw) + tiled_w_offset(nb, th, h);  // nb x h
     const int tid = threadIdx.x, nt = blockDim.x;
     const int ncg = h >> 2, cg = tid % ncg, rg = tid / ncg;
@@ -282,24 +317,42 @@ __global__ void right_w_kernel(const T *__restrict__ X, long ldx, int M, int N, 
     for (int i = 0; i < R; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
-    for (int cb = cbeg; cb < cend; cb += th) {
+    const auto stage = [&](int cb, int buf) {
         const int cols = min(th, cend - cb);
+        T *const xs = Xs + buf * th * h, *const vs = Vs + buf * th * ldv_s;
         for (int idx = tid; idx < th * h; idx += nt) {
-            int i = idx % h, c = idx / h;
-            Xs[c * h + i] = (i < hr && c < cols) ? X[(i0 + i) + (long)(cb + c) * ldx] : T(0);
+            const int i = idx % h, c = idx / h;
+            if (i < hr && c < cols)
+                cp_async1(xs + c * h + i, X + (i0 + i) + (long)(cb + c) * ldx);
+            else
+                xs[c * h + i] = T(0);
         }
         for (int idx = tid; idx < th * nb; idx += nt) {
-            int k = idx % nb, c = idx / nb, gc = cb + c;
-            T v = T(0);
-            if (c < cols) v = gc > k ? Vt[k + (long)gc * ldvt] : (gc == k ? T(1) : T(0));
-            Vs[c * ldv_s + k] = v;
+            const int k = idx % nb, c = idx / nb, gc = cb + c;
+            T *const d = vs + c * ldv_s + k;
+            if (c < cols && gc > k)
+                cp_async1(d, Vt + k + (long)gc * ldvt);
+            else
+                *d = c < cols && gc == k ? T(1) : T(0);
+        }
+        cp_async_commit();
+    };
+    if (cbeg < cend) stage(cbeg, 0);
+    for (int cb = cbeg, buf = 0; cb < cend; cb += th, buf ^= 1) {
+        const int cols = min(th, cend - cb);
+        if (cb + th < cend) {
+            stage(cb + th, buf ^ 1);
+            cp_async_wait<1>();
+        } else {
+            cp_async_wait<0>();
         }
         __syncthreads();
+        const T *const xs = Xs + buf * th * h, *const vs = Vs + buf * th * ldv_s;
 #pragma unroll U
         for (int c = 0; c < cols; ++c) {
             T x[4], v[R];
-            Vec4<T>::ld(Xs + c * h + 4 * cg, x);
-            const T *vc = Vs + c * ldv_s + R * rg;
+            Vec4<T>::ld(xs + c * h + 4 * cg, x);
+            const T *vc = vs + c * ldv_s + R * rg;
             if constexpr (R % 4 == 0) {
 #pragma unroll
                 for (int i = 0; i < R; i += 4) Vec4<T>::ld(vc + i, v + i);
@@ -454,7 +507,7 @@ struct Shape {
 // this count says that more SMs or quarters work.  Step 1 takes the number of splits and their
 // length (whole 64-byte lines) by it too.  A halving has to win 2 %: smaller blocks stage V more
 // often.  FP32 is bound by memory and keeps its tuned blocks and splits.  Updates of a whole
-// reduction, 64 x 64 blocks with three waves of splits before: 2048 x 2048, band 16, 35.9 -> 30.4 ms
+// reduction, 64 x 64 blocks with three waves of splits before: 2048 x 2048, band 16, 35.9 -> 28.3 ms
 // (21.6 at the pipe's rate); 256 x 256, band 32, 1.60 -> 0.70 ms.
 static double quarter_warps(long blocks, int threads) {
     const long sm = device_sm_count();
@@ -511,12 +564,13 @@ static Shape step3_shape(const UpdCfg &c, int strip, int len) {
 template <typename T, int U, int R>
 static cudaError_t run_step1(int side, const T *X, long ldx, int M, int N, const T *V, long ldv, int nb, const T *Tm,
                              const Shape &a, T *part, T *fin, unsigned int *tickets, cudaStream_t st) {
-    const size_t smem = sizeof(T) * ((size_t)tiled_w_offset(nb, a.th, a.w) + (size_t)nb * a.w);
+    const int th = a.th / 2;  // (two tiles in the room of one; a tile is a multiple of 4 lines)
+    const size_t smem = sizeof(T) * ((size_t)tiled_w_offset(nb, th, a.w) + (size_t)nb * a.w);
     const dim3 grid(((side == 0 ? N : M) + a.w - 1) / a.w, a.S);
     static PerDeviceOnce once[2];
     const auto kern = side == 0 ? left_w_kernel<T, R, U> : right_w_kernel<T, R, U>;
     allow_max_smem(kern, once[side]);
-    kern<<<grid, a.threads, smem, st>>>(X, ldx, M, N, V, ldv, nb, Tm, a.th, a.w, a.Ms, part, fin, tickets);
+    kern<<<grid, a.threads, smem, st>>>(X, ldx, M, N, V, ldv, nb, Tm, th, a.w, a.Ms, part, fin, tickets);
     return cudaGetLastError();
 }
 
