@@ -95,6 +95,42 @@ struct Half {
     using T = typename S::Elem;
     static constexpr int B = S::B, LD = S::kLd, LPR = S::LPR, CPT = S::CPT, RPT = S::RPT, GPP = S::GPP, NW = S::NW;
 
+    // A vector whose square leaves the normal range: H = I - m1 m2 u u^T does not depend on the
+    // length of u, so x becomes x 2^-ex with its largest entry in [0.5, 1), and the dot products are
+    // taken again.  False for a zero vector.  (All lanes of a team come here together; every LPR of
+    // them hold all of x.)
+    NLA_DEV static bool scaled_house(T (&x)[CPT], const T (&e)[RPT][CPT], T (&d)[RPT], T alpha, T &beta, T &u0, T &m1,
+                                     T &m2) {
+        m2 = T(0);
+        T mx = fabs(alpha), qt = T(0);
+#pragma unroll
+        for (int i = 0; i < CPT; ++i) mx = fmax(mx, fabs(x[i]));
+#pragma unroll
+        for (int o = 1; o < LPR; o <<= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (mx == T(0)) return false;
+        int ex;
+        frexp(mx, &ex);
+        const T f1 = ldexp(T(1), -(ex / 2)), f2 = ldexp(T(1), -(ex - ex / 2));  // normal numbers both
+#pragma unroll
+        for (int i = 0; i < CPT; ++i) {
+            x[i] = x[i] * f1 * f2;
+            qt = fma(x[i], x[i], qt);
+        }
+#pragma unroll
+        for (int o = 1; o < LPR; o <<= 1) qt += __shfl_xor_sync(0xffffffffu, qt, o);
+#pragma unroll
+        for (int v = 0; v < RPT; ++v) {
+            d[v] = T(0);
+#pragma unroll
+            for (int i = 0; i < CPT; ++i) d[v] = fma(e[v][i], x[i], d[v]);
+#pragma unroll
+            for (int o = 1; o < LPR; o <<= 1) d[v] += __shfl_xor_sync(0xffffffffu, d[v], o);
+        }
+        house(alpha * f1 * f2, qt, beta, u0, m1, m2);
+        beta = beta / f1 / f2;
+        return true;
+    }
+
     // One half step of a team at position k of sweep s: c0 = s + k B + 1 is its first column, sl0 that
     // column's slot in the window (wc slots), L its reflector length.  FAST: every vector and
     // entry exists and, on the right, the B columns do not wrap in the window.
@@ -180,15 +216,19 @@ struct Half {
         T beta, u0, m1, m2;
         if (NW == 1 || ttid < 32) {
             const T qt = __shfl_sync(0xffffffffu, d[0], 0);
-            house(alpha, qt, beta, u0, m1, m2);
-            if (magnitude_bits(qt) == 0u) beta = alpha, u0 = T(0), m1 = T(0), m2 = T(0);
+            beta = alpha, u0 = T(0), m1 = T(0), m2 = T(0);
+            if (!ordinary(fma(alpha, alpha, qt)))
+                m2 = T(1);  // to be scaled first
+            else if (magnitude_bits(qt) != 0u)
+                house(alpha, qt, beta, u0, m1, m2);
         }
         if constexpr (NW > 1) {
             if (ttid == 0) sc[0] = beta, sc[1] = u0, sc[2] = m1, sc[3] = m2;
             asm volatile("bar.sync %0, %1;" ::"r"(barid), "n"(32 * NW) : "memory");
             beta = sc[0], u0 = sc[1], m1 = sc[2], m2 = sc[3];
         }
-        const bool reflect = magnitude_bits(m1) != 0u;
+        bool reflect = magnitude_bits(m1) != 0u;
+        if (!reflect && magnitude_bits(m2) != 0u) reflect = scaled_house(x, e, d, alpha, beta, u0, m1, m2);
         if (p == 0) x[0] = u0;
 #pragma unroll
         for (int v = 0; v < RPT; ++v) {
