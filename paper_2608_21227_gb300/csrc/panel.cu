@@ -585,18 +585,14 @@ NLA_DEV void panel_scalars(float alpha, float xn2, float &beta, float &tau, floa
 }
 NLA_DEV void panel_scalars(double alpha, double xn2, double &beta, double &tau, double &scale) {
     const double q = fma(alpha, alpha, xn2);
-    if (!ordinary(q)) {  // (g below would overflow; tau and the scale do not)
-        const double r = sqrt(q);
-        beta = alpha >= 0.0 ? -r : r;
-        tau = (beta - alpha) / beta;
-        scale = 1.0 / (alpha - beta);
+    if (ordinary(q)) {
+        house_tau(alpha, xn2, beta, tau, scale);
         return;
     }
-    double u0, g, one;
-    house(alpha, xn2, beta, u0, g, one);  // g = 1 / (|beta| |u0|)
-    const double ug = u0 * g;             // +-1 / |beta|
-    tau = u0 * ug;
-    scale = g * -beta;  // sign(u0) = -sign(beta)
+    const double r = sqrt(q);
+    beta = alpha >= 0.0 ? -r : r;
+    tau = (beta - alpha) / beta;
+    scale = 1.0 / (alpha - beta);
 }
 
 template <typename T, int NB, int R>

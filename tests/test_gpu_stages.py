@@ -215,3 +215,22 @@ def test_fp64_update_shapes(nla, cfg, m, n):
     torch.cuda.synchronize()
     assert int(info.item()) == 0
     assert err_rel(S.cpu().numpy(), np.linalg.svd(A, compute_uv=False)) <= tol_for(0, max(m, n))
+
+
+@pytest.mark.parametrize("b", [16, 32])
+def test_fp64_panel_reflectors_are_orthogonal(nla, b):
+    # tau (1 + |v|^2) / 2 = 1 for the stored reflectors.  In units u = 2^-53, rounding independently to
+    # nearest: v's entries and their scale, the norm, its root, the sum in tau and tau itself leave
+    # about 0.8 u (rms) for 9 to 24 entries, whatever the method; a scalar that loses a bit shows as
+    # 1.9 u.  1.2 u lies between.
+    m, bad = b + 8, []
+    for seed in range(40):
+        t = to_device_colmajor(np.random.default_rng(seed).standard_normal((m, b)), torch.float64)
+        tauq, _, info = nla.gebrd_band(t, b)
+        A, tau = from_device_colmajor(t), tauq.cpu().numpy()
+        for j in range(b):
+            if m - j - 1 < 24:
+                v = A[j + 1:, j].astype(np.longdouble)
+                bad.append(float(tau[j] * (1 + v @ v) / 2 - 1) * 2.0 ** 53)
+    assert int(info.item()) == 0
+    assert np.sqrt(np.mean(np.square(bad))) <= 1.2
