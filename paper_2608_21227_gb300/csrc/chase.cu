@@ -95,40 +95,56 @@ struct Half {
     using T = typename S::Elem;
     static constexpr int B = S::B, LD = S::kLd, LPR = S::LPR, CPT = S::CPT, RPT = S::RPT, GPP = S::GPP, NW = S::NW;
 
-    // A vector whose square leaves the normal range: H = I - m1 m2 u u^T does not depend on the
-    // length of u, so x becomes x 2^-ex with its largest entry in [0.5, 1), and the dot products are
-    // taken again.  False for a zero vector.  (All lanes of a team come here together; every LPR of
-    // them hold all of x.)
-    NLA_DEV static bool scaled_house(T (&x)[CPT], const T (&e)[RPT][CPT], T (&d)[RPT], T alpha, T &beta, T &u0, T &m1,
-                                     T &m2) {
-        m2 = T(0);
-        T mx = fabs(alpha), qt = T(0);
-#pragma unroll
-        for (int i = 0; i < CPT; ++i) mx = fmax(mx, fabs(x[i]));
-#pragma unroll
-        for (int o = 1; o < LPR; o <<= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        if (mx == T(0)) return false;
-        int ex;
-        frexp(mx, &ex);
-        const T f1 = ldexp(T(1), -(ex / 2)), f2 = ldexp(T(1), -(ex - ex / 2));  // normal numbers both
-#pragma unroll
-        for (int i = 0; i < CPT; ++i) {
-            x[i] = x[i] * f1 * f2;
-            qt = fma(x[i], x[i], qt);
+    // The half step where the vector's square leaves the normal range: H = I - m1 m2 u u^T does not
+    // depend on the length of u, so x becomes x 2^-ex with its largest entry in [0.5, 1).  Rare, so
+    // plain: a thread per vector, straight from shared memory, and out of line (inside the step
+    // it took registers and 1 to 2 % of every step).
+    template <bool RIGHT>
+    __device__ __noinline__ static void scaled(T *win, int wc, int sl0, int n, int s, int k, int c0, int L, T *team,
+                                               int ttid, int barid) {
+        const auto sync = [&] {
+            if (NW == 1)
+                __syncwarp();
+            else
+                asm volatile("bar.sync %0, %1;" ::"r"(barid), "n"(32 * NW) : "memory");
+        };
+        sync();  // what the team left in the buffer for the next half is written again below
+        const int tr = k == 0 ? s : c0 - B;
+        const int nvec = RIGHT ? c0 + L - tr : min(c0 + 2 * B, n) - c0;
+        const auto at = [&](int g, int c) -> T & {  // entry c of vector g
+            const int w = RIGHT ? c : g;
+            const int sl = sl0 + w - (sl0 + w >= wc ? wc : 0);
+            return win[sl * LD + 2 * B + (RIGHT ? tr + g - c0 - c : c - g)];
+        };
+        const T *const buf = RIGHT ? team : team + B;
+        const bool first = RIGHT && k == 0;  // the sweep starts: x is still in the window
+        const auto x = [&](int i) { return first ? at(0, i) : buf[i]; };
+        T mx = T(0);
+        for (int i = 0; i < L; ++i) mx = fmax(mx, fabs(x(i)));
+        T beta = T(0), u0 = T(0), m1 = T(0), m2 = T(0), f1 = T(1), f2 = T(1);
+        if (mx > T(0)) {
+            int ex;
+            frexp(mx, &ex);
+            f1 = ldexp(T(1), -(ex / 2)), f2 = ldexp(T(1), -(ex - ex / 2));  // normal numbers both
+            T qt = T(0);
+            for (int i = 1; i < L; ++i) qt = fma(x(i) * f1 * f2, x(i) * f1 * f2, qt);
+            house(x(0) * f1 * f2, qt, beta, u0, m1, m2);
+            beta = beta / f1 / f2;
         }
-#pragma unroll
-        for (int o = 1; o < LPR; o <<= 1) qt += __shfl_xor_sync(0xffffffffu, qt, o);
-#pragma unroll
-        for (int v = 0; v < RPT; ++v) {
-            d[v] = T(0);
-#pragma unroll
-            for (int i = 0; i < CPT; ++i) d[v] = fma(e[v][i], x[i], d[v]);
-#pragma unroll
-            for (int o = 1; o < LPR; o <<= 1) d[v] += __shfl_xor_sync(0xffffffffu, d[v], o);
+        for (int g = ttid; g < nvec; g += 32 * NW) {
+            if (g > 0 && mx > T(0)) {
+                T d = u0 * at(g, 0);
+                for (int i = 1; i < L; ++i) d = fma(x(i) * f1 * f2, at(g, i), d);
+                const T w = d * m1 * m2;
+                at(g, 0) = fma(-w, u0, at(g, 0));
+                for (int i = 1; i < L; ++i) at(g, i) = fma(-w, x(i) * f1 * f2, at(g, i));
+            }
+            const int o = RIGHT ? g - (c0 - tr) : g - B;
+            if (o >= 0) (RIGHT ? team + B : team)[o] = at(g, 0);
         }
-        house(alpha * f1 * f2, qt, beta, u0, m1, m2);
-        beta = beta / f1 / f2;
-        return true;
+        sync();
+        if (ttid == 0 && mx > T(0))  // (x may have been vector 0 itself until here)
+            for (int i = 0; i < L; ++i) at(0, i) = i == 0 ? beta : T(0);
     }
 
     // One half step of a team at position k of sweep s: c0 = s + k B + 1 is its first column, sl0 that
@@ -212,23 +228,22 @@ struct Half {
             for (int o = 1; o < LPR; o <<= 1) d[v] += __shfl_xor_sync(0xffffffffu, d[v], o);
             first[v] = LPR == 1 ? e[v][0] : __shfl_sync(0xffffffffu, e[v][0], lane & ~(LPR - 1));
         }
-        // ---- scalars (by the warp that holds vector 0); a zero tail: H = I
+        // ---- scalars (by the warp that holds vector 0)
         T beta, u0, m1, m2;
         if (NW == 1 || ttid < 32) {
             const T qt = __shfl_sync(0xffffffffu, d[0], 0);
-            beta = alpha, u0 = T(0), m1 = T(0), m2 = T(0);
-            if (!ordinary(fma(alpha, alpha, qt)))
-                m2 = T(1);  // to be scaled first
-            else if (magnitude_bits(qt) != 0u)
-                house(alpha, qt, beta, u0, m1, m2);
+            house(alpha, qt, beta, u0, m1, m2);
+            // a zero tail: H = I; m2 without m1: the vector has to be scaled first (by selects: a branch
+            // would lengthen the chain)
+            const bool fits = ordinary(fma(alpha, alpha, qt));
+            if (magnitude_bits(qt) == 0u || !fits) beta = alpha, u0 = T(0), m1 = T(0), m2 = fits ? T(0) : T(1);
         }
         if constexpr (NW > 1) {
             if (ttid == 0) sc[0] = beta, sc[1] = u0, sc[2] = m1, sc[3] = m2;
             asm volatile("bar.sync %0, %1;" ::"r"(barid), "n"(32 * NW) : "memory");
             beta = sc[0], u0 = sc[1], m1 = sc[2], m2 = sc[3];
         }
-        bool reflect = magnitude_bits(m1) != 0u;
-        if (!reflect && magnitude_bits(m2) != 0u) reflect = scaled_house(x, e, d, alpha, beta, u0, m1, m2);
+        const bool reflect = magnitude_bits(m1) != 0u, rescale = !reflect && magnitude_bits(m2) != 0u;
         if (p == 0) x[0] = u0;
 #pragma unroll
         for (int v = 0; v < RPT; ++v) {
@@ -238,7 +253,7 @@ struct Half {
 #pragma unroll
             for (int i = 0; i < CPT; ++i) e[v][i] = fma(-w, x[i], e[v][i]);
             // (vector 0 becomes beta e1 below)
-            const bool own = (v > 0 || g0 > 0 || !reflect) && (FAST || gi < nvec);
+            const bool own = (v > 0 || g0 > 0 || !reflect) && (FAST || gi < nvec) && !rescale;
 #pragma unroll
             for (int i = 0; i < CPT; ++i)
                 if (own && (FAST || p + LPR * i < L)) at(v, i) = e[v][i];
@@ -256,6 +271,7 @@ struct Half {
                 *at0 = c == 0 ? beta : T(0);
             }
         }
+        if (__builtin_expect(rescale, 0)) scaled<RIGHT>(win, wc, sl0, n, s, k, c0, L, team, ttid, barid);
     }
 };
 
