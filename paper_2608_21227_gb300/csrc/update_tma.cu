@@ -294,9 +294,11 @@ qr_proj_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
 // FP32 accuracy from TF32 operands by the three-term split x = hi + lo: of X, hi = x with the
 // low 13 mantissa bits cleared (what the tensor core reads of an FP32 word); of V, hi is x
 // rounded to TF32, so that the dropped lo_x lo_v has no preferred sign; lo = x - hi (exact)
-// rounded to TF32: x . v ~ hi_x hi_v + hi_x lo_v + lo_x hi_v to 2^-22 relative.  The
-// first two products are one MMA against [V_hi; V_lo] (N = 2 NB, the hi copy of X
-// read once), the third a second MMA (N = NB) onto the columns of the other small product.
+// rounded to TF32: x . v ~ hi_x hi_v + hi_x lo_v + lo_x hi_v to 2^-22 relative.  Three
+// MMAs of one shape (N = NB) per K step: hi_x hi_v onto one accumulator, the two small products
+// onto another.  (The order of MMAs on the same columns is only promised for the same accumulator
+// and shape, so hi_x [V_hi; V_lo] as one MMA of 2 NB columns, which would read the hi copy of X
+// once, cannot share its second half with lo_x hi_v; 8192 x 8192 takes 110.6 ms, 110.9 with it.)
 // The tensor core rounds its accumulator toward zero, which shrinks W in proportion to the
 // number of MMAs summed one after another and with it, over the steps, every singular value
 // (-2.7e-8 of sigma_1 per MMA in the chain, 3.5e-6 at 8,192 rows).  So the K steps take turns on
@@ -378,9 +380,7 @@ qr_proj_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            // V_lo lies right after V_hi (NB rows of 128 bytes each): [V_hi; V_lo] is one B
-            // operand of 2 NB rows, so the hi copy of X is read once per K step
-            const uint32_t id2 = tc::idesc(2, 128, 2 * NB), id1 = tc::idesc(2, 128, NB);
+            const uint32_t id = tc::idesc(2, 128, NB);
             for (int t = 0; t < nt; ++t) {
                 const int st = t % S;
                 if (*(volatile int *)&sh_abort || !tc::mbar_wait(&conv[st], (uint32_t)((t / S) & 1), info)) {
@@ -389,12 +389,14 @@ qr_proj_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
                 }
                 tc::fence_after_sync();
                 const uint32_t ah = tc::smem_u32(xhi(st)), al = tc::smem_u32(xlo(st));
-                const uint32_t bh = tc::smem_u32(vhi(st));
+                const uint32_t bh = tc::smem_u32(vhi(st)), bl = tc::smem_u32(vlo(st));
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {  // 8 TF32 = 32 bytes of K per instruction
                     const uint32_t off = kk * 32, step = 4 * t + kk, d = tbase + step % kSets * 2 * NB;
-                    tc::mma_tf32(d, tc::sdesc_sw128(ah + off), tc::sdesc_sw128(bh + off), id2, step >= kSets ? 1u : 0u);
-                    tc::mma_tf32(d + NB, tc::sdesc_sw128(al + off), tc::sdesc_sw128(bh + off), id1, 1u);
+                    const uint32_t acc = step >= kSets ? 1u : 0u;
+                    tc::mma_tf32(d, tc::sdesc_sw128(ah + off), tc::sdesc_sw128(bh + off), id, acc);
+                    tc::mma_tf32(d + NB, tc::sdesc_sw128(ah + off), tc::sdesc_sw128(bl + off), id, acc);
+                    tc::mma_tf32(d + NB, tc::sdesc_sw128(al + off), tc::sdesc_sw128(bh + off), id, 1u);
                 }
                 tc::mma_commit(&empty[st]);  // the stage is free once these MMAs have read it
             }
@@ -688,9 +690,9 @@ lq_proj_tm_kernel(const __grid_constant__ CUtensorMap tmX, int M, int N, const f
     constexpr int H = 128;                            // rows per block = the MMA's M
     constexpr int kX = 4 * kLqXBox;                   // the stage's 128 rows
     constexpr int kB = NB * 128;                      // V^T of the stage's 32 columns (hi or lo)
-    // At NB = 16 the accumulators are laid out like qr_proj_tc's (A_hi [V_hi; V_lo] and A_lo V_hi
-    // onto its second half: two MMAs per K step); the wider forms take three MMAs onto NB columns
-    // (the split one would not leave room for three slots).  Against the accumulator's rounding
+    // At NB = 16 the accumulators are laid out like qr_proj_tc's (A_hi V_hi, and A_hi V_lo + A_lo V_hi);
+    // the wider forms sum all three products on NB columns (the split one would not leave room for
+    // three slots).  Against the accumulator's rounding
     // (qr_proj_tc) only two accumulators fit beside the slots, so blocks of kBlk stages take turns on
     // them and the converters add a finished block's to FP32 sums in registers: its MMAs are known to
     // have completed when they get the operand slot of the stage two after it, and the next block
@@ -759,7 +761,7 @@ lq_proj_tm_kernel(const __grid_constant__ CUtensorMap tmX, int M, int N, const f
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            const uint32_t id = tc::idesc(2, 128, NB), id2 = tc::idesc(2, 128, 2 * NB);
+            const uint32_t id = tc::idesc(2, 128, NB);
             for (int t = 0; t < nt; ++t) {
                 const int o = t % kLqStages;
                 if (*(volatile int *)&sh_abort || !tc::mbar_wait(&conv[o], (uint32_t)((t / kLqStages) & 1), info)) {
@@ -773,14 +775,10 @@ lq_proj_tm_kernel(const __grid_constant__ CUtensorMap tmX, int M, int N, const f
                 for (int kk = 0; kk < kLqCols / 8; ++kk) {  // 8 columns per instruction
                     const uint32_t off = kk * 32, acc = t % kBlk > 0 || kk > 0 ? 1u : 0u;
                     const uint32_t d = tbase + (uint32_t)(t / kBlk) % kSets * kSetStep;
-                    if constexpr (kStack) {  // B lo lies right after B hi: [V_hi; V_lo] is one operand
-                        tc::mma_tf32_tmem_a(d, ah + 8 * kk, tc::sdesc_sw128(bh + off), id2, acc);
-                        tc::mma_tf32_tmem_a(d + NB, al + 8 * kk, tc::sdesc_sw128(bh + off), id, 1u);
-                    } else {
-                        tc::mma_tf32_tmem_a(d, ah + 8 * kk, tc::sdesc_sw128(bh + off), id, acc);
-                        tc::mma_tf32_tmem_a(d, ah + 8 * kk, tc::sdesc_sw128(bl + off), id, 1u);
-                        tc::mma_tf32_tmem_a(d, al + 8 * kk, tc::sdesc_sw128(bh + off), id, 1u);
-                    }
+                    const uint32_t ds = kStack ? d + NB : d, accs = kStack ? acc : 1u;  // the small products'
+                    tc::mma_tf32_tmem_a(d, ah + 8 * kk, tc::sdesc_sw128(bh + off), id, acc);
+                    tc::mma_tf32_tmem_a(ds, ah + 8 * kk, tc::sdesc_sw128(bl + off), id, accs);
+                    tc::mma_tf32_tmem_a(ds, al + 8 * kk, tc::sdesc_sw128(bh + off), id, 1u);
                 }
                 tc::mma_commit(&ofree[o]);  // the operand slot is free once these MMAs have read it
             }

@@ -88,3 +88,51 @@ print("ok")
     r = subprocess.run([sys.executable, "-c", child, ROOT], env=dict(os.environ, **env), capture_output=True, text=True,
                        timeout=300)
     assert r.returncode == 0 and r.stdout.strip().endswith("ok"), r.stderr[-2000:]
+
+
+# The switches on shapes and configurations that do reach what they switch: with the update's parameters named, the
+# two-kernel FP32 update runs (leading dimensions of whole 16 bytes) at bands 16, 32 and 64, over enough columns to
+# go round its accumulators.
+TWO_KERNEL_CHILD = r"""
+import json, sys
+import numpy as np, torch
+sys.path.insert(0, sys.argv[1]); sys.path.insert(0, sys.argv[1] + "/tests")
+from paper_2608_21227_gb300 import nla
+from _util import err_rel, tol_for
+out = []
+for (m, n, b) in [(1100, 900, 16), (1032, 1000, 32), (1064, 1064, 64), (2100, 300, 16), (700, 650, 32)]:
+    A = np.random.default_rng(m + n + b).standard_normal((m, n)).astype(np.float32)
+    t = torch.from_numpy(np.ascontiguousarray(A.T)).cuda()
+    S, info = nla.gesvd_vals(t, cfg=nla.Cfg.make(*nla.plan_cfg(m, n, nla.F32, cfg=nla.Cfg.make(band=b))))
+    torch.cuda.synchronize()
+    e = err_rel(S.double().cpu().numpy(), np.linalg.svd(A.astype(np.float64), compute_uv=False))
+    out.append({"m": m, "n": n, "b": b, "info": int(info.item()), "err": e, "tol": tol_for(1, max(m, n)),
+                "values": S.cpu().numpy().tolist()})
+print(json.dumps(out))
+"""
+
+
+def _two_kernel(env):
+    r = subprocess.run([sys.executable, "-c", TWO_KERNEL_CHILD, ROOT], env=dict(os.environ, **env), capture_output=True,
+                       text=True, timeout=600)
+    assert r.returncode == 0, r.stderr[-2000:]
+    out = json.loads(r.stdout.strip().splitlines()[-1])
+    for rec in out:
+        assert rec["info"] == 0 and rec["err"] <= rec["tol"], {k: v for k, v in rec.items() if k != "values"}
+    return [rec["values"] for rec in out]
+
+
+@pytest.fixture(scope="module")
+def two_kernel_default():
+    return _two_kernel({})
+
+
+@pytest.mark.parametrize("mask", ["0", "1", "2"])
+def test_two_kernel_update_projections(two_kernel_default, mask):
+    # other sums, so other last digits: the switch has an effect on every shape
+    for a, b in zip(_two_kernel({"NLA_PROJ_TC": mask}), two_kernel_default):
+        assert a != b
+
+
+def test_two_kernel_update_in_plain_stream_order(two_kernel_default):
+    assert _two_kernel({"NLA_PDL": "0"}) == two_kernel_default
