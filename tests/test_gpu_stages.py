@@ -234,3 +234,41 @@ def test_fp64_panel_reflectors_are_orthogonal(nla, b):
                 bad.append(float(tau[j] * (1 + v @ v) / 2 - 1) * 2.0 ** 53)
     assert int(info.item()) == 0
     assert np.sqrt(np.mean(np.square(bad))) <= 1.2
+
+
+# The tensor core rounds its accumulator toward zero: -2.7e-8 of sigma_1 per MMA that a projection
+# sums one after another, on each side.  2,100 x 2,000 in 8 splits of 264: 33 K steps on 8 / 4 / 2
+# accumulators (band 16 / 32 / 64) on the QR side; on the LQ side blocks of 16 steps, of 48 MMAs at
+# band 32 and 99 of one split at band 64.  With 3e-7 for the unbiased rounding: 1.0e-6, 1.9e-6,
+# 3.5e-6.  (One accumulator a side at band 16 is 66 MMAs: 2.1e-6.)
+@pytest.mark.parametrize("b,tol", [(16, 1.0e-6), (32, 1.9e-6), (64, 3.5e-6)])
+def test_fp32_two_kernel_update_accuracy(nla, b, tol):
+    A = np.random.default_rng(b).uniform(-1.0, 1.0, (2100, 2000)).astype(np.float32)
+    cfg = nla.Cfg.make(*nla.plan_cfg(2100, 2000, nla.F32, cfg=nla.Cfg.make(band=b)))  # named: no one-launch update
+    t = to_device_colmajor(A, torch.float32)
+    S, info = nla.gesvd_vals(t, cfg=cfg, preserve_a=True)
+    again, _ = nla.gesvd_vals(t, cfg=cfg, preserve_a=True)
+    torch.cuda.synchronize()
+    assert int(info.item()) == 0
+    assert torch.equal(S, again)
+    assert err_rel(S.double().cpu().numpy(), np.linalg.svd(A.astype(np.float64), compute_uv=False)) <= tol
+
+
+@pytest.mark.parametrize("m,n,b,pad", [(1100, 900, 16, 0), (1101, 901, 16, 1), (1700, 1500, 16, 0), (1701, 1503, 16, 2),
+                                       (900, 800, 32, 0), (640, 30, 16, 0)])
+def test_one_launch_update_is_taken(nla, m, n, b, pad):
+    # more trailing columns than SMs hold at 4 and at 8 a block (4 x 152, 8 x 152), so that the QR side
+    # takes 8 and 16 lines a strip; the same configuration by name turns the one-launch update off, and
+    # sums in another order
+    A = np.random.default_rng(m + n).standard_normal((m, n)).astype(np.float32)
+    buf = torch.zeros(n, m + pad, device="cuda")
+    buf[:, :m] = torch.from_numpy(np.ascontiguousarray(A.T)).cuda()
+    ref = np.linalg.svd(A.astype(np.float64), compute_uv=False)
+    out = []
+    for c in (nla.Cfg.make(band=b), nla.Cfg.make(*nla.plan_cfg(m, n, nla.F32, cfg=nla.Cfg.make(band=b)))):
+        S, info = nla.gesvd_vals(buf.clone()[:, :m], cfg=c)  # (in place: the leading dimension is the caller's)
+        torch.cuda.synchronize()
+        assert int(info.item()) == 0
+        assert err_rel(S.double().cpu().numpy(), ref) <= tol_for(1, m)
+        out.append(S)
+    assert not torch.equal(out[0], out[1])
