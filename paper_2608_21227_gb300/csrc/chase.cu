@@ -312,9 +312,9 @@ NLA_DEV void copy_columns(typename S::Elem *win, int wc, typename S::Elem *AB, l
 // timeout raises sh_abort, which the teams act on together.
 constexpr int kChunkBars = 64;  // > chunks a window can hold
 
-template <class S>
+template <class S, bool BULK>
 __global__ void __launch_bounds__(32 * (S::kMaxWarps + 3))
-chase_kernel(typename S::Elem *AB, long ldab, int n, int G, int wc, int bulk, int *done, int *info) {
+chase_kernel(typename S::Elem *AB, long ldab, int n, int G, int wc, int *done, int *info) {
     using T = typename S::Elem;
     constexpr int B = S::B, NW = S::NW, LD = S::kLd;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -331,6 +331,18 @@ chase_kernel(typename S::Elem *AB, long ldab, int n, int G, int wc, int bulk, in
         *vabort = 1;
         return false;
     };
+    // A mover's view of a shared word.  With bulk copies one lane moves the columns; without them the
+    // whole warp does and meets in warp-wide operations, so all lanes act on lane 0's value, and on
+    // what was written before it (fence, then the warp barrier).
+    const auto seen = [&](volatile int *word) {
+        int v = *word;
+        if (!BULK) {
+            __threadfence_block();
+            __syncwarp();
+            v = __shfl_sync(0xffffffffu, v, 0);
+        }
+        return v;
+    };
     uint32_t chunk0 = 0;  // chunks of this block's earlier groups: chunk m uses barrier (chunk0 + m) % kChunkBars
     if (tid == 0) {
         sh_abort = 0;
@@ -338,6 +350,7 @@ chase_kernel(typename S::Elem *AB, long ldab, int n, int G, int wc, int bulk, in
         for (int i = 0; i < kChunkBars; ++i) tc::mbar_init(&cbar[i], 1);
         tma::fence_init();
     }
+    __syncthreads();
     for (int grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {
         const int s0 = grp * G, g = min(G, nsweeps - s0);
         const int lo0 = s0 + 1;                    // first column of the group
@@ -349,8 +362,7 @@ chase_kernel(typename S::Elem *AB, long ldab, int n, int G, int wc, int bulk, in
             sh_tau = 0;
             sh_fl = lo0 - 1;
         }
-        __syncthreads();
-        if (*vabort) break;
+        if (__syncthreads_or(*vabort)) break;  // (the same way for every thread)
         if (warp < G * NW) {
             // ---------------- teams
             const int it = warp / NW, ttid = tid - it * 32 * NW, s = s0 + it;
@@ -420,11 +432,11 @@ chase_kernel(typename S::Elem *AB, long ldab, int n, int G, int wc, int bulk, in
             }
         } else if (warp == G * NW + 1) {
             // ---------------- flusher (one lane with bulk copies, the whole warp without)
-            if (!bulk || lane == 0) {
+            if (!BULK || lane == 0) {
                 int flushed = lo0 - 1;
                 for (;;) {
-                    if (*vabort) break;
-                    const int t = *vtau;  // steps < t are complete
+                    if (seen(vabort)) break;
+                    const int t = seen(vtau);  // steps < t are complete
                     __threadfence_block();
                     // columns <= fin are final: the last started sweep is the lowest, and a sweep that
                     // has not started will start one column further on
@@ -436,7 +448,7 @@ chase_kernel(typename S::Elem *AB, long ldab, int n, int G, int wc, int bulk, in
                     }
                     if (fin > flushed) {
                         const int j0 = flushed + 1;
-                        if (bulk) {
+                        if (BULK) {
                             fence_async_all();  // the teams' writes precede the copies' reads
                             const int sl = j0 % wc, k1 = min(fin - flushed, wc - sl), k2 = fin - flushed - k1;
                             bulk_store(AB + (long)j0 * LD, win + (size_t)sl * LD, (uint32_t)(k1 * LD * sizeof(T)));
@@ -454,6 +466,7 @@ chase_kernel(typename S::Elem *AB, long ldab, int n, int G, int wc, int bulk, in
                             st_release(&done[grp], t < ntau ? flushed + 1 : INT_MAX);
                             *vfl = flushed;  // the loader may reuse these slots now
                         }
+                        if (!BULK) __syncwarp();
                     }
                     if (t >= ntau) break;
                 }
@@ -461,24 +474,24 @@ chase_kernel(typename S::Elem *AB, long ldab, int n, int G, int wc, int bulk, in
             __syncwarp();
         } else {
             // ---------------- loader
-            if (!bulk || lane == 0) {
+            if (!BULK || lane == 0) {
                 int have = grp > 0 ? 0 : INT_MAX;  // columns < have are final in the previous group
                 int m = 0;
-                for (; m < nch && !*vabort;) {
+                for (; m < nch && !seen(vabort);) {
                     const int j0 = lo0 + m * B, cnt = min(B, n - j0);
                     if (j0 + cnt > have) {
                         // every lane acquires, so that its own copies see what the previous group
                         // wrote; the smallest value seen is final for all of them
                         have = ld_acquire(&done[grp - 1]);
-                        if (!bulk) have = __reduce_min_sync(0xffffffffu, have);
+                        if (!BULK) have = __reduce_min_sync(0xffffffffu, have);
                         fence_async_all();  // what was acquired precedes the copies' reads
                         continue;
                     }
-                    if (j0 + cnt - 1 > *vfl + wc) continue;  // no room in the window yet
+                    if (j0 + cnt - 1 > seen(vfl) + wc) continue;  // no room in the window yet
                     __threadfence_block();
                     const uint32_t c = chunk0 + m;
                     uint64_t *bar = &cbar[c % kChunkBars];
-                    if (bulk) {
+                    if (BULK) {
                         fence_async_all();  // the slots' earlier reads and writes precede the copies
                         const int sl = j0 % wc, k1 = min(cnt, wc - sl), k2 = cnt - k1;
                         tma::expect_tx(bar, (uint32_t)(cnt * LD * sizeof(T)));
@@ -518,11 +531,13 @@ __global__ void repack_kernel(const T *__restrict__ src, long lds, T *__restrict
 template <class S>
 cudaError_t launch(typename S::Elem *AB, long ldab, int n, int gmax, int *done, int *info, cudaStream_t st) {
     using T = typename S::Elem;
-    auto kern = chase_kernel<S>;
     constexpr size_t kBudget = 220 * 1024;
+    const bool bulk = ldab == S::kLd && reinterpret_cast<uintptr_t>(AB) % 16 == 0;
+    const auto kern = bulk ? chase_kernel<S, true> : chase_kernel<S, false>;
     static PerDeviceOnce attr;
-    attr.run([&] {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBudget);
+    attr.run([] {
+        cudaFuncSetAttribute(chase_kernel<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBudget);
+        cudaFuncSetAttribute(chase_kernel<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBudget);
         cudaGetLastError();
     });
     const size_t col = (size_t)S::kLd * sizeof(T);
@@ -542,7 +557,6 @@ cudaError_t launch(typename S::Elem *AB, long ldab, int n, int gmax, int *done, 
     cudaError_t err = cudaMemsetAsync(done, 0, sizeof(int) * (size_t)ngroups, st);
     if (err != cudaSuccess) return err;
     const int wc = (kLag * G - 1) * S::B + G + 1 + pf * S::B;
-    const int bulk = ldab == S::kLd && reinterpret_cast<uintptr_t>(AB) % 16 == 0 ? 1 : 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(std::min(ngroups, device_sm_count()));
     cfg.blockDim = dim3(32 * (G * S::NW + 3));
@@ -553,7 +567,7 @@ cudaError_t launch(typename S::Elem *AB, long ldab, int n, int gmax, int *done, 
     at[0].val.cooperative = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, AB, ldab, n, G, wc, bulk, done, info);
+    return cudaLaunchKernelEx(&cfg, kern, AB, ldab, n, G, wc, done, info);
 }
 
 }  // namespace

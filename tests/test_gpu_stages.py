@@ -272,3 +272,40 @@ def test_one_launch_update_is_taken(nla, m, n, b, pad):
         assert err_rel(S.double().cpu().numpy(), ref) <= tol_for(1, m)
         out.append(S)
     assert not torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("dt", [0, 1])
+@pytest.mark.parametrize("n,b", [(700, 8), (1500, 16), (900, 32), (600, 64), (900, 24), (400, 5)])
+def test_chase_storage_forms_agree(nla, dt, n, b):
+    # the same chase whether columns move as bulk copies (packed), element by element (a workspace of
+    # counters only, no workspace at all, other leading dimensions), and every time: d and e bit for bit
+    import ctypes
+
+    i, j = np.indices((n, n))
+    D = np.where((j - i >= 0) & (j - i <= b), np.random.default_rng(n + b).standard_normal((n, n)), 0.0)
+    tdt = torch.float64 if dt == 0 else torch.float32
+    L, st = nla.lib(), torch.cuda.current_stream().cuda_stream
+    vp = ctypes.c_void_p
+    L.nla_band2bd_noalloc.argtypes = [ctypes.c_int] * 3 + [vp, ctypes.c_int, vp, vp, vp, vp]
+    need = ctypes.c_size_t(0)
+    assert L.nla_band2bd_workspace(n, b, dt, ctypes.byref(need)) == 0
+    AB0 = nla.band_extract(to_device_colmajor(D, tdt), b)
+    results = []
+    for ldab, work_bytes in [(3 * b + 1, need.value), (3 * b + 1, 4 * n), (3 * b + 7, 4 * n), (3 * b + 1, None)] * 2:
+        AB = torch.zeros(n, ldab, dtype=tdt, device="cuda")
+        AB[:, :3 * b + 1] = AB0[:, :3 * b + 1]
+        d = torch.zeros(n, dtype=torch.float64, device="cuda")
+        e = torch.zeros(n, dtype=torch.float64, device="cuda")
+        info = torch.zeros(1, dtype=torch.int32, device="cuda")
+        args = (n, b, dt, AB.data_ptr(), ldab, d.data_ptr(), e.data_ptr())
+        if work_bytes is None:
+            assert L.nla_band2bd_noalloc(*args, info.data_ptr(), st) == 0
+        else:
+            work = torch.empty(max(work_bytes, 256), dtype=torch.uint8, device="cuda")
+            assert L.nla_band2bd(*args, work.data_ptr(), work_bytes, info.data_ptr(), None, st) == 0
+        torch.cuda.synchronize()
+        assert int(info.item()) == 0
+        results.append((d, e[:n - 1]))
+    for d, e in results[1:]:
+        assert torch.equal(d, results[0][0]) and torch.equal(e, results[0][1])
+    assert err_rel(oracle.bdsvd(d.cpu().numpy(), e.cpu().numpy()), np.linalg.svd(D, compute_uv=False)) <= tol_for(dt, n)
