@@ -444,8 +444,9 @@ NLA_DEV bool wait_loaded(volatile int *sh_hi, int hi, volatile int *sh_abort, in
 template <typename T>
 __global__ void band2bd_group_kernel(T *AB, long ldab, int n, int b, int G, int wc, int pf, int *done, int *info) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    // chase progress, loaded-up-to column, flushed-up-to column, loader finished, abort flag
-    __shared__ int sh_tau, sh_hi, sh_fl, sh_ldone, sh_abort;
+    // chase progress, loaded-up-to column, flushed-up-to column, loader finished, abort flag, and the
+    // abort flag as the chase warps act on it (all in the same step: they meet in barriers)
+    __shared__ int sh_tau, sh_hi, sh_fl, sh_ldone, sh_abort, sh_stop;
     const int ldw = (3 * b + 2) & ~1;  // even: lanes walking a row hit distinct banks
     Win<T> W{reinterpret_cast<T *>(smem_raw), ldw, wc, 2 * b};
     T *vbase = W.w + (size_t)wc * ldw;  // 64 entries per chase warp
@@ -454,7 +455,20 @@ __global__ void band2bd_group_kernel(T *AB, long ldab, int n, int b, int G, int 
     const int nsweeps = n - 2;
     const int ngroups = (nsweeps + G - 1) / G;
     volatile int *vtau = &sh_tau, *vhi = &sh_hi, *vfl = &sh_fl, *vldone = &sh_ldone, *vabort = &sh_abort;
-    if (tid == 0) sh_abort = 0;
+    volatile int *vstop = &sh_stop;
+    // A mover warp acts on lane 0's view of a shared word, and on what was written before it (fence,
+    // then the warp barrier): its lanes meet in warp-wide operations.
+    const auto seen = [](volatile int *word) {
+        const int v = *word;
+        __threadfence_block();
+        __syncwarp();
+        return __shfl_sync(0xffffffffu, v, 0);
+    };
+    if (tid == 0) {
+        sh_abort = 0;
+        sh_stop = 0;
+    }
+    __syncthreads();
     for (int grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {
         const int s0 = grp * G, g = min(G, nsweeps - s0);
         int lo0, hi0;
@@ -466,8 +480,7 @@ __global__ void band2bd_group_kernel(T *AB, long ldab, int n, int b, int G, int 
             sh_fl = lo0 - 1;
             sh_ldone = 0;
         }
-        __syncthreads();
-        if (*vabort) break;
+        if (__syncthreads_or(*vabort)) break;  // (the same way for every thread)
         if (warp < G) {
             // ---------------- chase warps
             T *v = vbase + warp * 64;
@@ -508,10 +521,12 @@ __global__ void band2bd_group_kernel(T *AB, long ldab, int n, int b, int G, int 
                 }
                 // the right reflectors of this step all precede every left reflector:
                 // with sweeps two steps apart that is the order the sequential chase needs
+                if (warp == 0 && lane == 0) *vstop = *vabort;
                 asm volatile("bar.sync 1, %0;" ::"r"(32 * G) : "memory");
+                const int stop = *vstop;
                 if (ok && mine) warp_chase_step<T>(W, n, b, s, k, wslot, v, 1);  // left reflector
                 asm volatile("bar.sync 1, %0;" ::"r"(32 * G) : "memory");
-                if (*vabort) break;
+                if (stop) break;
                 if (warp == 0 && lane == 0) {
                     __threadfence_block();
                     *vtau = tau + 1;
@@ -522,9 +537,8 @@ __global__ void band2bd_group_kernel(T *AB, long ldab, int n, int b, int G, int 
             int flushed = lo0 - 1;
             unsigned idle = 32;  // backoff while there is nothing to write back
             for (;;) {
-                if (*vabort) break;
-                const int t = *vtau;  // steps < t are complete
-                __threadfence_block();
+                if (seen(vabort)) break;
+                const int t = seen(vtau);  // steps < t are complete
                 int lo, hi;
                 bool active;
                 group_need(n, b, s0, g, t, lo, hi, active);
@@ -540,9 +554,8 @@ __global__ void band2bd_group_kernel(T *AB, long ldab, int n, int b, int G, int 
                         }
                     }
                     __syncwarp();
-                    __threadfence_block();
-                    if (*vabort) break;
-                    const int fin = *vhi;
+                    if (seen(vabort)) break;
+                    const int fin = seen(vhi);
                     if (fin > flushed) mover_copy<T, false>(W, A, n, b, flushed + 1, fin, lane);
                     __threadfence();
                     __syncwarp();
@@ -559,6 +572,7 @@ __global__ void band2bd_group_kernel(T *AB, long ldab, int n, int b, int G, int 
                         st_release(&done[grp], flushed + 1);
                         *vfl = flushed;  // the loader may reuse these slots now
                     }
+                    __syncwarp();
                     idle = 32;
                 } else {
                     __nanosleep(idle);
@@ -571,9 +585,8 @@ __global__ void band2bd_group_kernel(T *AB, long ldab, int n, int b, int G, int 
             int have = grp > 0 ? 0 : INT_MAX;  // columns < have are final in the previous group
             unsigned idle = 32;  // backoff while nothing new can be loaded
             for (;;) {
-                if (*vabort) break;
-                const int t = *vtau;
-                __threadfence_block();
+                if (seen(vabort)) break;
+                const int t = seen(vtau);
                 int lo, hi;
                 bool active;
                 group_need(n, b, s0, g, t, lo, hi, active);
@@ -583,8 +596,7 @@ __global__ void band2bd_group_kernel(T *AB, long ldab, int n, int b, int G, int 
                 bool at;
                 group_need(n, b, s0, g, t + pf, lt, want, at);
                 want = max(want, hi);
-                want = min(want, *vfl + wc);
-                __threadfence_block();
+                want = min(want, seen(vfl) + wc);
                 bool worked = false;
                 if (want > loaded) {
                     if (have - 1 < want) {  // (never for group 0)
@@ -592,7 +604,7 @@ __global__ void band2bd_group_kernel(T *AB, long ldab, int n, int b, int G, int 
                             // the current step cannot start without its columns: wait for those
                             if (lane == 0 && !spin_until_geq(&done[grp - 1], hi + 1, info, 64)) *vabort = 1;
                             __syncwarp();
-                            if (*vabort) break;
+                            if (seen(vabort)) break;
                         }
                         // every lane acquires, so that its own copies below see what the previous
                         // group wrote; the smallest value seen is final for all of them
