@@ -275,29 +275,44 @@ struct Half {
     }
 };
 
-// Mover warp, element by element (a band whose leading dimension is not the packed one):
-// columns j0..j1, 3B+1 storage rows each.  Loads are asynchronous copies that all issue
-// before the one wait.
+// Mover warp, element by element (a band whose leading dimension is not the packed one): columns
+// j0 .. j0 + cnt - 1, 3B+1 storage rows each, of which only those inside the matrix are touched.
+// Loads are asynchronous copies; stores are read four columns at a time before the first is stored.
+// (Waiting for each chunk's loads and a division per column bound the chase before: n = 4096, B = 16,
+// FP32, with a counters-only workspace 19.4 -> 12.3 ms; B = 32, n = 3000 29.5 -> 20.9.)
 template <class S, bool LOAD>
-NLA_DEV void copy_columns(typename S::Elem *win, int wc, typename S::Elem *AB, long ldab, int n, int j0, int j1, int lane) {
+NLA_DEV void copy_columns(typename S::Elem *win, int wc, typename S::Elem *AB, long ldab, int n, int j0, int cnt, int lane) {
     using T = typename S::Elem;
-    constexpr int H = 3 * S::B + 1;
-    for (int j = j0; j <= j1; ++j) {
-        T *cw = win + (size_t)(j % wc) * S::kLd;
-        T *cg = AB + (long)j * ldab;
+    constexpr int B = S::B, H = 3 * B + 1, QI = (H + 31) / 32, CU = LOAD ? 1 : 4;
+    const int sl0 = j0 % wc;
+    const auto inside = [&](int c, int q) { return q < H && (unsigned)(j0 + c + q - 2 * B) < (unsigned)n; };
+    const auto slot = [&](int c) { return win + (size_t)(sl0 + c - (sl0 + c >= wc ? wc : 0)) * S::kLd; };
+    T *const src = AB + (long)j0 * ldab;
+    for (int c0 = 0; c0 < cnt; c0 += CU) {
+        T r[CU][QI];
 #pragma unroll
-        for (int q0 = 0; q0 < H; q0 += 32) {
-            const int q = q0 + lane, i = j + q - 2 * S::B;
-            if (q >= H || i < 0 || i >= n) continue;
-            if (LOAD)
-                asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(tc::smem_u32(cw + q)), "l"(cg + q),
-                             "n"((int)sizeof(T))
-                             : "memory");
-            else
-                __stcg(cg + q, cw[q]);
+        for (int u = 0; u < CU; ++u)
+#pragma unroll
+            for (int i = 0; i < QI; ++i) {
+                const int c = c0 + u, q = 32 * i + lane;
+                if (c >= cnt || !inside(c, q)) continue;
+                if (LOAD)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(tc::smem_u32(slot(c) + q)),
+                                 "l"(src + (long)c * ldab + q), "n"((int)sizeof(T))
+                                 : "memory");
+                else
+                    r[u][i] = slot(c)[q];
+            }
+        if (!LOAD) {
+#pragma unroll
+            for (int u = 0; u < CU; ++u)
+#pragma unroll
+                for (int i = 0; i < QI; ++i) {
+                    const int c = c0 + u, q = 32 * i + lane;
+                    if (c < cnt && inside(c, q)) __stcg(src + (long)c * ldab + q, r[u][i]);
+                }
         }
     }
-    if (LOAD) asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 // Block = G teams, then a clerk, a flusher and a loader warp.  The teams run the group's sweeps
@@ -347,7 +362,8 @@ chase_kernel(typename S::Elem *AB, long ldab, int n, int G, int wc, int *done, i
     if (tid == 0) {
         sh_abort = 0;
         sh_stop = 0;
-        for (int i = 0; i < kChunkBars; ++i) tc::mbar_init(&cbar[i], 1);
+        // (a chunk completes with the one lane that issued it, or with every lane's own copies)
+        for (int i = 0; i < kChunkBars; ++i) tc::mbar_init(&cbar[i], BULK ? 1 : 32);
         tma::fence_init();
     }
     __syncthreads();
@@ -457,7 +473,7 @@ chase_kernel(typename S::Elem *AB, long ldab, int n, int G, int wc, int *done, i
                             tma::wait_all();
                             fence_async_all();  // the copies' writes precede the release
                         } else {
-                            copy_columns<S, false>(win, wc, AB, ldab, n, j0, fin, lane);
+                            copy_columns<S, false>(win, wc, AB, ldab, n, j0, fin - flushed, lane);
                             __threadfence();
                             __syncwarp();
                         }
@@ -498,15 +514,14 @@ chase_kernel(typename S::Elem *AB, long ldab, int n, int G, int wc, int *done, i
                         bulk_load(win + (size_t)sl * LD, AB + (long)j0 * LD, (uint32_t)(k1 * LD * sizeof(T)), bar);
                         if (k2 > 0) bulk_load(win, AB + (long)(j0 + k1) * LD, (uint32_t)(k2 * LD * sizeof(T)), bar);
                     } else {
-                        copy_columns<S, true>(win, wc, AB, ldab, n, j0, j0 + cnt - 1, lane);
-                        __threadfence_block();
-                        __syncwarp();
-                        if (lane == 0) tma::arrive(bar);
+                        copy_columns<S, true>(win, wc, AB, ldab, n, j0, cnt, lane);
+                        asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
                     }
                     ++m;
                 }
-                // giving up: let the copies in flight land before the block may leave
-                for (int i = max(0, m - kChunkBars); i < m && *vabort && lane == 0; ++i) {
+                // let the copies in flight land before the block may leave
+                if (!BULK) asm volatile("cp.async.wait_all;" ::: "memory");
+                for (int i = max(0, m - kChunkBars); BULK && i < m && *vabort; ++i) {
                     const uint32_t c = chunk0 + i;
                     tc::mbar_wait(&cbar[c % kChunkBars], c / kChunkBars & 1, info);
                 }
