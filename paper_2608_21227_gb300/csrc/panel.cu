@@ -595,6 +595,10 @@ NLA_DEV void panel_scalars(double alpha, double xn2, double &beta, double &tau, 
     scale = 1.0 / (alpha - beta);
 }
 
+// Whether the scale of a short vector times an entry of the largest size overflows (above 2^60, 2^480).
+NLA_DEV bool too_large(float scale) { return (__float_as_uint(scale) & 0x7fffffffu) > 187u << 23; }
+NLA_DEV bool too_large(double scale) { return ((unsigned)__double2hiint(scale) & 0x7fffffffu) > 1503u << 20; }
+
 template <typename T, int NB, int R>
 __global__ void __launch_bounds__(32 * (kRegWarps + 1), 1)
 panel_reg_kernel(T *__restrict__ P, long rs, long cs, int M, int nb, int nw, T *__restrict__ tau,
@@ -744,9 +748,14 @@ panel_reg_kernel(T *__restrict__ P, long rs, long cs, int M, int nb, int nw, T *
                 if (c == j) taus[j] = tau[j] = tj;
             }
             // ---- rows below j: a_c -= x (scale w_c); row j: a_c -= w_c, beta in column j
-            const T m = -scale * w;
+            if (__builtin_expect(too_large(scale), 0)) {  // scale w may overflow: v = x / (alpha - beta) first
 #pragma unroll
-            for (int i = 0; i < R; ++i) a[i] = fma(x[i], m, a[i]);
+                for (int i = 0; i < R; ++i) a[i] = fma(x[i] * scale, -w, a[i]);
+            } else {
+                const T m = -scale * w;
+#pragma unroll
+                for (int i = 0; i < R; ++i) a[i] = fma(x[i], m, a[i]);
+            }
             if (p == 0 && warp * HV * R < NB) {
                 if (pivot) top[j][c] = c < j ? rv * myscale : c == j ? beta : rv - w;
 #pragma unroll

@@ -80,3 +80,53 @@ def test_band_fp64_graded(nla, b, low):
         S, info2 = nla.bdsvd_vals(d, e)
         assert int(info2.item()) == 0
         _check(S, info, M, tol_for(0, n))
+
+
+@pytest.mark.parametrize("dt,tiny,big,medium", [(1, 4e-20, 1.2e19, 1e10), (0, 4e-156, 8e153, 1e100)])
+@pytest.mark.parametrize("m,band", [(40, 16), (40, 32), (3000, 16), (3000, 32)])
+def test_panel_quotient_of_column_sizes_overflows(nla, dt, tiny, big, medium, m, band):
+    # columns 0 and 1: one entry of size tiny, two of size big, whose quotient overflows while no square does
+    n = 40
+    A = np.random.default_rng(m).standard_normal((m, n)) * medium
+    A[:, :2] = 0.0
+    A[1, 0] = tiny
+    A[0, 1] = A[1, 1] = big
+    t = to_device_colmajor(A, torch.float32 if dt else torch.float64)
+    A = t.double().cpu().numpy().T
+    _, _, info = nla.gebrd_band(t, band)
+    D = np.triu(t.double().cpu().numpy().T[:n, :n])
+    D = np.where(np.subtract.outer(np.arange(n), np.arange(n)) >= -band, D, 0.0)
+    torch.cuda.synchronize()
+    assert int(info.item()) == 0
+    s1 = np.hypot(big, big)
+    ref = np.linalg.svd(A / s1, compute_uv=False)
+    assert err_rel(np.linalg.svd(D / s1, compute_uv=False), ref) <= tol_for(dt, m)
+
+
+@pytest.mark.parametrize("b", [8, 16, 32, 64])
+def test_band_quotient_overflows(nla, b):
+    # rows of size 1e-156 beside rows of size 1e152
+    n = 150
+    i, j = np.indices((n, n))
+    D = np.where((j - i >= 0) & (j - i <= b), np.random.default_rng(b).uniform(0.5, 1.0, (n, n)), 0.0)
+    D *= np.where(np.arange(n) % 3 == 0, 2e-156, 4e153 / (2 * b))[:, None]
+    d, e, info = nla.band2bd(nla.band_extract(to_device_colmajor(D, torch.float64), b), b)
+    S, info2 = nla.bdsvd_vals(d, e)
+    torch.cuda.synchronize()
+    assert int(info2.item()) == 0
+    _check(S, info, D, tol_for(0, n))
+
+
+@pytest.mark.parametrize("dt", [0, 1])
+def test_band_zero_blocks(nla, dt):
+    # zero vectors take no reflector: diagonal parts, zero rows and columns
+    n, b = 200, 16
+    i, j = np.indices((n, n))
+    D = np.where((j - i >= 0) & (j - i <= b), np.random.default_rng(7).standard_normal((n, n)), 0.0)
+    D[50:90][:, 50:] = np.where(np.eye(n)[50:90][:, 50:] > 0, D[50:90][:, 50:], 0.0)
+    D[120:140] = 0.0
+    D[:, 160:180] = 0.0
+    tdt = torch.float32 if dt else torch.float64
+    d, e, info = nla.band2bd(nla.band_extract(to_device_colmajor(D, tdt), b), b)
+    S, _ = nla.bdsvd_vals(d, e, dtype=tdt)
+    _check(S, info, D, tol_for(dt, n))
