@@ -128,8 +128,10 @@ nla_status nla_gesvd_vals(int m, int n, nla_dtype dtype, void *dA, int lda, void
  * and leading dimensions; dA_array / dS_array: DEVICE arrays of device
  * pointers; matrix i is column major m_i x n_i and is read, not modified;
  * dS_array[i] receives min(m_i, n_i) values, descending.  max_m, max_n bound
- * every m_i, n_i (min(max_m, max_n) <= 256).  dInfo: `batch` device ints (0 =
- * success, -NLA_ERR_UNSUPPORTED for a matrix outside the bounds).  Matrices
+ * every m_i, n_i, or every larger and every smaller dimension
+ * (min(max_m, max_n) <= 256).  dInfo: `batch` device ints (0 = success,
+ * -NLA_ERR_UNSUPPORTED for a matrix with both dimensions above 256, or outside
+ * the bounds with more than 49,152 and than max_m max_n entries).  Matrices
  * are ordered by size on the device; the tuned table (kt_load_config) may set
  * the least threads per matrix for each size bucket.  Nothing is read from the
  * host at run time, so the call can be captured in a CUDA graph and replayed.
@@ -176,7 +178,7 @@ nla_status nla_band_extract(int n, int band, nla_dtype dtype, const void *dA, in
  * diagonal and superdiagonal.  dWork: >= nla_band2bd_workspace bytes (the
  * sweeps' progress counters and, for bands of 8, 16, 32 and 64, a packed copy of
  * the band; with room for the counters only, n ints, the chase works on dAB
- * itself, which is 5 to 20 % slower up to band 16 and up to 2.5 times at band 64
+ * itself, which takes up to 1.2 times as long up to band 16 and 2.5 at band 64
  * unless dAB is 16-byte aligned and ldab is the packed leading dimension,
  * 3*band + 1 rounded up to whole 16 bytes: whole columns of ldab entries are
  * then moved.  The library allocates nothing on this path). */

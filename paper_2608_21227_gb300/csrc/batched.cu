@@ -47,7 +47,7 @@ constexpr int kWarps = 16, kThreads = 32 * kWarps;
 constexpr int kBuckets = 5;      // size buckets of the tuned table, by element count
 constexpr int kBucketElems = 48 * 1024;
 constexpr int kClasses = 5;      // 0: N <= 256, 1: N <= 192 (16 warps), 2: N <= 128 (8), 3: N <= 64 (4), 4: N <= 32 (1)
-constexpr int kCostBins = 128;   // per class, eighths of a power of two of the cost
+constexpr int kCostBins = 128;   // per class, quarters of a power of two of the cost
 
 // Least threads per matrix for each size bucket (the tuned table's group sizes): a matrix is
 // given to the smallest class that holds its N and has as many threads.
@@ -537,7 +537,7 @@ cudaError_t one_launch(const float *A, int M, int N, int lda, bool tr, float *S,
 __global__ void __launch_bounds__(kThreads, 1)
 batched_svd_kernel(const int *__restrict__ dM, const int *__restrict__ dN, const int *__restrict__ dLda,
                    float *const *dA, float *const *dS, const int *__restrict__ order, unsigned int *ctl,
-                   size_t slot_elems, int *dInfo) {
+                   int max_m, int max_n, int *dInfo) {
     extern __shared__ __align__(16) float smem[];
     __shared__ int sh_unit;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -559,8 +559,11 @@ batched_svd_kernel(const int *__restrict__ dM, const int *__restrict__ dN, const
             const int i = order[pos];
             const int m = dM[i], n = dN[i], lda = dLda[i];
             const int M = max(m, n), N = min(m, n);
-            // (matrices beyond the sizes the caller declared are refused)
-            const bool ok = N <= 256 && ((long)M * N <= kBucketElems || (size_t)((M + 3) & ~3) * N <= slot_elems);
+            // Large matrices beyond the declared bounds are refused.  The bounds may be those of m_i and n_i
+            // or of the larger and the smaller dimension; up to max_m max_n entries are accepted either way.
+            const bool within = (m <= max_m && n <= max_n) || (long)M * N <= kBucketElems ||
+                                (long)((M + 3) & ~3) * N <= (long)((max(max_m, 1) + 3) & ~3) * max(max_n, 1);
+            const bool ok = N <= 256 && within;
             if (ok && N > 0) {
                 const float *A = dA[i];
                 float *S = dS[i];
@@ -628,7 +631,7 @@ nla_status nla_gesvd_vals_batched(int batch, nla_dtype dtype, const int *dM, con
     if (dtype != NLA_F32) return berr(NLA_ERR_UNSUPPORTED, "the batched kernel supports FP32 only");
     if (batch < 0 || max_m < 0 || max_n < 0) return berr(NLA_ERR_ARG, "negative size");
     if (batch == 0) return NLA_OK;
-    if (max_n > 256) return berr(NLA_ERR_UNSUPPORTED, "min(m_i, n_i) must be <= 256");
+    if (std::min(max_m, max_n) > 256) return berr(NLA_ERR_UNSUPPORTED, "min(m_i, n_i) must be <= 256");
     if (!dM || !dN || !dLda || !dA_array || !dS_array || !dInfo || !dWork)
         return berr(NLA_ERR_ARG, "null device pointer");
     size_t need = 0;
@@ -639,7 +642,6 @@ nla_status nla_gesvd_vals_batched(int batch, nla_dtype dtype, const int *dM, con
     char *w = reinterpret_cast<char *>(dWork);
     unsigned int *ctl = reinterpret_cast<unsigned int *>(w);
     int *order = reinterpret_cast<int *>(w + 256);
-    const size_t slot = (size_t)((std::max(max_m, 1) + 3) & ~3) * std::max(max_n, 1);
     BatchCfg cfg;
     for (int b = 0; b < kBuckets; ++b) {
         const int g = nla::g_batched_group[b];
@@ -656,7 +658,7 @@ nla_status nla_gesvd_vals_batched(int batch, nla_dtype dtype, const int *dM, con
         batched_prep_kernel<<<1, 1024, 0, st>>>(batch, dM, dN, order, ctl, cfg);
         const int blocks = std::min(nla::device_sm_count(), batch);
         batched_svd_kernel<<<blocks, kThreads, smem, st>>>(dM, dN, dLda, (float *const *)dA_array, (float *const *)dS_array,
-                                                           order, ctl, slot, dInfo);
+                                                           order, ctl, max_m, max_n, dInfo);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return berr(NLA_ERR_CUDA, cudaGetErrorString(e));

@@ -174,3 +174,29 @@ def test_single_small_matrix(nla, m, n):
         torch.cuda.synchronize()
         assert int(info.item()) == 0 and torch.equal(t, keep)
         assert err_rel(S.cpu().numpy(), ref) <= 5e-6 * max(m, n)
+
+
+@pytest.mark.parametrize("shapes,max_m,max_n", [([(200, 250), (200, 246), (3, 250)], 200, 250),
+                                                ([(100, 1000), (7, 999)], 100, 1000), ([(1000, 100)], 1000, 100),
+                                                ([(255, 3001), (256, 256)], 256, 3001)])
+def test_bounds_of_rows_and_columns(nla, shapes, max_m, max_n):
+    # bounds given for m_i and n_i (the binding gives the larger and the smaller dimension): wide matrices at them
+    mats = [np.random.default_rng(m + n).standard_normal((m, n)).astype(np.float32) for m, n in shapes]
+    b = make_batch(nla, mats)
+    b.max_m, b.max_n = max_m, max_n
+    S, info = nla.gesvd_vals_batched(b)
+    check(S, info, mats)
+
+
+def test_matrices_beyond_the_bounds_are_refused(nla):
+    mats = [np.random.default_rng(i).standard_normal(s).astype(np.float32) for i, s in enumerate([(300, 260), (400, 200), (20, 10)])]
+    b = make_batch(nla, mats)
+    b.max_m, b.max_n = 200, 200
+    for s in b.S:
+        s.fill_(-1.0)
+    _, info = nla.gesvd_vals_batched(b)
+    torch.cuda.synchronize()
+    assert info.tolist() == [-7, -7, 0] and float(b.S[0].max()) == -1.0 and float(b.S[1].max()) == -1.0
+    b.max_m, b.max_n = 300, 257
+    with pytest.raises(nla.NLAError):
+        nla.gesvd_vals_batched(b)
