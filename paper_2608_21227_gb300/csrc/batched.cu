@@ -354,7 +354,8 @@ struct Worker {
                         float s = 0.f;
 #pragma unroll
                         for (int q = 0; q < NW / 2; ++q) s += part[((t & 1) * (NW / 2) + q) * C::kPart + row];
-                        s += __shfl_xor_sync(__activemask(), s, 1);
+                        static_assert(RH % 16 == 0, "a warp's 16 rows exist together");
+                        s += __shfl_xor_sync(0xffffffffu, s, 1);
                         if ((t & 1) == 0) ys[row] = s;
                     }
                     sync();
