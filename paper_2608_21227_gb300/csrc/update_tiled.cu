@@ -594,6 +594,7 @@ static cudaError_t run_tiled(int side, T *X, long ldx, int M, int N, const T *V,
     T *fin = part + (size_t)kMaxSplit * 64 * std::max(M, N);
     const int strip = side == 0 ? N : M, len = side == 0 ? M : N;
     const Shape a = step1_shape<T>(side, nb, R, c, strip, len), b = step3_shape<T>(c, strip, len);
+    if (a.Ms <= 0) return cudaErrorInvalidConfiguration;  // no block shape fits: a zero W otherwise
     const auto step1 = a.R == 1   ? run_step1<T, U, 1>
                        : a.R == 2 ? run_step1<T, U, 2>
                        : a.R == 4 ? run_step1<T, U, 4>
