@@ -413,16 +413,6 @@ qr_proj_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
                 break;
             }
             const int r0 = rbeg + t * kBoxRows;  // trailing-matrix row of the stage's first row
-            float *vh = reinterpret_cast<float *>(vhi(st));
-            if (r0 < NB) {
-                // V(r, k) with r <= k: 1 on the diagonal, 0 above (entry (r, k) of the box:
-                // row k, 16-byte chunk (r/4) ^ (k & 7), word r % 4)
-                for (int e = ct; e < NB * kBoxRows; e += 128) {
-                    const int k = e / kBoxRows, rr = e % kBoxRows, r = r0 + rr;
-                    if (r <= k) vh[k * 32 + ((((rr >> 2) ^ (k & 7))) << 2) + (rr & 3)] = r == k ? 1.f : 0.f;
-                }
-                asm volatile("bar.sync 2, 128;" ::: "memory");
-            }
             const float4 *xs = reinterpret_cast<const float4 *>(xhi(st));
             float4 *xl = reinterpret_cast<float4 *>(xlo(st));
 #pragma unroll 4
@@ -431,10 +421,21 @@ qr_proj_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
                 xl[e] = make_float4(tf32_lo(v.x, tf32_hi(v.x)), tf32_lo(v.y, tf32_hi(v.y)), tf32_lo(v.z, tf32_hi(v.z)),
                                     tf32_lo(v.w, tf32_hi(v.w)));
             }
-            float4 *vs = reinterpret_cast<float4 *>(vh);
+            float4 *vs = reinterpret_cast<float4 *>(vhi(st));
             float4 *vl = reinterpret_cast<float4 *>(vlo(st));
             for (int e = ct; e < vbytes / 16; e += 128) {
-                const float4 v = vs[e], h = make_float4(tf32_rn(v.x), tf32_rn(v.y), tf32_rn(v.z), tf32_rn(v.w));
+                float4 v = vs[e];
+                // V(r, k) with r <= k: 1 on the diagonal, 0 above.  16-byte chunk e of the box is row k = e / 8,
+                // rows 4 ((e & 7) ^ (k & 7)) .. of the stage.  (Masked where it is converted: no barrier that
+                // a warp could wait at after another has given up.)
+                if (r0 < NB) {
+                    const int k = e >> 3, r = r0 + 4 * ((e & 7) ^ (k & 7));
+                    v.x = r > k ? v.x : r == k ? 1.f : 0.f;
+                    v.y = r + 1 > k ? v.y : r + 1 == k ? 1.f : 0.f;
+                    v.z = r + 2 > k ? v.z : r + 2 == k ? 1.f : 0.f;
+                    v.w = r + 3 > k ? v.w : r + 3 == k ? 1.f : 0.f;
+                }
+                const float4 h = make_float4(tf32_rn(v.x), tf32_rn(v.y), tf32_rn(v.z), tf32_rn(v.w));
                 vs[e] = h;
                 vl[e] = make_float4(tf32_lo(v.x, h.x), tf32_lo(v.y, h.y), tf32_lo(v.z, h.z), tf32_lo(v.w, h.w));
             }
