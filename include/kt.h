@@ -189,6 +189,7 @@ size_t kt_mlp_param_count(void);
 nla_status kt_mlp_forward_backward(const float *dParams, const float *dX, const float *dY, int rows,
                                    float *dPred, float *dGrads, void *dWork, size_t work_bytes,
                                    nla_stream_t stream);
+/* Bytes of dWork for any batch of up to `rows` rows (non-decreasing in rows). */
 size_t kt_mlp_work_bytes(int rows);
 
 /* One Adam step on device buffers (count parameters), step number t >= 1. */

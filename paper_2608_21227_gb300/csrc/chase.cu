@@ -591,7 +591,7 @@ cudaError_t launch(typename S::Elem *AB, long ldab, int n, int gmax, int *done, 
 template <typename T>
 cudaError_t band_repack(const T *src, long lds, T *dst, long ldd, int n, int b, cudaStream_t st) {
     const long total = (long)n * (3 * b + 1);
-    const int blocks = (int)std::min<long>((total + 255) / 256, 152L * 8);
+    const int blocks = (int)std::min<long>((total + 255) / 256, 8L * device_sm_count());
     repack_kernel<T><<<blocks, 256, 0, st>>>(src, lds, dst, ldd, n, 3 * b + 1);
     return cudaGetLastError();
 }

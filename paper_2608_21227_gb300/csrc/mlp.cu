@@ -16,6 +16,7 @@
 
 #include "../../include/kt.h"
 #include "common.cuh"
+#include "kernels.cuh"
 #include "tuned.h"
 
 namespace {
@@ -50,10 +51,11 @@ constexpr int kMlpThreads = 256;
 constexpr size_t mlp_smem_floats(int R) { return (size_t)kH * kLd + (size_t)R * 16 + (size_t)5 * R * kLd + R + 8; }
 
 // Rows per tile: small batches are spread over more blocks (8 rows: two blocks per SM fit).
-int mlp_tile(int rows) { return rows <= 8 * 304 ? 8 : 32; }
+int mlp_small_rows() { return 16 * nla::device_sm_count(); }
+int mlp_tile(int rows) { return rows <= mlp_small_rows() ? 8 : 32; }
 int mlp_blocks(int rows) {
-    const int tiles = (rows + mlp_tile(rows) - 1) / mlp_tile(rows);
-    return std::min(tiles, mlp_tile(rows) == 8 ? 304 : 152);
+    const int tile = mlp_tile(rows), sms = nla::device_sm_count();
+    return std::min((rows + tile - 1) / tile, tile == 8 ? 2 * sms : sms);
 }
 
 // Ws(k, o) = W[o * K + k] (TRANS) or Ws(o, k) = W[o * K + k], K = kH.
@@ -157,6 +159,7 @@ mlp_kernel(const float *__restrict__ P, const float *__restrict__ X, const float
     constexpr size_t oB[kLayers] = {(size_t)kH * kIn, oW[1] + kH * kH, oW[2] + kH * kH, oW[3] + kH};
     float *dP = part + (size_t)blockIdx.x * kParams;
     bool first = true;
+    float loss = 0.f;  // of this warp's rows
     for (int row0 = blockIdx.x * R; row0 < rows; row0 += gridDim.x * R, first = false) {
         __syncthreads();
         for (int i = tid; i < R * 16; i += kMlpThreads) {
@@ -206,7 +209,7 @@ mlp_kernel(const float *__restrict__ P, const float *__restrict__ X, const float
             }
             if (c == 0) {
                 gout[r0 + r] = 2.f * d / (float)rows;
-                if (train && loss_acc && row < rows) atomicAdd(loss_acc, d * d / (float)rows);
+                loss += d * d / (float)rows;
             }
         }
         if (!train) continue;
@@ -259,6 +262,7 @@ mlp_kernel(const float *__restrict__ P, const float *__restrict__ X, const float
             *d = first ? s : *d + s;
         }
     }
+    if (train && loss_acc && c == 0) atomicAdd(loss_acc, loss);
 }
 
 // grads[i] = sum over the blocks' partial sums, in block order.  32 parameters x 8 slices of
@@ -281,15 +285,21 @@ __global__ void grad_sum_kernel(const float *__restrict__ part, int nblk, float 
     }
 }
 
-// Floats of work for a batch of `rows`: the predictions and the blocks' partial gradients.
-size_t work_floats(int rows) { return (size_t)((rows + 63) & ~63) + (size_t)mlp_blocks(rows) * kParams; }
+// Floats of work for a batch of `rows`: the predictions and, to train, the blocks' partial gradients.
+size_t pred_floats(int rows) { return ((size_t)rows + 63) & ~(size_t)63; }
+size_t work_floats(int rows) { return pred_floats(rows) + (size_t)mlp_blocks(rows) * kParams; }
+// The same for any batch of up to `rows` (the number of blocks halves above mlp_small_rows).
+size_t work_floats_up_to(int rows) {
+    const int small = mlp_small_rows();
+    return rows > small ? std::max(work_floats(rows), work_floats(small)) : work_floats(rows);
+}
 
 // Predictions (into pred) and, when grads is given, the gradients of the mean squared error.
 cudaError_t mlp_pass(cudaStream_t st, const float *P, const float *X, const float *y, int rows, float *work,
                      float *pred, float *grads, float *loss_acc) {
     const int R = mlp_tile(rows), nblk = mlp_blocks(rows);
     const size_t smem = mlp_smem_floats(R) * sizeof(float);
-    float *part = work + ((rows + 63) & ~63);
+    float *part = work + pred_floats(rows);
     auto kern = R == 8 ? mlp_kernel<8> : mlp_kernel<32>;
     static nla::PerDeviceOnce attr;
     attr.run([] {
@@ -391,7 +401,7 @@ nla_status mlp_predict_host(const char *model_path, const float *X, int rows, fl
     cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
     nla_status s = NLA_OK;
     if (cudaMalloc(&dP, kParams * sizeof(float)) || cudaMalloc(&dX, Xs.size() * sizeof(float)) ||
-        cudaMalloc(&dW, work_floats(rows) * sizeof(float))) {
+        cudaMalloc(&dW, pred_floats(rows) * sizeof(float))) {
         cudaGetLastError();
         s = merr(NLA_ERR_CUDA, "MLP inference: allocation failed");
     } else {
@@ -415,12 +425,12 @@ extern "C" {
 
 size_t kt_mlp_param_count(void) { return kParams; }
 
-size_t kt_mlp_work_bytes(int rows) { return work_floats(std::max(rows, 1)) * sizeof(float); }
+size_t kt_mlp_work_bytes(int rows) { return work_floats_up_to(std::max(rows, 1)) * sizeof(float); }
 
 nla_status kt_mlp_forward_backward(const float *dParams, const float *dX, const float *dY, int rows, float *dPred,
                                    float *dGrads, void *dWork, size_t work_bytes, nla_stream_t stream) {
     if (rows <= 0 || !dParams || !dX || !dY || !dGrads || !dWork) return merr(NLA_ERR_ARG, "bad arguments");
-    if (work_bytes < kt_mlp_work_bytes(rows)) return merr(NLA_ERR_WORKSPACE, "MLP workspace too small");
+    if (work_bytes < work_floats(rows) * sizeof(float)) return merr(NLA_ERR_WORKSPACE, "MLP workspace too small");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     cudaError_t e = mlp_pass(st, dParams, dX, dY, rows, reinterpret_cast<float *>(dWork), dPred, dGrads, nullptr);
     return e == cudaSuccess ? NLA_OK : merr(NLA_ERR_CUDA, cudaGetErrorString(e));

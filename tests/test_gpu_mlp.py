@@ -102,3 +102,24 @@ def test_training_learns_a_known_surface(kt, tmp_path):
     pred = kt.mlp_predict(model, X[:512])
     mse = float(np.mean((pred - y[:512]) ** 2))
     assert mse < 0.1 * float(np.var(y)), (mse, float(np.var(y)), loss)
+
+
+@pytest.mark.parametrize("rows", [2432, 2000, 17])
+def test_workspace_of_a_larger_batch_serves(kt, rows):
+    import ctypes
+
+    g = torch.Generator(device="cuda")
+    g.manual_seed(rows)
+    params = torch.from_numpy(pack(omlp.init(15, seed=5))).cuda()
+    X = torch.randn(rows, 15, generator=g, device="cuda")
+    y = torch.randn(rows, generator=g, device="cuda")
+    pred, grads = kt.mlp_forward_backward(params, X, y)
+    L, vp = kt.lib(), ctypes.c_void_p
+    for largest in (2433, 4096):
+        work = torch.empty(int(L.kt_mlp_work_bytes(largest)), dtype=torch.uint8, device="cuda")
+        p2, g2 = torch.empty_like(pred), torch.empty_like(grads)
+        assert L.kt_mlp_forward_backward(vp(params.data_ptr()), vp(X.data_ptr()), vp(y.data_ptr()), rows, vp(p2.data_ptr()),
+                                         vp(g2.data_ptr()), vp(work.data_ptr()), work.numel(),
+                                         vp(torch.cuda.current_stream().cuda_stream)) == 0
+        torch.cuda.synchronize()
+        assert torch.equal(p2, pred) and torch.equal(g2, grads)

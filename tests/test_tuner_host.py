@@ -87,3 +87,10 @@ def test_features_layout(kt):
     want[11] = 1  # FP32
     want[14] = 1  # BF16 update
     assert np.allclose(f, want)
+
+
+def test_mlp_workspace_grows_with_the_batch(kt):
+    # a workspace for the largest batch serves every smaller one (the tile height changes with the rows)
+    rows = list(range(1, 80)) + [2000, 2368, 2369, 2431, 2432, 2433, 2500, 4096, 16000]
+    need = [kt.lib().kt_mlp_work_bytes(r) for r in rows]
+    assert all(a <= b for a, b in zip(need, need[1:]))
