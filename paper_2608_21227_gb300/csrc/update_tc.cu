@@ -5,10 +5,10 @@
 // mixed-precision form of the contraction).
 //
 // Two launches per side (as in the SIMT path): step 1 on a grid of
-// (32-wide strips) x (splits of the reduction dimension), the last block of a
+// (strips of LW = 32 or 64 lines) x (splits of the reduction dimension), the last block of a
 // strip applying T; step 3 on a 2-D grid of 128 x 128 output tiles.
-// QR side (strips of 32 columns of X in step 1, 128 in step 3):
-//   1. W^T (32 x nbp) = X_strip^T V, accumulated over 32-row tiles.  Each tile
+// QR side (strips of LW columns of X in step 1, 128 in step 3):
+//   1. W^T (LW x nbp) = X_strip^T V, accumulated over 32-row tiles.  Each tile
 //      of X is scaled per column by 2^-e (e = exponent of the column's largest
 //      magnitude in that tile), rounded to TF32/BF16 and multiplied on the
 //      tensor cores into one of two TMEM accumulators; the previous tile's
@@ -48,7 +48,6 @@ namespace {
 
 constexpr int kTcThreads = 256;   // 8 warps
 constexpr int kStrip = 128;       // UMMA M; step 3's strip width
-constexpr int kLines = 32;        // step 1's strip width
 constexpr int kKt = 32;           // rows (QR) / columns (LQ) of X per step-1 tile
 constexpr int kTmemCols = 256;    // self-test accumulator columns
 
@@ -272,12 +271,13 @@ __global__ void __launch_bounds__(128) tc_selftest_kernel(const float *A, const 
 //
 // Bound: the conversions.  A block's tiles follow one another (each adds to the running sum, and
 // the splits are fixed by the order of the sums), so a launch lasts as long as one block converts
-// its split.  A strip therefore has 32 lines, not the MMA's 128: the tensor cores idle anyway, and
-// the other rows of the tile are not written and their products not read.  The tiles are loaded
+// its split.  A strip therefore has 32 or 64 lines (launch_tc has the line between them), not the MMA's
+// 128: the tensor cores idle anyway, and the other rows of the tile are not written and their
+// products not read.  The tiles are loaded
 // one ahead; K entries are shared out so that a warp's stores to the K-major tile meet in at most
 // two banks' turns (lanes along K met 8 ways).  X 4096 x 1024, nb 16, TF32: 152 -> 48 us (QR), 91 ->
-// 57 us (LQ); 64 lines 1.2x, 128 lines 1.9x as long, at 5120 x 5120 0.95x and 1.09x.
-template <int PREC, int SIDE>
+// 57 us (LQ).
+template <int PREC, int SIDE, int LW>
 __global__ void __launch_bounds__(kTcThreads, 2)
 tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *__restrict__ V, long ldv, int nb,
             int nbp, const double *__restrict__ Tm, int Ls, float *part, int *pexp, float *fin, int *finexp,
@@ -286,22 +286,22 @@ tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ int sh_last;
     constexpr int es = P::es, rb1 = kKt * es;
-    constexpr int kWarps = kTcThreads / 32;
+    constexpr int kWarps = kTcThreads / 32, NL = LW / 32;
     constexpr int nsp = P::split ? 2 : 1;                    // hi (and lo) copies of each tile
     unsigned char *A1 = sm;                                  // 2 x [128 x kKt]  X tile (strip line x K)
     unsigned char *B1 = A1 + 2 * kStrip * rb1;               // 2 x [64 x kKt]   V tile (reflector x K)
     unsigned char *A1l = B1 + 2 * 64 * rb1;                  // lo copies (compensated forms)
     unsigned char *B1l = A1l + (nsp - 1) * 2 * kStrip * rb1;
-    int *ex1 = reinterpret_cast<int *>(B1l + (nsp - 1) * 2 * 64 * rb1);  // 2 x kLines
-    int *lmax = ex1 + 2 * kLines;                                // kWarps x kLines biased exponents (LQ)
-    TcShared *sh = reinterpret_cast<TcShared *>(lmax + kWarps * kLines);
-    float *Wsh = reinterpret_cast<float *>(sm);              // reused after the MMAs: nbp x kLines
+    int *ex1 = reinterpret_cast<int *>(B1l + (nsp - 1) * 2 * 64 * rb1);  // 2 x LW
+    int *lmax = ex1 + 2 * LW;                                // kWarps x LW biased exponents (LQ)
+    TcShared *sh = reinterpret_cast<TcShared *>(lmax + kWarps * LW);
+    float *Wsh = reinterpret_cast<float *>(sm);              // reused after the MMAs: nbp x LW
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int q = warp & 3, hh = warp >> 2;
     // strip lines: QR -> columns of X, LQ -> rows of X; reduction dimension: the other one
-    const int L0 = blockIdx.x * kLines;
+    const int L0 = blockIdx.x * LW;
     const int Lext = SIDE == 0 ? N : M, Kext = SIDE == 0 ? M : N;
-    const int lw = min(kLines, Lext - L0);
+    const int lw = min(LW, Lext - L0);
     const int s = blockIdx.y, S = gridDim.y;
     const int kbeg = s * Ls, kend = min(Kext, kbeg + Ls);
     if (warp == 0) {
@@ -320,7 +320,8 @@ tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *
     const uint32_t tbase = sh->tmem_base;
     const uint32_t id1 = tc::idesc(P::fmt, 128, nbp);
     const int half = nbp / 2;
-    const bool reader = q == 0;  // warps 0 and 4 hold the strip's lines (TMEM lanes 0 .. 31), half the reflectors each
+    const bool reader = q < NL;  // warps q and q + 4 hold lines 32 q .. (TMEM lanes), half the reflectors each
+    const int rline = 32 * q + lane;
     float acc[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) acc[i] = 0.f;
@@ -332,14 +333,18 @@ tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *
     const int kq = SIDE == 0 ? (lane & 7) : warp * 4;
     constexpr int kStep = SIDE == 0 ? 8 : 1;
     const int ntiles = (kend - kbeg + kKt - 1) / kKt;
-    double xv[4], vv[2][4];
+    double xv[NL][4], vv[2][4];
     const auto load_tile = [&](int t) {
         const int k0 = kbeg + t * kKt + kq;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int g = k0 + i * kStep;
             const bool in = g < kend;
-            xv[i] = in && lr < lw ? (SIDE == 0 ? X[g + (long)(L0 + lr) * ldx] : X[(L0 + lr) + (long)g * ldx]) : 0.0;
+#pragma unroll
+            for (int u = 0; u < NL; ++u) {
+                const int l = 32 * u + lr;
+                xv[u][i] = in && l < lw ? (SIDE == 0 ? X[g + (long)(L0 + l) * ldx] : X[(L0 + l) + (long)g * ldx]) : 0.0;
+            }
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 const int n = 32 * u + lr;
@@ -367,25 +372,32 @@ tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *
         if (t < ntiles) {
             unsigned char *const At = A1 + buf * kStrip * rb1, *const Atl = A1l + buf * kStrip * rb1;
             unsigned char *const Bt = B1 + buf * 64 * rb1, *const Btl = B1l + buf * 64 * rb1;
-            int emx = max(max(f64_biased_exp(xv[0]), f64_biased_exp(xv[1])),
-                          max(f64_biased_exp(xv[2]), f64_biased_exp(xv[3])));
-            if (SIDE == 0) {
+            int emx[NL];
 #pragma unroll
-                for (int o = 1; o < 8; o <<= 1) emx = max(emx, __shfl_xor_sync(0xffffffffu, emx, o));
-            } else {
-                lmax[warp * kLines + lane] = emx;
+            for (int u = 0; u < NL; ++u) {
+                emx[u] = max(max(f64_biased_exp(xv[u][0]), f64_biased_exp(xv[u][1])),
+                             max(f64_biased_exp(xv[u][2]), f64_biased_exp(xv[u][3])));
+                if (SIDE == 0) {
+#pragma unroll
+                    for (int o = 1; o < 8; o <<= 1) emx[u] = max(emx[u], __shfl_xor_sync(0xffffffffu, emx[u], o));
+                } else {
+                    lmax[warp * LW + 32 * u + lane] = emx[u];
+                }
             }
 #pragma unroll
             for (int u = 0; u < 2; ++u)
                 if (32 * u < nbp) put_row(Bt, Btl, 32 * u + lr, vv[u], 0);
-            if (SIDE == 1) {
-                __syncthreads();
+            if (SIDE == 1) __syncthreads();
 #pragma unroll
-                for (int w = 0; w < kWarps; ++w) emx = max(emx, lmax[w * kLines + lane]);
+            for (int u = 0; u < NL; ++u) {
+                if (SIDE == 1) {
+#pragma unroll
+                    for (int w = 0; w < kWarps; ++w) emx[u] = max(emx[u], lmax[w * LW + 32 * u + lane]);
+                }
+                const int e = tile_exp_from_biased(emx[u]);
+                if (SIDE == 0 ? (lane & 7) == 0 : warp == 0) ex1[buf * LW + 32 * u + lr] = e;
+                put_row(At, Atl, 32 * u + lr, xv[u], e);
             }
-            const int e = tile_exp_from_biased(emx);
-            if (SIDE == 0 ? (lane & 7) == 0 : warp == 0) ex1[buf * kLines + lr] = e;
-            put_row(At, Atl, lr, xv, e);
             if (t + 1 < ntiles) load_tile(t + 1);
             tc::fence_async_smem();
             tc::fence_before_sync();
@@ -409,7 +421,7 @@ tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *
             // (ok and reader are warp-uniform: the TMEM loads below are warp-collective, so every
             // lane executes them; a line whose tile is all zero adds its product with factor 0)
             if (ok && reader) {
-                const int et = ex1[pb * kLines + lane];
+                const int et = ex1[pb * LW + rline];
                 float sc = 0.f;
                 if (et != kNoExp) {
                     if (et > erun) {
@@ -424,7 +436,7 @@ tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *
                 for (int c = 0; c < 32; c += 16) {
                     if (c >= half) break;
                     float v[16];
-                    tc::tmem_ld16(tbase + pb * 64 + hh * half + c, v);
+                    tc::tmem_ld16(tbase + pb * 64 + hh * half + c + ((uint32_t)(32 * q) << 16), v);
                     tc::tmem_wait_ld();
 #pragma unroll
                     for (int i = 0; i < 16; ++i) acc[c + i] += v[i] * sc;
@@ -442,11 +454,11 @@ tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *
     if (warp == 0) tc::tmem_dealloc(tbase, 128);
     if (sh->fail) return;
     // ---- partial of this split; the last block of the strip finishes
-    if (reader && lane < lw) {
+    if (reader && rline < lw) {
 #pragma unroll
         for (int i = 0; i < 32; ++i)
-            if (i < half) part[((size_t)s * nbp + hh * half + i) * Lext + L0 + lane] = acc[i];
-        if (hh == 0) pexp[(size_t)s * Lext + L0 + lane] = erun;
+            if (i < half) part[((size_t)s * nbp + hh * half + i) * Lext + L0 + rline] = acc[i];
+        if (hh == 0) pexp[(size_t)s * Lext + L0 + rline] = erun;
     }
     __threadfence();
     __syncthreads();
@@ -455,10 +467,10 @@ tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *
     if (!sh_last) return;
     __threadfence();
     // the line's common exponent: the largest of its splits' (kNoExp: all zero)
-    int *lexp = reinterpret_cast<int *>(Wsh + (size_t)nbp * kLines);
-    float *Tf = reinterpret_cast<float *>(lexp + kLines);  // T in FP32, nb x nb
+    int *lexp = reinterpret_cast<int *>(Wsh + (size_t)nbp * LW);
+    float *Tf = reinterpret_cast<float *>(lexp + LW);  // T in FP32, nb x nb
     for (int i = tid; i < nb * nb; i += blockDim.x) Tf[i] = (float)Tm[i];
-    if (tid < kLines) {
+    if (tid < LW) {
         int em = kNoExp;
 #pragma unroll
         for (int qq = 0; qq < 8; ++qq)
@@ -467,8 +479,8 @@ tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *
         if (tid < lw) finexp[L0 + tid] = em == kNoExp ? 0 : em;
     }
     __syncthreads();
-    for (int idx = tid; idx < nbp * kLines; idx += blockDim.x) {
-        const int l = idx % kLines, k = idx / kLines;
+    for (int idx = tid; idx < nbp * LW; idx += blockDim.x) {
+        const int l = idx % LW, k = idx / LW;
         float sum = 0.f;
         if (l < lw && lexp[l] != kNoExp)
 #pragma unroll
@@ -478,15 +490,15 @@ tc_w_kernel(const double *__restrict__ X, long ldx, int M, int N, const double *
                     if (es_ != kNoExp)
                         sum += __ldcg(part + ((size_t)qq * nbp + k) * Lext + L0 + l) * exp2_nonpos(es_ - lexp[l]);
                 }
-        Wsh[k * kLines + l] = sum;
+        Wsh[k * LW + l] = sum;
     }
     __syncthreads();
-    for (int idx = tid; idx < nbp * kLines; idx += blockDim.x) {
-        const int l = idx % kLines, kk = idx / kLines;
+    for (int idx = tid; idx < nbp * LW; idx += blockDim.x) {
+        const int l = idx % LW, kk = idx / LW;
         float v = 0.f;
         // QR: W'(kk) = sum_{k <= kk} T(k, kk) W(k);  LQ: Y'(kk) = sum_{k <= kk} Y(k) T(k, kk) -- same form
         if (kk < nb)
-            for (int k = 0; k <= kk; ++k) v += Tf[k + kk * nb] * Wsh[k * kLines + l];
+            for (int k = 0; k <= kk; ++k) v += Tf[k + kk * nb] * Wsh[k * LW + l];
         if (l < lw) fin[(size_t)kk * Lext + L0 + l] = v;
     }
     if (tid == 0) tickets[blockIdx.x] = 0u;
@@ -649,25 +661,25 @@ tc_x_kernel(double *__restrict__ X, long ldx, int M, int N, const double *__rest
     if (warp == 0) tc::tmem_dealloc(tbase, 128);
 }
 
-size_t tc_w_smem(int es, int nsp) {
+size_t tc_w_smem(int es, int nsp, int lw) {
     const size_t rb1 = (size_t)kKt * es;
-    return std::max((size_t)nsp * (2 * kStrip * rb1 + 2 * 64 * rb1) + (size_t)(2 + kTcThreads / 32) * kLines * 4 +
+    return std::max((size_t)nsp * (2 * kStrip * rb1 + 2 * 64 * rb1) + (size_t)(2 + kTcThreads / 32) * lw * 4 +
                         sizeof(TcShared) + 64,
-                    (size_t)64 * kLines * 4 + kLines * 4 + (size_t)64 * 64 * 4 + 64);
+                    (size_t)64 * lw * 4 + lw * 4 + (size_t)64 * 64 * 4 + 64);
 }
 size_t tc_x_smem(int es, int nbp, int nsp) {
     return (size_t)nsp * 2 * kStrip * nbp * es + kStrip * 4 + 2 * kStrip * 4 + sizeof(TcShared) + 64;
 }
 
-template <int PREC, int SIDE>
+template <int PREC, int SIDE, int LW>
 cudaError_t launch_tc_w(const double *X, long ldx, int M, int N, const double *V, long ldv, int nb, int nbp,
                         const double *Tm, int S, int Ls, float *part, int *pexp, float *fin, int *finexp,
                         const UpdScratch &sc, int *info, cudaStream_t st) {
     static PerDeviceOnce once;
-    allow_max_smem(tc_w_kernel<PREC, SIDE>, once);
+    allow_max_smem(tc_w_kernel<PREC, SIDE, LW>, once);
     const int Lext = SIDE == 0 ? N : M;
-    tc_w_kernel<PREC, SIDE><<<dim3((Lext + kLines - 1) / kLines, S), kTcThreads,
-                                  tc_w_smem(Prec<PREC>::es, Prec<PREC>::split ? 2 : 1), st>>>(
+    tc_w_kernel<PREC, SIDE, LW><<<dim3((Lext + LW - 1) / LW, S), kTcThreads,
+                                  tc_w_smem(Prec<PREC>::es, Prec<PREC>::split ? 2 : 1, LW), st>>>(
         X, ldx, M, N, V, ldv, nb, nbp, Tm, Ls, part, pexp, fin, finexp, sc.tickets, info);
     return cudaGetLastError();
 }
@@ -701,8 +713,13 @@ cudaError_t launch_tc(double *X, long ldx, int M, int N, const double *V, long l
     float *fin = part + (size_t)8 * 64 * L;
     int *pexp = reinterpret_cast<int *>(fin + (size_t)64 * L);
     int *finexp = pexp + (size_t)8 * L;
-    cudaError_t e =
-        launch_tc_w<PREC, SIDE>(X, ldx, M, N, V, ldv, nb, nbp, Tm, S, Ls, part, pexp, fin, finexp, sc, info, st);
+    // step 1: 64 lines a strip where that still gives every SM its two blocks.  Trailing updates of a whole
+    // reduction, ms, 32 / 64 lines everywhere / this rule: 2,048 square 13.0 / 15.2 / 13.0; 4,096 47.8 / 48.1 /
+    // 46.2; 6,144 123.7 / 114.3 / 112.4; the line at 1.4 or 2 times as many blocks 46.4 and 47.8 at 4,096.
+    // (128 lines: 21.6, 58.7 and 125.4.)
+    const bool wide = (long)((Lext + 63) / 64) * S >= 2L * device_sm_count();
+    const auto step1 = wide ? launch_tc_w<PREC, SIDE, 64> : launch_tc_w<PREC, SIDE, 32>;
+    cudaError_t e = step1(X, ldx, M, N, V, ldv, nb, nbp, Tm, S, Ls, part, pexp, fin, finexp, sc, info, st);
     if (e != cudaSuccess) return e;
     return nbp == 32 ? launch_tc_x<PREC, SIDE, 32>(X, ldx, M, N, V, ldv, nb, fin, finexp, info, st)
                      : launch_tc_x<PREC, SIDE, 64>(X, ldx, M, N, V, ldv, nb, fin, finexp, info, st);

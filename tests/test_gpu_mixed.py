@@ -235,3 +235,18 @@ def test_mixed_update_edges(nla, prec, m, n, b):
     A = inputs.prescribed(m, n, inputs.geometric_sigma(k, 1e4), seed=m + n)
     err = err_rel(mixed_run(nla, A, prec, b), oracle.svdvals(A))
     assert err <= 10 * U_OF[prec] * math.sqrt(max(m, n) / b)
+
+
+@pytest.mark.parametrize("update,u", [(1, 2.0 ** -11), (2, 2.0 ** -8), (3, 2.0 ** -20), (4, 2.0 ** -15)])
+@pytest.mark.parametrize("m,n,b", [(2500, 2469, 16), (2600, 2600, 32)])
+def test_projection_strips_of_64_lines(nla, update, u, m, n, b):
+    # from about 2,400 lines on the projection takes 64 a strip (below 32, in the same reduction), here with
+    # ragged last strips; against the native FP64 update within the first-order model 10 u sqrt(n / b)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(m + b)
+    A = torch.randn(n, m, generator=g, device="cuda", dtype=torch.float64)
+    ref, _ = nla.gesvd_vals(A, cfg=nla.Cfg.make(band=b), preserve_a=True)
+    S, info = nla.gesvd_vals(A, update=update, cfg=nla.Cfg.make(band=b), preserve_a=True)
+    torch.cuda.synchronize()
+    assert int(info.item()) == 0
+    assert err_rel(S.cpu().numpy(), ref.cpu().numpy()) <= 10.0 * u * math.sqrt(n / b)
