@@ -30,7 +30,7 @@
 //
 // Measured on GB300 (one warp per sweep, 16 sweeps a block, element copies -> this kernel):
 // FP32 B = 16 n = 1024 4.43 -> 2.4 ms, n = 8192 38.1 -> 21.6 ms; FP32 B = 32 n = 3000 47.8 ->
-// 12.6 ms; FP64 B = 16 n = 2048 35.4 -> 17.2 ms, B = 32 n = 256 9.1 -> 3.7 ms.  A block step is
+// 12.8 ms; FP64 B = 16 n = 2048 35.4 -> 16.5 ms, B = 32 n = 256 9.1 -> 3.6 ms.  A block step is
 // 1,370 cycles with one FP32 team and 1,900 with eight (B = 16), 5,080 in FP64; the hand-off
 // between groups costs another 10,000 cycles a group.  Hence the group sizes below: FP32 8 to 12
 // sweeps measured within 1 %, 4 gave 26 % and 16 8 % more; FP64 B = 16 two sweeps 8.4 against 9.6 ms

@@ -40,9 +40,12 @@ NLA_DEV double widen(unsigned f, int e) {
 // (a vector below 2^-480 or above 2^496 in length) 1 / q itself overflows or is subnormal, so the
 // callers keep the factors apart or scale the vector first.
 NLA_DEV bool ordinary(double q) { return (unsigned)__double2hiint(q) - 0x03f00000u < 0x7e000000u - 0x03f00000u; }
+// FP32 keeps the factors apart everywhere.  What is left: (u^T row) m1 m2 overflows where a vector
+// below 2^-63 meets coefficients above 2^62; below 2^-66 its norm has lost its digits anyway, and a
+// test on the chain cost 3 % of the chase.
 NLA_DEV bool ordinary(float) { return true; }
 
-// Outside ordinary() nothing below is valid.  The FP64 scalars start from FP32 estimates (2^-22) of
+// The FP64 scalars, for an ordinary q only, start from FP32 estimates (2^-22) of
 // q = alpha^2 + qt, r = |x| = sqrt(q), and take one third-order step each (the Householder
 // iterations of order 3 for the inverse square root and the reciprocal: the error becomes the cube,
 // below 2^-60).  FP64 instructions are what counts: about a dozen one after another, where the

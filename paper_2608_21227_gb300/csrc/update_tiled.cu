@@ -70,6 +70,8 @@ NLA_DEV int swz(int r, int c, int w) { return r * w + ((((c >> 2) ^ (r & 7))) <<
 
 constexpr int kMaxSplit = 8;
 
+// Step 3, and what a configuration is checked by: one tile of th lines, V's rows and W.  (Step 1
+// takes two tiles of th / 2 lines in the same room.)
 size_t tiled_smem(int side, int elem, int nb, int th, int w) {
     (void)side;
     return (size_t)elem * ((size_t)th * w + (size_t)th * (nb + 4) + (size_t)nb * w);
@@ -108,8 +110,8 @@ __global__ void left_w_kernel(const T *__restrict__ X, long ldx, int M, int N, c
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int sh_last;
     const int ldv_s = nb + 4;
-    T *Xs = reinterpret_cast<T *>(smem_raw);  // th x w, swizzled
-    T *Vs = Xs + (size_t)2 * th * w;             // th x (nb+4) row-major
+    T *Xs = reinterpret_cast<T *>(smem_raw);  // 2 x th x w, swizzled
+    T *Vs = Xs + (size_t)2 * th * w;             // 2 x th x (nb+4) row-major
     T *Ws = reinterpret_cast<T *>(smem_raw) + tiled_w_offset(nb, th, w);  // nb x w row-major
     const int tid = threadIdx.x, nt = blockDim.x;
     const int ncg = w >> 2, cg = tid % ncg, rg = tid / ncg;
