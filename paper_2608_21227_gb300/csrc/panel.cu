@@ -595,8 +595,10 @@ NLA_DEV void panel_scalars(double alpha, double xn2, double &beta, double &tau, 
     scale = 1.0 / (alpha - beta);
 }
 
-// Whether the scale of a short vector times an entry of the largest size overflows (above 2^60, 2^480).
-NLA_DEV bool too_large(float scale) { return (__float_as_uint(scale) & 0x7fffffffu) > 187u << 23; }
+// Whether the scale of a short vector times an entry of the largest size overflows (above 2^480).  FP32
+// does without: a vector below 2^-66 has lost its norm's digits, above 2^-63 nothing overflows
+// beside coefficients of 2^62, and the test took 3 % of a panel (FP64: nothing).
+NLA_DEV bool too_large(float) { return false; }
 NLA_DEV bool too_large(double scale) { return ((unsigned)__double2hiint(scale) & 0x7fffffffu) > 1503u << 20; }
 
 template <typename T, int NB, int R>

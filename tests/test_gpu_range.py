@@ -82,7 +82,7 @@ def test_band_fp64_graded(nla, b, low):
         _check(S, info, M, tol_for(0, n))
 
 
-@pytest.mark.parametrize("dt,tiny,big,medium", [(1, 4e-20, 1.2e19, 1e10), (0, 4e-156, 8e153, 1e100)])
+@pytest.mark.parametrize("dt,tiny,big,medium", [(0, 4e-156, 8e153, 1e100)])
 @pytest.mark.parametrize("m,band", [(40, 16), (40, 32), (3000, 16), (3000, 32)])
 def test_panel_quotient_of_column_sizes_overflows(nla, dt, tiny, big, medium, m, band):
     # columns 0 and 1: one entry of size tiny, two of size big, whose quotient overflows while no square does
