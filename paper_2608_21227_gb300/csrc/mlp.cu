@@ -41,7 +41,7 @@ constexpr size_t kParams = (size_t)kH * kIn + kH + 2 * ((size_t)kH * kH + kH) + 
 // Why fused: as separate matrix products the step was 17 launches whose weight gradients had
 // K = rows on 16 blocks (4096 rows: 101 us per product, 90 us per bias sum).  What bounds it
 // now is shared-memory reads (a thread's 4 x 4 outputs read 8 values per 16 FMAs).
-// One training step of 4096 rows: 1501 -> 59 us.
+// One training step of 4096 rows: 1501 -> 57 us.
 //
 // Shared memory (floats): Ws kH x kLd (one layer's weights, transposed for the forward pass),
 // X R x 16, H1..H3 and two gradient buffers R x kLd.
