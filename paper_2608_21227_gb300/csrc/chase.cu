@@ -108,7 +108,6 @@ struct Half {
             else
                 asm volatile("bar.sync %0, %1;" ::"r"(barid), "n"(32 * NW) : "memory");
         };
-        sync();  // what the team left in the buffer for the next half is written again below
         const int tr = k == 0 ? s : c0 - B;
         const int nvec = RIGHT ? c0 + L - tr : min(c0 + 2 * B, n) - c0;
         const auto at = [&](int g, int c) -> T & {  // entry c of vector g
@@ -119,20 +118,23 @@ struct Half {
         const T *const buf = RIGHT ? team : team + B;
         const bool first = RIGHT && k == 0;  // the sweep starts: x is still in the window
         const auto x = [&](int i) { return first ? at(0, i) : buf[i]; };
+        // a zero vector, not rare in a matrix with zero blocks: H = I, and nothing has changed (in
+        // integers: an FP64 maximum holds the pipe for 64 cycles an entry)
+        unsigned bits = 0u;
+        for (int i = 0; i < L; ++i) bits |= magnitude_bits(x(i));
+        if (bits == 0u) return;
         T mx = T(0);
         for (int i = 0; i < L; ++i) mx = fmax(mx, fabs(x(i)));
-        T beta = T(0), u0 = T(0), m1 = T(0), m2 = T(0), f1 = T(1), f2 = T(1);
-        if (mx > T(0)) {
-            int ex;
-            frexp(mx, &ex);
-            f1 = ldexp(T(1), -(ex / 2)), f2 = ldexp(T(1), -(ex - ex / 2));  // normal numbers both
-            T qt = T(0);
-            for (int i = 1; i < L; ++i) qt = fma(x(i) * f1 * f2, x(i) * f1 * f2, qt);
-            house(x(0) * f1 * f2, qt, beta, u0, m1, m2);
-            beta = beta / f1 / f2;
-        }
+        sync();  // what the team left in the buffer for the next half is written again below
+        int ex;
+        frexp(mx, &ex);
+        const T f1 = ldexp(T(1), -(ex / 2)), f2 = ldexp(T(1), -(ex - ex / 2));  // normal numbers both
+        T beta, u0, m1, m2, qt = T(0);
+        for (int i = 1; i < L; ++i) qt = fma(x(i) * f1 * f2, x(i) * f1 * f2, qt);
+        house(x(0) * f1 * f2, qt, beta, u0, m1, m2);
+        beta = beta / f1 / f2;
         for (int g = ttid; g < nvec; g += 32 * NW) {
-            if (g > 0 && mx > T(0)) {
+            if (g > 0) {
                 T d = u0 * at(g, 0);
                 for (int i = 1; i < L; ++i) d = fma(x(i) * f1 * f2, at(g, i), d);
                 const T w = d * m1 * m2;
@@ -143,7 +145,7 @@ struct Half {
             if (o >= 0) (RIGHT ? team + B : team)[o] = at(g, 0);
         }
         sync();
-        if (ttid == 0 && mx > T(0))  // (x may have been vector 0 itself until here)
+        if (ttid == 0)  // (x may have been vector 0 itself until here)
             for (int i = 0; i < L; ++i) at(0, i) = i == 0 ? beta : T(0);
     }
 
